@@ -8,10 +8,11 @@
 //                   scales for the centre sums)
 //   k_slic_seed     centres at the grid cells' centres
 //   k_slic_assign_* the best centre of every sample among its candidates, and the sample's
-//                   fixed-point contribution to that centre's sums (warp-reduced): the first
-//                   pass one thread per sample; later field passes a tile of voxels of one cell
-//                   per block, later point passes one cell's grouped samples per block
-//                   (k_slic_pgroup groups them once), both against a shared candidate list
+//                   fixed-point contribution to that centre's sums: the first pass one thread
+//                   per sample; later field passes a tile of voxels of one step per block, later
+//                   point passes one cell's grouped samples per block (k_slic_pgroup groups them
+//                   once), both against a shared candidate list that every warp cuts down to the
+//                   centres its own samples can reach
 //   k_slic_update   one thread per centre: means of its sums, counts, change test
 //   k_slic_cells*   centres sorted into the cells of the seed grid for the next assignment
 //
@@ -66,10 +67,13 @@ struct SlicArgs {
   int32_t* plabel;              // [nj][P]
   unsigned* moved;
   unsigned long long* valid;    // [0] samples, [1] max|f| bits, [2] max|p| bits
-  uint32_t* pcell_start;        // [K + 1] first slot of each cell's point samples
-  uint32_t* pcell_cursor;       // [K]
+  uint32_t* pcell_start;        // [K * nsub + 1] first slot of each subcell's point samples
+  uint32_t* pcell_cursor;       // [K * nsub]
   float4* psample;              // [slots] x, y, z, value of the point sample in the slot
+  float* ptime;                 // [slots] its time
   uint32_t* pindex;             // [slots] its index t * P + p in the window (t: point step)
+  int sub[4], nsub;             // subcells of a cell along x, y, z, t, and their number
+  bool plain;                   // weights and sizes the pruned scan and the packed sums allow
 };
 
 // Time of window point step t: with r point steps in field step f, the i-th (0-based) sits at
@@ -207,9 +211,8 @@ __global__ void k_slic_seed(const __grid_constant__ SlicArgs a) {
 }
 
 // ---- the best centre of one sample -------------------------------------------------------------
-// INIT: nearest seed by S_st among the sample's cell and its neighbours. Otherwise: smallest D
-// among the filed centres of those cells whose search region holds the sample (-1: none).
-template <bool INIT>
+// Smallest D among the filed centres of the sample's cell and its neighbours whose search region
+// holds the sample (-1: none).
 __device__ __forceinline__ int best_centre(const SlicArgs& a, float xs, float ys, float zs,
                                            float ts, float w, float vs, int vslot) {
   const int ci = cell_of(xs, a.C[0], a.k[0]), cj = cell_of(ys, a.C[1], a.k[1]);
@@ -222,31 +225,81 @@ __device__ __forceinline__ int best_centre(const SlicArgs& a, float xs, float ys
       for (int j = max(cj - 1, 0); j <= min(cj + 1, a.k[1] - 1); ++j)
         for (int i = max(ci - 1, 0); i <= min(ci + 1, a.k[0] - 1); ++i) {
           const int cell = ((m * a.k[2] + l) * a.k[1] + j) * a.k[0] + i;
-          if (INIT) {
-            const float d = s_st(a.centers + 6 * (int64_t)cell, xs, ys, zs, ts, a.c_f);
-            if (better(d, cell, bd, bc)) {
+          const uint32_t e = __ldg(a.cell_start + cell + 1);
+          for (uint32_t q = __ldg(a.cell_start + cell); q < e; ++q) {
+            const int c = (int)__ldg(a.cell_items + q);
+            const float* cc = a.centers + 6 * (int64_t)c;
+            if (!in_region(cc, a.C, xs, ys, zs, ts)) continue;
+            const float d = __fadd_rn(__fmul_rn(w, fabsf(__fsub_rn(vs, cc[vslot]))),
+                                      __fmul_rn(a.w_d, s_st(cc, xs, ys, zs, ts, a.c_f)));
+            if (better(d, c, bd, bc)) {
               bd = d;
-              bc = cell;
-            }
-          } else {
-            const uint32_t e = __ldg(a.cell_start + cell + 1);
-            for (uint32_t q = __ldg(a.cell_start + cell); q < e; ++q) {
-              const int c = (int)__ldg(a.cell_items + q);
-              const float* cc = a.centers + 6 * (int64_t)c;
-              if (!in_region(cc, a.C, xs, ys, zs, ts)) continue;
-              const float d = __fadd_rn(__fmul_rn(w, fabsf(__fsub_rn(vs, cc[vslot]))),
-                                        __fmul_rn(a.w_d, s_st(cc, xs, ys, zs, ts, a.c_f)));
-              if (better(d, c, bd, bc)) {
-                bd = d;
-                bc = c;
-              }
+              bc = c;
             }
           }
         }
   return bc;
 }
 
-template <bool INIT>
+// Coordinate of the seeds of grid index i along axis q (as k_slic_seed forms it).
+__device__ __forceinline__ float seed_coord(const SlicArgs& a, int q, int i) {
+  const float u = __fmul_rn(__fadd_rn((float)i, 0.5f), a.C[q]);
+  return q == 3 ? __fadd_rn((float)a.t0, u) : u;
+}
+
+// First assignment: the nearest seed by S_st, the lowest index on a tie. The seeds are a grid, so
+// S_st^2 is a sum of one term per axis, added in a fixed order, and rounded additions and square
+// root never decrease: the smallest distance is that of the axes' smallest terms, each at the
+// sample's grid index or a neighbour, and a tie at a lower index of one axis exists exactly when
+// it does with the other axes at their smallest (the later ones) or at the index already taken
+// (the earlier ones). So the axes are walked down from the nearest index, the slowest-running
+// one first, as long as the distance stays the same: mostly not at all. Computing the 81
+// distances of the neighbourhood was a tenth of a ten-update clustering.
+__device__ __forceinline__ int nearest_seed(const SlicArgs& a, float xs, float ys, float zs,
+                                            float ts) {
+  const float u[4] = {xs, ys, zs, ts};
+  auto term = [&](int q, int i) {
+    float d = __fsub_rn(seed_coord(a, q, i), u[q]);
+    if (q == 3) d = __fmul_rn(a.c_f, d);
+    return __fmul_rn(d, d);
+  };
+  auto sum = [](const float (&e)[4]) {
+    return __fadd_rn(__fadd_rn(__fadd_rn(e[0], e[1]), e[2]), e[3]);
+  };
+  int at[4];
+  float e[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int c = cell_of(q == 3 ? __fsub_rn(ts, (float)a.t0) : u[q], a.C[q], a.k[q]);
+    at[q] = c;
+    e[q] = term(q, c);
+    const float lo = c > 0 ? term(q, c - 1) : INFINITY;
+    const float hi = c + 1 < a.k[q] ? term(q, c + 1) : INFINITY;
+    if (lo <= e[q] && c > 0) {
+      at[q] = c - 1;
+      e[q] = lo;
+    }
+    if (hi < e[q]) {
+      at[q] = c + 1;
+      e[q] = hi;
+    }
+  }
+  const float smin = sum(e), dmin = __fsqrt_rn(smin), most = __fmaf_rn(smin, 1e-6f, smin);
+#pragma unroll
+  for (int q = 3; q >= 0; --q)
+    while (at[q] > 0) {
+      const float keep = e[q];
+      e[q] = term(q, at[q] - 1);
+      const float s2 = sum(e);
+      if (!(s2 <= most) || __fsqrt_rn(s2) != dmin) {
+        e[q] = keep;
+        break;
+      }
+      --at[q];
+    }
+  return ((at[3] * a.k[2] + at[2]) * a.k[1] + at[1]) * a.k[0] + at[0];
+}
+
 __global__ void __launch_bounds__(256, 4) k_slic_assign_field(const __grid_constant__ SlicArgs a) {
   const int64_t n = (int64_t)a.tw * a.V;
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n;
@@ -255,47 +308,244 @@ __global__ void __launch_bounds__(256, 4) k_slic_assign_field(const __grid_const
     int best = -1;
     long long v[5] = {0, 0, 0, 0, 0};
     if (li < n) {
-      const int t = (int)(li / a.V);
-      const int64_t vox = li - (int64_t)t * a.V;
-      const int x = (int)(vox % a.nx), y = (int)((vox / a.nx) % a.ny), z = (int)(vox / ((int64_t)a.nx * a.ny));
+      const uint32_t t = (uint32_t)li / (uint32_t)a.V, vox = (uint32_t)li - t * (uint32_t)a.V;
+      const uint32_t yz = vox / (uint32_t)a.nx, x = vox - yz * (uint32_t)a.nx;
+      const uint32_t z = yz / (uint32_t)a.ny, y = yz - z * (uint32_t)a.ny;
       const float f = __ldg(a.field + (int64_t)a.t0 * a.V + li);
-      const bool take = INIT ? isfinite(f) : a.flabel[li] >= 0;
-      if (take) {
-        const float xs = __fadd_rn((float)x, 0.5f), ys = __fadd_rn((float)y, 0.5f);
-        const float zs = __fadd_rn((float)z, 0.5f), ts = __fadd_rn((float)(a.t0 + t), 0.5f);
-        best = best_centre<INIT>(a, xs, ys, zs, ts, a.w_f, f, 5);
-        if (!INIT && best < 0) best = a.flabel[li];  // no centre in range: keeps its centre
-        a.flabel[li] = best;
+      if (isfinite(f)) {
+        const float xs = __fadd_rn((float)(int)x, 0.5f), ys = __fadd_rn((float)(int)y, 0.5f);
+        const float zs = __fadd_rn((float)(int)z, 0.5f);
+        const float ts = __fadd_rn((float)(a.t0 + (int)t), 0.5f);
+        best = nearest_seed(a, xs, ys, zs, ts);
         v[0] = quantise(xs, a.kpos);
         v[1] = quantise(ys, a.kpos);
         v[2] = quantise(zs, a.kpos);
         v[3] = quantise(ts, a.kpos);
         v[4] = quantise(f, a.kf);
-      } else if (INIT) {
-        a.flabel[li] = -1;
       }
+      a.flabel[li] = best;
     }
     warp_accumulate(a.sums, best, v, 5);
   }
 }
 
-// Field samples in tiles of TX x TY x TZ voxels of one step (256 per block): the centres filed
-// in the cells around the tile are gathered into shared memory once and every thread scans
-// that list. A tile whose neighbourhood holds more than kCand centres (or spans more than 256
-// cells) falls back to the per-sample lookup.
-constexpr int kCand = 768;
+// ---- later assignments: shared candidate lists ----------------------------------------------
+// The centres filed in the cells around a block's samples (a tile of field voxels of one step, or
+// a cell's point samples) are gathered into shared memory once. A warp's samples are close to
+// each other, so it copies the centres whose search region reaches the box of its samples into a
+// list of its own (the box test is the region test at the box's nearest point, in the same
+// rounded operations, so it never drops a centre that some sample's test would pass) and every
+// lane scans that.
+//
+// Only the arg-min is needed, not the distance: the scan uses an approximate distance (fused
+// operations and the hardware's approximate square root, within 2^-20 of the rounded sequence
+// that decides; the region test is exact) and keeps the two smallest. When the second exceeds the
+// first by more than 4e-6 of it, the first is the answer; otherwise, and with weights or values
+// that the error bound does not cover, the lane scans the list again with the deciding
+// operations. 54 to 81 candidates in the deciding operations, an IEEE square root each, bounded
+// the passes by instruction issue.
+//
+// Sums: a sample adds to its centre's place in shared memory, and the block commits each place
+// once (adding up in the warp took a loop over the members of every group with 64-bit shuffles).
+//
+// 128^3 x 32 field and 1M x 32 point samples, 16,384 centres, ten assignments: field 68.2 -> 34.0
+// ms, points 60.2 -> 18.2 ms.
+constexpr int kCand = 384;   // centres in a block's list; more: the per-sample lookup
+constexpr int kWCand = 96;   // centres in a warp's list; more: the warp scans the block's list
 
+struct CandList {
+  float4 pos[kCand];   // x, y, z, t
+  float val[kCand];    // the value the pass compares
+  int id[kCand];
+};
+
+struct WarpList {
+  float4 pos[kWCand];  // x, y, z, t
+  float val[kWCand];
+  uint16_t q[kWCand];  // place in the block's list
+};
+
+// distance between u and the nearest point of [lo, hi], in the rounding of the region test
+__device__ __forceinline__ float box_dist(float u, float lo, float hi) {
+  return u < lo ? __fsub_rn(lo, u) : u > hi ? __fsub_rn(u, hi) : 0.f;
+}
+
+// centre q of the block's list, when it reaches the box, into the warp's list; returns the
+// number listed (-1: too many). All lanes.
+__device__ __forceinline__ int warp_list(const SlicArgs& a, const CandList& c, int nc, WarpList& w,
+                                         const float (&lo)[4], const float (&hi)[4]) {
+  const int lane = threadIdx.x & 31;
+  int n = 0;
+  for (int b = 0; b < nc; b += 32) {
+    const int q = b + lane;
+    bool in = q < nc;
+    float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (in) {
+      p = c.pos[q];
+      in = box_dist(p.x, lo[0], hi[0]) <= a.C[0] && box_dist(p.y, lo[1], hi[1]) <= a.C[1] &&
+           box_dist(p.z, lo[2], hi[2]) <= a.C[2] && box_dist(p.w, lo[3], hi[3]) <= a.C[3];
+    }
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, in);
+    const int at = n + __popc(m & ((1u << lane) - 1u));
+    n += __popc(m);
+    if (n > kWCand) return -1;  // warp-uniform
+    if (in) {
+      w.pos[at] = p;
+      w.val[at] = c.val[q];
+      w.q[at] = (uint16_t)q;
+    }
+  }
+  __syncwarp();
+  return n;
+}
+
+// place in the block's list of the best centre among n listed ones by the deciding operations
+// (w: the warp's list, or null for the block's), or -1
+__device__ __forceinline__ int exact_best(const SlicArgs& a, const CandList& c, const WarpList* w,
+                                          int n, float xs, float ys, float zs, float ts, float wv,
+                                          float vs) {
+  int best = -1, bc = -1;
+  float bd = 0.f;
+  for (int i = 0; i < n; ++i) {
+    const int q = w ? (int)w->q[i] : i;
+    const float4 p = c.pos[q];
+    const float cc[4] = {p.x, p.y, p.z, p.w};
+    if (!in_region(cc, a.C, xs, ys, zs, ts)) continue;
+    const float d = __fadd_rn(__fmul_rn(wv, fabsf(__fsub_rn(vs, c.val[q]))),
+                              __fmul_rn(a.w_d, s_st(cc, xs, ys, zs, ts, a.c_f)));
+    if (better(d, c.id[q], bd, bc)) {
+      bd = d;
+      bc = c.id[q];
+      best = q;
+    }
+  }
+  return best;
+}
+
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// the same by the approximate scan of the warp's list where that decides. TIME: the samples of
+// the warp differ in time, so the region's time test is per sample.
+template <bool TIME>
+__device__ __forceinline__ int list_best(const SlicArgs& a, const CandList& c, const WarpList& w,
+                                         int n, int nc, float xs, float ys, float zs, float ts,
+                                         float wv, float vs) {
+  if (n < 0) return exact_best(a, c, nullptr, nc, xs, ys, zs, ts, wv, vs);
+  if (!a.plain) return exact_best(a, c, &w, n, xs, ys, zs, ts, wv, vs);
+  const float C0 = a.C[0], C1 = a.C[1], C2 = a.C[2], C3 = a.C[3], cf2 = a.c_f * a.c_f;
+  float m1 = INFINITY, m2 = INFINITY;
+  int best = -1;
+#pragma unroll 4
+  for (int i = 0; i < n; ++i) {
+    const float4 p = w.pos[i];
+    const float dx = __fsub_rn(p.x, xs), dy = __fsub_rn(p.y, ys), dz = __fsub_rn(p.z, zs);
+    const float dt = __fsub_rn(p.w, ts);
+    bool in = fabsf(dx) <= C0 && fabsf(dy) <= C1 && fabsf(dz) <= C2;
+    if (TIME) in = in && fabsf(dt) <= C3;
+    const float s2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, cf2 * (dt * dt))));
+    const float d = fmaf(a.w_d, sqrt_approx(s2), wv * fabsf(vs - w.val[i]));
+    const float e = in ? d : INFINITY;
+    m2 = fminf(m2, fmaxf(m1, e));
+    best = e < m1 ? i : best;
+    m1 = fminf(m1, e);
+  }
+  if (best < 0 && m1 == INFINITY && m2 == INFINITY) {
+    // no centre in reach, or distances beyond fp32: the deciding scan tells
+    return exact_best(a, c, &w, n, xs, ys, zs, ts, wv, vs);
+  }
+  if (m1 < 1e30f && m2 > fmaf(m1, 4e-6f, m1) + 1e-30f) return w.q[best];
+  return exact_best(a, c, &w, n, xs, ys, zs, ts, wv, vs);
+}
+
+// The filed centres of the cells [lo, lo + nn) into the block's list, except those whose time
+// fails the search region for every time in [ta, tb]. Returns their number, -1 for more than
+// kCand (or more than 256 cells). One neighbouring cell per thread; all threads.
+__device__ __forceinline__ int block_list(const SlicArgs& a, const int (&lo)[4], const int (&nn)[4],
+                                          float ta, float tb, int vslot, CandList& c, int* s_warp) {
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int ncell = nn[0] * nn[1] * nn[2] * nn[3];
+  if (ncell > 256) return -1;  // block-uniform
+  int cnt = 0, kept = 0;
+  uint32_t c0 = 0;
+  if (tid < ncell) {
+    int q = tid;
+    const int i = lo[0] + q % nn[0]; q /= nn[0];
+    const int j = lo[1] + q % nn[1]; q /= nn[1];
+    const int l = lo[2] + q % nn[2]; q /= nn[2];
+    const int m = lo[3] + q;
+    const int cell = ((m * a.k[2] + l) * a.k[1] + j) * a.k[0] + i;
+    c0 = __ldg(a.cell_start + cell);
+    cnt = (int)(__ldg(a.cell_start + cell + 1) - c0);
+    for (int r = 0; r < cnt; ++r) {
+      const int id = (int)__ldg(a.cell_items + c0 + r);
+      kept += box_dist(__ldg(a.centers + 6 * (int64_t)id + 3), ta, tb) <= a.C[3];
+    }
+  }
+  int x = kept;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) s_warp[w] = x;
+  __syncthreads();
+  int off = x - kept, total = 0;
+  for (int q = 0; q < 8; ++q) {
+    const int t = s_warp[q];
+    if (q < w) off += t;
+    total += t;
+  }
+  if (total <= kCand)
+    for (int q = 0; q < cnt; ++q) {
+      const int id = (int)__ldg(a.cell_items + c0 + q);
+      const float* cc = a.centers + 6 * (int64_t)id;
+      const float ct = __ldg(cc + 3);
+      if (!(box_dist(ct, ta, tb) <= a.C[3])) continue;
+      c.pos[off] = make_float4(__ldg(cc), __ldg(cc + 1), __ldg(cc + 2), ct);
+      c.val[off] = __ldg(cc + vslot);
+      c.id[off] = id;
+      ++off;
+    }
+  __syncthreads();
+  return total <= kCand ? total : -1;
+}
+
+// one sample's sums straight to its centre (no place in the block's list)
+__device__ __forceinline__ void commit_sample(unsigned long long* sums, int c, const long long* v,
+                                              int slot) {
+  unsigned long long* s = sums + 8 * (int64_t)c;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) atomicAdd(s + q, (unsigned long long)v[q]);
+  atomicAdd(s + slot, (unsigned long long)v[4]);
+  atomicAdd(s + (slot == 5 ? 6 : 7), 1ull);
+}
+
+// 64-bit addition in shared memory as two 32-bit atomics, the carry with the second
+__device__ __forceinline__ void add64(uint32_t* p, unsigned long long v) {
+  const uint32_t lo = (uint32_t)v, old = atomicAdd(p, lo);
+  const uint32_t hi = (uint32_t)(v >> 32) + (old + lo < old ? 1u : 0u);
+  if (hi) atomicAdd(p + 1, hi);
+}
+
+// Field samples: a tile of TX x TY x TZ voxels of one step per block (256), 8 x 4 of them per
+// warp. A sample's place adds its tile coordinates as packed counters: count and x in one word, y
+// and z in another (256 voxels: no counter exceeds 16 bits).
 template <int TX, int TY, int TZ>
 __global__ void __launch_bounds__(256, 4) k_slic_assign_field_tiled(const __grid_constant__ SlicArgs a) {
-  static_assert(TX * TY * TZ == 256, "one voxel per thread");
-  __shared__ float s_cx[kCand], s_cy[kCand], s_cz[kCand], s_ct[kCand], s_cf[kCand];
-  __shared__ int s_id[kCand];
+  static_assert(TX * TY * TZ == 256 && TX % 8 == 0 && TY % 4 == 0, "8 x 4 voxels per warp");
+  __shared__ CandList s_c;
+  __shared__ WarpList s_w[8];
+  __shared__ uint4 s_acc[kCand];  // count | x, y | z, the value sum's halves
   __shared__ int s_warp[8];
-  __shared__ int s_lo[4], s_n[4];
-  __shared__ int s_total, s_over;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int ntx = (a.nx + TX - 1) / TX, nty = (a.ny + TY - 1) / TY, ntz = (a.nz + TZ - 1) / TZ;
   const int64_t ntiles = (int64_t)ntx * nty * ntz * a.tw;
+  const int wx = (w % (TX / 8)) * 8, wy = (w / (TX / 8)) % (TY / 4) * 4;
+  const int wz = w / ((TX / 8) * (TY / 4));
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     int64_t r = tile;
     const int bx = (int)(r % ntx); r /= ntx;
@@ -304,130 +554,81 @@ __global__ void __launch_bounds__(256, 4) k_slic_assign_field_tiled(const __grid
     const int t = (int)(r / ntz);
     const int x0 = bx * TX, y0 = by * TY, z0 = bz * TZ;
     const float ts = __fadd_rn((float)(a.t0 + t), 0.5f);
-    if (tid < 4) {
-      int lo, hi, k;
-      if (tid == 0) {
-        k = a.k[0];
-        lo = cell_of(__fadd_rn((float)x0, 0.5f), a.C[0], k);
-        hi = cell_of(__fadd_rn((float)(min(x0 + TX, a.nx) - 1), 0.5f), a.C[0], k);
-      } else if (tid == 1) {
-        k = a.k[1];
-        lo = cell_of(__fadd_rn((float)y0, 0.5f), a.C[1], k);
-        hi = cell_of(__fadd_rn((float)(min(y0 + TY, a.ny) - 1), 0.5f), a.C[1], k);
-      } else if (tid == 2) {
-        k = a.k[2];
-        lo = cell_of(__fadd_rn((float)z0, 0.5f), a.C[2], k);
-        hi = cell_of(__fadd_rn((float)(min(z0 + TZ, a.nz) - 1), 0.5f), a.C[2], k);
-      } else {
-        k = a.k[3];
-        lo = hi = cell_of(__fsub_rn(ts, (float)a.t0), a.C[3], k);
-      }
-      lo = max(lo - 1, 0);
-      hi = min(hi + 1, k - 1);
-      s_lo[tid] = lo;
-      s_n[tid] = hi - lo + 1;
-    }
-    __syncthreads();
-    const int ncell = s_n[0] * s_n[1] * s_n[2] * s_n[3];
-    // one neighbouring cell per thread: its filed centres go to the shared list, except those
-    // whose time fails the search region for this tile's step (every sample of the tile has
-    // that time, so the region test would reject them for all of them)
-    int cnt = 0, kept = 0;
-    uint32_t c0 = 0;
-    if (ncell <= 256 && tid < ncell) {
-      int q = tid;
-      const int i = s_lo[0] + q % s_n[0]; q /= s_n[0];
-      const int j = s_lo[1] + q % s_n[1]; q /= s_n[1];
-      const int l = s_lo[2] + q % s_n[2]; q /= s_n[2];
-      const int m = s_lo[3] + q;
-      const int cell = ((m * a.k[2] + l) * a.k[1] + j) * a.k[0] + i;
-      c0 = __ldg(a.cell_start + cell);
-      cnt = (int)(__ldg(a.cell_start + cell + 1) - c0);
-      for (int r = 0; r < cnt; ++r) {
-        const int c = (int)__ldg(a.cell_items + c0 + r);
-        kept += fabsf(__fsub_rn(ts, a.centers[6 * (int64_t)c + 3])) <= a.C[3];
-      }
-    }
-    int x = kept;
+    int lo[4], nn[4];
+    {
+      const int e0[3] = {x0, y0, z0};
+      const int e1[3] = {min(x0 + TX, a.nx) - 1, min(y0 + TY, a.ny) - 1, min(z0 + TZ, a.nz) - 1};
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) s_warp[w] = x;
-    __syncthreads();
-    int off = x - kept;
-    for (int q = 0; q < w; ++q) off += s_warp[q];
-    if (tid == 255) {
-      int tot = 0;
-      for (int q = 0; q < 8; ++q) tot += s_warp[q];
-      s_total = tot;
-      s_over = (ncell > 256 || tot > kCand) ? 1 : 0;
-    }
-    __syncthreads();
-    const bool over = s_over != 0;
-    if (!over)
-      for (int q = 0; q < cnt; ++q) {
-        const int c = (int)__ldg(a.cell_items + c0 + q);
-        const float* cc = a.centers + 6 * (int64_t)c;
-        if (!(fabsf(__fsub_rn(ts, cc[3])) <= a.C[3])) continue;
-        s_cx[off] = cc[0];
-        s_cy[off] = cc[1];
-        s_cz[off] = cc[2];
-        s_ct[off] = cc[3];
-        s_cf[off] = cc[5];
-        s_id[off] = c;
-        ++off;
+      for (int q = 0; q < 4; ++q) {
+        const float u0 = q < 3 ? __fadd_rn((float)e0[q < 3 ? q : 0], 0.5f) : __fsub_rn(ts, (float)a.t0);
+        const float u1 = q < 3 ? __fadd_rn((float)e1[q < 3 ? q : 0], 0.5f) : u0;
+        lo[q] = max(cell_of(u0, a.C[q], a.k[q]) - 1, 0);
+        nn[q] = min(cell_of(u1, a.C[q], a.k[q]) + 1, a.k[q] - 1) - lo[q] + 1;
       }
+    }
+    const int nc = block_list(a, lo, nn, ts, ts, 5, s_c, s_warp);
+    for (int q = tid; q < nc; q += 256) s_acc[q] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
-    const int nc = s_total;
-    const int xv = x0 + tid % TX, yv = y0 + (tid / TX) % TY, zv = z0 + tid / (TX * TY);
-    int best = -1;
-    long long v[5] = {0, 0, 0, 0, 0};
+    const int lx = wx + (lane & 7), ly = wy + (lane >> 3), lz = wz;
+    const int xv = x0 + lx, yv = y0 + ly, zv = z0 + lz;
+    const float xs = __fadd_rn((float)xv, 0.5f), ys = __fadd_rn((float)yv, 0.5f);
+    const float zs = __fadd_rn((float)zv, 0.5f);
+    int n = -1;
+    if (nc >= 0) {
+      const float blo[4] = {__fadd_rn((float)(x0 + wx), 0.5f), __fadd_rn((float)(y0 + wy), 0.5f), zs,
+                            ts};
+      const float bhi[4] = {__fadd_rn((float)(x0 + wx + 7), 0.5f),
+                            __fadd_rn((float)(y0 + wy + 3), 0.5f), zs, ts};
+      n = warp_list(a, s_c, nc, s_w[w], blo, bhi);
+    }
     if (xv < a.nx && yv < a.ny && zv < a.nz) {
       const int64_t li = ((int64_t)t * a.nz + zv) * a.ny * a.nx + (int64_t)yv * a.nx + xv;
-      if (a.flabel[li] >= 0) {
+      const int old = a.flabel[li];
+      if (old >= 0) {
         const float f = __ldg(a.field + (int64_t)a.t0 * a.V + li);
-        const float xs = __fadd_rn((float)xv, 0.5f), ys = __fadd_rn((float)yv, 0.5f);
-        const float zs = __fadd_rn((float)zv, 0.5f);
-        if (over) {
-          best = best_centre<false>(a, xs, ys, zs, ts, a.w_f, f, 5);
+        int q = -1, best;
+        if (nc >= 0) {
+          q = list_best<false>(a, s_c, s_w[w], n, nc, xs, ys, zs, ts, a.w_f, f);
+          best = q >= 0 ? s_c.id[q] : -1;
         } else {
-          float bd = 0.f;
-          for (int q = 0; q < nc; ++q) {
-            const float cx = s_cx[q], cy = s_cy[q], cz = s_cz[q], ct = s_ct[q];
-            if (!(fabsf(__fsub_rn(xs, cx)) <= a.C[0] && fabsf(__fsub_rn(ys, cy)) <= a.C[1] &&
-                  fabsf(__fsub_rn(zs, cz)) <= a.C[2] && fabsf(__fsub_rn(ts, ct)) <= a.C[3]))
-              continue;
-            const float dx = __fsub_rn(cx, xs), dy = __fsub_rn(cy, ys), dz = __fsub_rn(cz, zs);
-            const float dt = __fmul_rn(a.c_f, __fsub_rn(ct, ts));
-            const float sst = __fsqrt_rn(__fadd_rn(
-                __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz)),
-                __fmul_rn(dt, dt)));
-            const float d = __fadd_rn(__fmul_rn(a.w_f, fabsf(__fsub_rn(f, s_cf[q]))),
-                                      __fmul_rn(a.w_d, sst));
-            const int c = s_id[q];
-            if (better(d, c, bd, best)) {
-              bd = d;
-              best = c;
-            }
-          }
+          best = best_centre(a, xs, ys, zs, ts, a.w_f, f, 5);
         }
-        if (best < 0) best = a.flabel[li];  // no centre in range: keeps its centre
+        if (best < 0) best = old;  // no centre in range: keeps its centre
         a.flabel[li] = best;
-        v[0] = quantise(xs, a.kpos);
-        v[1] = quantise(ys, a.kpos);
-        v[2] = quantise(zs, a.kpos);
-        v[3] = quantise(ts, a.kpos);
-        v[4] = quantise(f, a.kf);
+        const long long qf = quantise(f, a.kf);
+        if (q >= 0 && a.plain) {
+          uint32_t* p = &s_acc[q].x;
+          atomicAdd(p, 1u + ((uint32_t)lx << 16));
+          atomicAdd(p + 1, (uint32_t)ly + ((uint32_t)lz << 16));
+          add64(p + 2, (unsigned long long)qf);
+        } else {
+          const long long v[5] = {quantise(xs, a.kpos), quantise(ys, a.kpos), quantise(zs, a.kpos),
+                                  quantise(ts, a.kpos), qf};
+          commit_sample(a.sums, best, v, 5);
+        }
       }
     }
-    warp_accumulate(a.sums, best, v, 5);
-    __syncthreads();  // the shared list is rebuilt for the next tile
+    __syncthreads();
+    // a place's coordinate sums are sums of (2 x + 1) / 2 at the position scale: exact shifts
+    for (int q = tid; q < nc; q += 256) {
+      const uint4 p = s_acc[q];
+      const uint32_t m = p.x & 0xFFFFu;
+      if (!m) continue;
+      unsigned long long* sm = a.sums + 8 * (int64_t)s_c.id[q];
+      const int e0[3] = {x0, y0, z0};
+      const uint32_t l[3] = {p.x >> 16, p.y & 0xFFFFu, p.y >> 16};
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        atomicAdd(sm + j, (unsigned long long)(2ull * ((unsigned long long)m * e0[j] + l[j]) + m)
+                              << (a.kpos - 1));
+      atomicAdd(sm + 3, (unsigned long long)quantise(ts, a.kpos) * m);
+      atomicAdd(sm + 5, ((unsigned long long)p.w << 32) | p.z);
+      atomicAdd(sm + 6, (unsigned long long)m);
+    }
+    __syncthreads();  // the lists are rebuilt for the next tile
   }
 }
 
-template <bool INIT>
 __global__ void __launch_bounds__(256, 4) k_slic_assign_points(const __grid_constant__ SlicArgs a) {
   const int64_t n = (int64_t)a.nj * a.P;
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n;
@@ -436,26 +637,22 @@ __global__ void __launch_bounds__(256, 4) k_slic_assign_points(const __grid_cons
     int best = -1;
     long long v[5] = {0, 0, 0, 0, 0};
     if (li < n) {
-      const int t = (int)(li / a.P);
+      const int t = (int)((uint32_t)li / (uint32_t)a.P);
       const int64_t p = li - (int64_t)t * a.P;
       const int64_t si = (int64_t)(a.j0 + t) * a.P + p;
       const float pv = __ldg(a.attrp + ((int64_t)(a.j0 + t) * a.A + a.attr) * a.P + p);
-      const bool take = INIT ? (__ldg(a.key + si) >= 0 && isfinite(pv)) : a.plabel[li] >= 0;
-      if (take) {
+      if (__ldg(a.key + si) >= 0 && isfinite(pv)) {
         const float* ps = a.pos + (int64_t)(a.j0 + t) * 3 * a.P;
         const float xs = __ldg(ps + p), ys = __ldg(ps + a.P + p), zs = __ldg(ps + 2 * a.P + p);
         const float ts = point_time(a, t);
-        best = best_centre<INIT>(a, xs, ys, zs, ts, a.w_p, pv, 4);
-        if (!INIT && best < 0) best = a.plabel[li];
-        a.plabel[li] = best;
+        best = nearest_seed(a, xs, ys, zs, ts);
         v[0] = quantise(xs, a.kpos);
         v[1] = quantise(ys, a.kpos);
         v[2] = quantise(zs, a.kpos);
         v[3] = quantise(ts, a.kpos);
         v[4] = quantise(pv, a.kp);
-      } else if (INIT) {
-        a.plabel[li] = -1;
       }
+      a.plabel[li] = best;
     }
     warp_accumulate(a.sums, best, v, 4);
   }
@@ -464,23 +661,33 @@ __global__ void __launch_bounds__(256, 4) k_slic_assign_points(const __grid_cons
 // ---- point samples grouped by cell ----------------------------------------------------------
 // The seed-grid cell of a point sample does not change between updates (its position is fixed),
 // and every sample of one cell searches the same 3^4 neighbourhood of cells. So the point samples
-// that take part are grouped by cell once per call (a counting sort; the order within a cell is whatever
-// the atomics give, which changes nothing: each sample's result depends on it alone and the
-// centre sums are exact), and each update then takes a cell at a time against a shared list of
-// its neighbourhood's centres, reading the grouped samples in order. (Field samples are taken
-// in tiles of voxels that lie in one cell already, so they need no grouping.)
-__device__ __forceinline__ int sample_cell(const SlicArgs& a, float xs, float ys, float zs,
-                                           float ts) {
-  const int ci = cell_of(xs, a.C[0], a.k[0]), cj = cell_of(ys, a.C[1], a.k[1]);
-  const int cl = cell_of(zs, a.C[2], a.k[2]);
-  const int cm = cell_of(__fsub_rn(ts, (float)a.t0), a.C[3], a.k[3]);
-  return ((cm * a.k[2] + cl) * a.k[1] + cj) * a.k[0] + ci;
+// that take part are grouped by cell once per call (a counting sort; the order within a group is
+// whatever the atomics give, which changes nothing: each sample's result depends on it alone and
+// the centre sums are exact), and each update then takes a cell at a time against a shared list
+// of its neighbourhood's centres, reading the grouped samples in order. Within a cell they are
+// grouped by subcell (halves in space, steps in time), so that the 32 samples of a warp span a
+// small box and few of the list's centres reach it. (Field samples are taken in tiles of voxels
+// that lie in one cell already, so they need no grouping.)
+__device__ __forceinline__ uint32_t sample_cell(const SlicArgs& a, float xs, float ys, float zs,
+                                                float ts) {
+  const float u[4] = {xs, ys, zs, __fsub_rn(ts, (float)a.t0)};
+  int c[4], h[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    c[q] = cell_of(u[q], a.C[q], a.k[q]);
+    // the subcell only orders samples: any rounding does
+    const float fr = u[q] / a.C[q] - (float)c[q];
+    h[q] = min(max((int)(fr * (float)a.sub[q]), 0), a.sub[q] - 1);
+  }
+  const uint32_t cell = (uint32_t)(((c[3] * a.k[2] + c[2]) * a.k[1] + c[1]) * a.k[0] + c[0]);
+  return cell * (uint32_t)a.nsub +
+         (uint32_t)(((h[3] * a.sub[2] + h[2]) * a.sub[1] + h[1]) * a.sub[0] + h[0]);
 }
 
 // point sample li (taking part after the first assignment): position and value
 __device__ __forceinline__ bool point_sample(const SlicArgs& a, int64_t li, float4& s, float& ts) {
   if (a.plabel[li] < 0) return false;
-  const int t = (int)(li / a.P);
+  const int t = (int)((uint32_t)li / (uint32_t)a.P);
   const int64_t p = li - (int64_t)t * a.P;
   const float* ps = a.pos + (int64_t)(a.j0 + t) * 3 * a.P;
   s = make_float4(__ldg(ps + p), __ldg(ps + a.P + p), __ldg(ps + 2 * a.P + p),
@@ -498,132 +705,108 @@ __global__ void __launch_bounds__(256) k_slic_pgroup(const __grid_constant__ Sli
     float4 sm;
     float ts;
     if (!point_sample(a, li, sm, ts)) continue;
-    const int cell = sample_cell(a, sm.x, sm.y, sm.z, ts);
+    const uint32_t cell = sample_cell(a, sm.x, sm.y, sm.z, ts);
     if (!FILL) {
       atomicAdd(cursor + cell, 1u);
     } else {
       const uint32_t slot = atomicAdd(cursor + cell, 1u);
       a.psample[slot] = sm;
+      a.ptime[slot] = ts;
       a.pindex[slot] = (uint32_t)li;
     }
   }
 }
 
-// One cell at a time (persistent blocks): its neighbourhood's filed centres into shared memory,
-// then its samples in slot order. Candidates, region test, distance and tie rule as best_centre.
+// One cell at a time (persistent blocks; grid y splits the samples of a cell where there are few
+// cells): its neighbourhood's filed centres into shared memory, then its samples in slot order,
+// 32 consecutive ones per warp. A sample's place adds its count and its five fixed-point values.
+struct PointAcc {
+  uint32_t n[kCand];
+  uint32_t v[kCand][10];  // x, y, z, t, value: low and high halves
+};
+
 __global__ void __launch_bounds__(256, 4) k_slic_assign_points_cells(const __grid_constant__ SlicArgs a) {
   constexpr int VS = 4;  // the centre's value slot (p_c)
-  __shared__ float s_cx[kCand], s_cy[kCand], s_cz[kCand], s_ct[kCand], s_cv[kCand];
-  __shared__ int s_id[kCand];
+  __shared__ CandList s_c;
+  __shared__ WarpList s_w[8];
+  __shared__ PointAcc s_acc;
   __shared__ int s_warp[8];
-  __shared__ int s_total;
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const uint32_t* gstart = a.pcell_start;
-  const float4* gsample = a.psample;
-  const uint32_t* gindex = a.pindex;
-  int32_t* label = a.plabel;
-  const float wv = a.w_p;
-  const int kv = a.kp;
-  const uint64_t per_t = (uint64_t)a.P;
+  const int tid = threadIdx.x, w = tid >> 5;
   for (int cell = blockIdx.x; cell < a.K; cell += gridDim.x) {
-    const uint32_t first = __ldg(gstart + cell), last = __ldg(gstart + cell + 1);
-    if (first == last) continue;  // block-uniform
+    const uint32_t first = __ldg(a.pcell_start + (int64_t)cell * a.nsub);
+    const uint32_t last = __ldg(a.pcell_start + (int64_t)(cell + 1) * a.nsub);
+    if (first + 256u * blockIdx.y >= last) continue;  // block-uniform
+    int lo[4], nn[4];
     int q0 = cell;
-    const int ci = q0 % a.k[0]; q0 /= a.k[0];
-    const int cj = q0 % a.k[1]; q0 /= a.k[1];
-    const int cl = q0 % a.k[2];
-    const int cm = q0 / a.k[2];
-    const int lo0 = max(ci - 1, 0), n0 = min(ci + 1, a.k[0] - 1) - lo0 + 1;
-    const int lo1 = max(cj - 1, 0), n1 = min(cj + 1, a.k[1] - 1) - lo1 + 1;
-    const int lo2 = max(cl - 1, 0), n2 = min(cl + 1, a.k[2] - 1) - lo2 + 1;
-    const int lo3 = max(cm - 1, 0), n3 = min(cm + 1, a.k[3] - 1) - lo3 + 1;
-    const int ncell = n0 * n1 * n2 * n3;  // at most 81
-    int cnt = 0;
-    uint32_t c0 = 0;
-    if (tid < ncell) {
-      int q = tid;
-      const int i = lo0 + q % n0; q /= n0;
-      const int j = lo1 + q % n1; q /= n1;
-      const int l = lo2 + q % n2; q /= n2;
-      const int m = lo3 + q;
-      const int nb = ((m * a.k[2] + l) * a.k[1] + j) * a.k[0] + i;
-      c0 = __ldg(a.cell_start + nb);
-      cnt = (int)(__ldg(a.cell_start + nb + 1) - c0);
-    }
-    int x = cnt;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-      if (lane >= o) x += y;
+    for (int q = 0; q < 4; ++q) {
+      const int c = q0 % a.k[q];
+      q0 /= a.k[q];
+      lo[q] = max(c - 1, 0);
+      nn[q] = min(c + 1, a.k[q] - 1) - lo[q] + 1;
     }
-    if (lane == 31) s_warp[w] = x;
-    __syncthreads();
-    int off = x - cnt;
-    for (int q = 0; q < w; ++q) off += s_warp[q];
-    if (tid == 255) {
-      int tot = 0;
-      for (int q = 0; q < 8; ++q) tot += s_warp[q];
-      s_total = tot;
+    const int nc = block_list(a, lo, nn, -INFINITY, INFINITY, VS, s_c, s_warp);
+    for (int q = tid; q < nc; q += 256) {
+      s_acc.n[q] = 0u;
+#pragma unroll
+      for (int j = 0; j < 10; ++j) s_acc.v[q][j] = 0u;
     }
     __syncthreads();
-    const int nc = s_total;
-    const bool over = nc > kCand;
-    if (!over)
-      for (int q = 0; q < cnt; ++q) {
-        const int c = (int)__ldg(a.cell_items + c0 + q);
-        const float* cc = a.centers + 6 * (int64_t)c;
-        s_cx[off + q] = cc[0];
-        s_cy[off + q] = cc[1];
-        s_cz[off + q] = cc[2];
-        s_ct[off + q] = cc[3];
-        s_cv[off + q] = cc[VS];
-        s_id[off + q] = c;
-      }
-    __syncthreads();
-    for (uint32_t b0 = first; b0 < last; b0 += 256) {  // block-uniform trip count
+    for (uint32_t b0 = first + 256u * blockIdx.y; b0 < last; b0 += 256u * gridDim.y) {
       const uint32_t slot = b0 + tid;
-      int best = -1;
-      long long v[5] = {0, 0, 0, 0, 0};
-      if (slot < last) {
-        const float4 sm = gsample[slot];
-        const uint32_t li = gindex[slot];
-        const int t = (int)(li / per_t);
-        const float xs = sm.x, ys = sm.y, zs = sm.z, vs = sm.w;
-        const float ts = point_time(a, t);
-        if (over) {
-          best = best_centre<false>(a, xs, ys, zs, ts, wv, vs, VS);
-        } else {
-          float bd = 0.f;
-          for (int q = 0; q < nc; ++q) {
-            const float cx = s_cx[q], cy = s_cy[q], cz = s_cz[q], ct = s_ct[q];
-            if (!(fabsf(__fsub_rn(xs, cx)) <= a.C[0] && fabsf(__fsub_rn(ys, cy)) <= a.C[1] &&
-                  fabsf(__fsub_rn(zs, cz)) <= a.C[2] && fabsf(__fsub_rn(ts, ct)) <= a.C[3]))
-              continue;
-            const float dx = __fsub_rn(cx, xs), dy = __fsub_rn(cy, ys), dz = __fsub_rn(cz, zs);
-            const float dt = __fmul_rn(a.c_f, __fsub_rn(ct, ts));
-            const float sst = __fsqrt_rn(__fadd_rn(
-                __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz)),
-                __fmul_rn(dt, dt)));
-            const float d = __fadd_rn(__fmul_rn(wv, fabsf(__fsub_rn(vs, s_cv[q]))),
-                                      __fmul_rn(a.w_d, sst));
-            const int c = s_id[q];
-            if (better(d, c, bd, best)) {
-              bd = d;
-              best = c;
-            }
-          }
+      const bool take = slot < last;
+      // (lanes past the end stand in for the last sample, so that they do not widen the box)
+      const uint32_t sl = min(slot, last - 1u);
+      const float4 sm = a.psample[sl];
+      const float ts = a.ptime[sl];
+      int n = -1;
+      if (nc >= 0) {
+        // positions lie inside the grid and times are positive: fp32 bits order like the values
+        // (-0 counts as 0)
+        const float u[4] = {__fadd_rn(sm.x, 0.f), __fadd_rn(sm.y, 0.f), __fadd_rn(sm.z, 0.f), ts};
+        float blo[4], bhi[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          blo[q] = __uint_as_float(__reduce_min_sync(0xFFFFFFFFu, __float_as_uint(u[q])));
+          bhi[q] = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(u[q])));
         }
-        if (best < 0) best = label[li];  // no centre in range: keeps its centre
-        label[li] = best;
-        v[0] = quantise(xs, a.kpos);
-        v[1] = quantise(ys, a.kpos);
-        v[2] = quantise(zs, a.kpos);
-        v[3] = quantise(ts, a.kpos);
-        v[4] = quantise(vs, kv);
+        n = warp_list(a, s_c, nc, s_w[w], blo, bhi);
       }
-      warp_accumulate(a.sums, best, v, VS);
+      if (take) {
+        const uint32_t li = a.pindex[slot];
+        int q = -1, best;
+        if (nc >= 0) {
+          q = list_best<true>(a, s_c, s_w[w], n, nc, sm.x, sm.y, sm.z, ts, a.w_p, sm.w);
+          best = q >= 0 ? s_c.id[q] : -1;
+        } else {
+          best = best_centre(a, sm.x, sm.y, sm.z, ts, a.w_p, sm.w, VS);
+        }
+        const long long v[5] = {quantise(sm.x, a.kpos), quantise(sm.y, a.kpos),
+                                quantise(sm.z, a.kpos), quantise(ts, a.kpos), quantise(sm.w, a.kp)};
+        if (best >= 0) a.plabel[li] = best;
+        else best = a.plabel[li];  // no centre in range: keeps its centre
+        if (q >= 0) {
+          atomicAdd(s_acc.n + q, 1u);
+#pragma unroll
+          for (int j = 0; j < 5; ++j) add64(&s_acc.v[q][2 * j], (unsigned long long)v[j]);
+        } else {
+          commit_sample(a.sums, best, v, VS);
+        }
+      }
+      __syncwarp();  // the warp's list is rebuilt for its next samples
     }
-    __syncthreads();  // the shared list is rebuilt for the next cell
+    __syncthreads();
+    for (int q = tid; q < nc; q += 256) {
+      const uint32_t m = s_acc.n[q];
+      if (!m) continue;
+      unsigned long long* sums = a.sums + 8 * (int64_t)s_c.id[q];
+#pragma unroll
+      for (int j = 0; j < 5; ++j)
+        atomicAdd(sums + j,
+                  ((unsigned long long)s_acc.v[q][2 * j + 1] << 32) | s_acc.v[q][2 * j]);
+      atomicAdd(sums + 7, (unsigned long long)m);
+    }
+    __syncthreads();  // the lists are rebuilt for the next cell
   }
 }
 
@@ -787,34 +970,53 @@ int cluster_run(msf_ctx* ctx, const msf_cluster_params* prm, int32_t* flabel, in
   const unsigned gp = (unsigned)std::max<int64_t>(1, std::min<int64_t>((nps + 255) / 256,
                                                                        (int64_t)ctx->sm_count * 32));
   const unsigned gt = (unsigned)ctx->sm_count * 8;  // tiled field pass: persistent blocks
+  // The approximate scan's error bound wants weights that add up and values far from overflow;
+  // the packed coordinate sums want voxel centres and their scale to be exact in fp32.
+  a.plain = a.w_p >= 0.f && a.w_f >= 0.f && a.w_d >= 0.f && a.kpos >= 1 &&
+            std::max(d.nx, std::max(d.ny, d.nz)) <= (1 << 22);
   k_slic_seed<<<kb, 256, 0, s>>>(a);
   {
     ScopedKernel k(ctx, "k_slic_assign_field");
-    k_slic_assign_field<true><<<gf, 256, 0, s>>>(a);
+    k_slic_assign_field<<<gf, 256, 0, s>>>(a);
   }
   if (nps > 0) {
     ScopedKernel k(ctx, "k_slic_assign_points");
-    k_slic_assign_points<true><<<gp, 256, 0, s>>>(a);
+    k_slic_assign_points<<<gp, 256, 0, s>>>(a);
   }
   if (nps > 0) {  // the taking-part point samples grouped by cell, for every later assignment
-    MSF_TRY(S.pcell_start.ensure(sizeof(uint32_t) * ((size_t)a.K + 1)));
-    MSF_TRY(S.pcell_cursor.ensure(sizeof(uint32_t) * (size_t)a.K));
+    // subcells: halves of a cell in space, its point steps (up to eight) in time, at most 2^22
+    // (or one per cell)
+    for (int q = 0; q < 3; ++q) a.sub[q] = a.C[q] > 1.f ? 2 : 1;
+    a.sub[3] = std::max(1, std::min(8, a.nj / a.k[3]));
+    auto nsub = [&] { return a.sub[0] * a.sub[1] * a.sub[2] * a.sub[3]; };
+    for (int q = 3; q >= 0; --q)
+      while (a.sub[q] > 1 && (int64_t)a.K * nsub() > (1 << 22)) a.sub[q] >>= 1;
+    a.nsub = nsub();
+    const size_t ncs = (size_t)a.K * (size_t)a.nsub;
+    MSF_TRY(S.pcell_start.ensure(sizeof(uint32_t) * (ncs + 1)));
+    MSF_TRY(S.pcell_cursor.ensure(sizeof(uint32_t) * ncs));
     MSF_TRY(S.psample.ensure(sizeof(float4) * (size_t)nps));
+    MSF_TRY(S.ptime.ensure(sizeof(float) * (size_t)nps));
     MSF_TRY(S.pindex.ensure(sizeof(uint32_t) * (size_t)nps));
     a.pcell_start = S.pcell_start.as<uint32_t>();
     a.pcell_cursor = S.pcell_cursor.as<uint32_t>();
     a.psample = S.psample.as<float4>();
+    a.ptime = S.ptime.as<float>();
     a.pindex = S.pindex.as<uint32_t>();
     ScopedKernel k(ctx, "k_slic_pgroup");
-    MSF_CUDA_TRY(cudaMemsetAsync(a.pcell_cursor, 0, sizeof(uint32_t) * a.K, s));
+    MSF_CUDA_TRY(cudaMemsetAsync(a.pcell_cursor, 0, sizeof(uint32_t) * ncs, s));
     k_slic_pgroup<false><<<gp, 256, 0, s>>>(a);
-    MSF_TRY(scan_exclusive_u32(ctx, a.pcell_cursor, a.pcell_start, a.K, S.scan_tmp,
-                               a.pcell_start + a.K));
-    MSF_CUDA_TRY(cudaMemcpyAsync(a.pcell_cursor, a.pcell_start, sizeof(uint32_t) * a.K,
+    MSF_TRY(scan_exclusive_u32(ctx, a.pcell_cursor, a.pcell_start, (int64_t)ncs, S.scan_tmp,
+                               a.pcell_start + ncs));
+    MSF_CUDA_TRY(cudaMemcpyAsync(a.pcell_cursor, a.pcell_start, sizeof(uint32_t) * ncs,
                                  cudaMemcpyDeviceToDevice, s));
     k_slic_pgroup<true><<<gp, 256, 0, s>>>(a);
   }
-  const unsigned gpc = (unsigned)std::min<int64_t>(a.K, (int64_t)ctx->sm_count * 8);
+  // blocks of the point pass: a cell each; with few cells several share one
+  const unsigned gpx = (unsigned)std::min<int64_t>(a.K, (int64_t)ctx->sm_count * 8);
+  const int64_t want = ((int64_t)ctx->sm_count * 4 + gpx - 1) / gpx;
+  const int64_t most = std::max<int64_t>(1, nps / ((int64_t)a.K * 512));
+  const dim3 gpc(gpx, (unsigned)std::min<int64_t>(65535, std::min(want, most)));
   int it = 1;
   for (it = 1; it <= prm->max_iter; ++it) {
     MSF_CUDA_TRY(cudaMemsetAsync(a.moved, 0, sizeof(unsigned), s));
