@@ -43,3 +43,46 @@ def test_summaries_match_oracle(gpu, orc, nx, ny, nz, T, P, K, lab):
         assert np.array_equal(g[k], o[k], equal_nan=True), k
     for k in ("std_field", "std_point"):  # fp64 sums in no fixed order
         np.testing.assert_allclose(g[k], o[k], rtol=1e-9, atol=1e-12, equal_nan=True)
+
+
+@pytest.mark.parametrize("n", [1, 3, 4, 5, 1027, 300001])
+@pytest.mark.parametrize("shift", [0, 1, 2])  # labels that start off a 16-byte boundary
+def test_relabel_matches_numpy(gpu, n, shift):
+    rng = np.random.default_rng(n + shift)
+    K = 77
+    lab = rng.integers(-2, K, size=n + shift).astype(np.int32)
+    m = rng.permutation(K).astype(np.int32)
+    ctx = gpu.Context(0)
+    try:
+        d = torch.as_tensor(lab).cuda()
+        ctx.relabel(d[shift:], torch.as_tensor(m).cuda())
+        want = lab.copy()
+        want[shift:] = np.where(lab[shift:] >= 0, m[np.maximum(lab[shift:], 0)], lab[shift:])
+        assert np.array_equal(d.cpu().numpy(), want)
+        for at in {0, n // 2, n - 1}:  # one label out of range anywhere: nothing changes
+            bad = torch.as_tensor(lab).cuda()
+            bad[shift + at] = K
+            before = bad.clone()
+            with pytest.raises(gpu.MsfError) as e:
+                ctx.relabel(bad[shift:], torch.as_tensor(m).cuda())
+            assert e.value.status == gpu.MSF_ERR_INVALID_ARG
+            assert torch.equal(bad, before)
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("K", [2, 256, 257, 700, 5000])
+def test_merge_chains_match_oracle(gpu, orc, K):
+    """Chains of matches that cross the pair tiles, groups interleaved by index."""
+    rng = np.random.default_rng(K)
+    c = np.zeros((K, 6), np.float32)
+    g = rng.integers(0, 5, K)
+    c[:, 4] = (10.0 ** g) * (1 + 0.004 * rng.permutation(K) / K * 40)
+    c[:, 5] = 1.0
+    ctx = gpu.Context(0)
+    try:
+        m, n = ctx.merge_clusters(torch.as_tensor(c).cuda(), 0.002)
+    finally:
+        ctx.close()
+    om, on = orc.merge_clusters(c, 0.002, 3)
+    assert n == on and np.array_equal(m, om)
