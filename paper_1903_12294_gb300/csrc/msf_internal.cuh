@@ -795,15 +795,15 @@ __device__ __forceinline__ unsigned long long limb_sum(unsigned m, unsigned long
   return (unsigned long long)s0 + ((unsigned long long)s1 << 21) + ((unsigned long long)s2 << 42);
 }
 
-// Point samples of one warp (lane: ok, feature fid, attributes at attr_p + j * P): the lanes
+// Point samples of one warp (lane: ok, feature fid, attribute values val(j)): the lanes
 // with the same feature reduce in the warp (exact 64-bit fixed-point sums; double-float sums of
 // squares), and one lane per feature hands the sums to sink(f, j, qs, h, l, w, dbl, one): the sum
 // of squares is h + l (a double-float pair, each exact in fp32), or w in fp64 when dbl is set
 // (non-finite or extreme values, rare); one is set when all the warp's samples belong to f (the
-// call then has a single leader). All 32 lanes must call this.
-template <class Sink>
-__device__ __forceinline__ void reduce_samples(const FeatAcc& acc, bool ok, int64_t fid,
-                                               const float* attr_p, int64_t P, Sink&& sink) {
+// call then has a single leader). AMAX: most attributes. All 32 lanes must call this.
+template <int AMAX, class Val, class Sink>
+__device__ __forceinline__ void reduce_samples(const FeatAcc& acc, bool ok, int64_t fid, Val&& val,
+                                               Sink&& sink) {
   const unsigned act = __ballot_sync(0xFFFFFFFFu, ok);
   if (!act) return;
   const int lane = threadIdx.x & 31;
@@ -812,8 +812,10 @@ __device__ __forceinline__ void reduce_samples(const FeatAcc& acc, bool ok, int6
   const int first = __ffs(act) - 1;
   const int64_t f0 = __shfl_sync(0xFFFFFFFFu, fid, first);
   if (__all_sync(0xFFFFFFFFu, !ok || fid == f0)) {
-    for (int j = 0; j < acc.A; ++j) {
-      const float v = ok ? __ldg(attr_p + (int64_t)j * P) : 0.f;
+#pragma unroll
+    for (int j = 0; j < AMAX; ++j) {
+      if (j >= acc.A) break;
+      const float v = ok ? val(j) : 0.f;
       const unsigned long long u = ok ? (unsigned long long)quantise(v, acc.kscale[j]) : 0ull;
       // exact 64-bit sum (mod 2^64) from three lane reductions of 21/21/22-bit parts
       const uint32_t s0 = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)(u & 0x1FFFFFull));
@@ -855,8 +857,10 @@ __device__ __forceinline__ void reduce_samples(const FeatAcc& acc, bool ok, int6
   // 2^-52 of the largest drop out, well inside the sums' fp64-level tolerance.
   const unsigned grp = __match_any_sync(act, fid);
   const int leader = __ffs(grp) - 1;
-  for (int j = 0; j < acc.A; ++j) {
-    const float v = __ldg(attr_p + (int64_t)j * P);
+#pragma unroll
+  for (int j = 0; j < AMAX; ++j) {
+    if (j >= acc.A) break;
+    const float v = val(j);
     const unsigned long long u = (unsigned long long)quantise(v, acc.kscale[j]);
     const unsigned long long qs = limb_sum(grp, u);
     const float d = isfinite(v) ? v : 0.f;
@@ -891,37 +895,29 @@ __device__ __forceinline__ void reduce_samples(const FeatAcc& acc, bool ok, int6
   }
 }
 
-// reduce_samples committing straight to the accumulators (copy blockIdx.x % K)
-__device__ __forceinline__ void accumulate_samples(const FeatAcc& acc, bool ok, int64_t fid,
-                                                   const float* attr_p, int64_t P) {
-  reduce_samples(acc, ok, fid, attr_p, P,
-                 [&](int64_t f, int j, unsigned long long qs, float h, float l, double w,
-                     bool dbl, bool) {
-                   const int64_t i = (int64_t)(blockIdx.x & (acc.K - 1)) * acc.F + f;
-                   atomicAdd(acc.sq + i * acc.A + j, qs);
-                   if (dbl) atomicAdd(acc.sa2 + i * acc.A + j, w);
-                   else add_pair(acc.sa2 + i * acc.A + j, h, l);
-                 });
-}
+// A warp's sums for some features kept in shared memory: the first feature the warp commits
+// claims its way (most point samples of a labelling often belong to one large feature), and its
+// later sums add there without atomics; every other feature goes straight to the accumulators.
+// Within one reduce_samples call a feature has one leader lane, so the cached sums have a single
+// writer at a time. A warp has kHotWays caches, a feature's by its index, and a block commits
+// what its warps hold once: each commit of a feature that most warps meet queues behind the
+// others' at the same few addresses. The sums of squares are fp64 (a few additions by one lane per
+// 32 samples): a double-float sum kept that long would lose digits of the deviations.
+constexpr int kHotWays = 4;
 
-// A warp's sums for one feature kept in shared memory: the first feature the warp commits
-// claims it (most point samples of a labelling often belong to one large feature), and its later
-// sums add there without atomics; every other feature goes straight to the accumulators. The
-// warp flushes the cache once at the end. Within one reduce_samples call a feature has one
-// leader lane, so the cached sums have a single writer at a time.
 struct HotCache {
   long long fid;
   unsigned long long sq[MSF_MAX_ATTR];
-  float sh[MSF_MAX_ATTR], sl[MSF_MAX_ATTR];  // sums of squares, double-float
+  double s2[MSF_MAX_ATTR];  // sums of squares
 };
 
-__device__ __forceinline__ void hot_clear(HotCache& h) {
-  if ((threadIdx.x & 31) == 0) {
-    h.fid = -1;
+__device__ __forceinline__ void hot_clear(HotCache (&h)[kHotWays]) {
+  const int lane = threadIdx.x & 31;
+  if (lane < kHotWays) {
+    h[lane].fid = -1;
     for (int j = 0; j < MSF_MAX_ATTR; ++j) {
-      h.sq[j] = 0ull;
-      h.sh[j] = 0.f;
-      h.sl[j] = 0.f;
+      h[lane].sq[j] = 0ull;
+      h[lane].s2[j] = 0.0;
     }
   }
   __syncwarp();
@@ -933,26 +929,25 @@ __device__ __forceinline__ void hot_commit(const FeatAcc& acc, HotCache& c) {
   const int64_t i = (int64_t)(blockIdx.x & (acc.K - 1)) * acc.F + c.fid;
   for (int j = 0; j < acc.A; ++j) {
     atomicAdd(acc.sq + i * acc.A + j, c.sq[j]);
-    add_pair(acc.sa2 + i * acc.A + j, c.sh[j], c.sl[j]);
+    atomicAdd(acc.sa2 + i * acc.A + j, c.s2[j]);
     c.sq[j] = 0ull;
-    c.sh[j] = c.sl[j] = 0.f;
+    c.s2[j] = 0.0;
   }
   c.fid = -1;
 }
 
-// reduce_samples committing through the warp's cache (double-float additions in fp32). With
-// EVICT a call whose samples all belong to one other feature commits the cached feature and
-// caches that one instead: samples walked in voxel order come in runs of one feature, and the
-// run at hand is the one worth caching.
-template <bool EVICT = false>
-__device__ __forceinline__ void accumulate_samples_hot(const FeatAcc& acc, HotCache& c, bool ok,
-                                                       int64_t fid, const float* attr_p,
-                                                       int64_t P) {
-  reduce_samples(acc, ok, fid, attr_p, P,
+// reduce_samples committing through the warp's caches. A call whose samples all belong to one
+// other feature commits the cached feature of its way and caches that one instead: samples walked
+// in voxel order come in runs of one feature, and the run at hand is the one worth caching.
+template <int AMAX, class Val>
+__device__ __forceinline__ void accumulate_samples_hot(const FeatAcc& acc, HotCache (&cs)[kHotWays],
+                                                       bool ok, int64_t fid, Val&& val) {
+  reduce_samples<AMAX>(acc, ok, fid, val,
                  [&](int64_t f, int j, unsigned long long qs, float h, float l, double w,
                      bool dbl, bool one) {
+                   HotCache& c = cs[(((uint32_t)f * 0x9E3779B1u) >> 16) & (kHotWays - 1)];
                    if (j == 0) {
-                     if (EVICT && one && c.fid != f) {
+                     if (one && c.fid != f) {
                        hot_commit(acc, c);  // the single leader of this call: no race
                        c.fid = f;
                      } else if (c.fid < 0) {
@@ -960,26 +955,37 @@ __device__ __forceinline__ void accumulate_samples_hot(const FeatAcc& acc, HotCa
                                  (unsigned long long)f);
                      }
                    }
-                   const int64_t i = (int64_t)(blockIdx.x & (acc.K - 1)) * acc.F + f;
                    if (c.fid == f) {
                      c.sq[j] += qs;
-                     if (dbl) atomicAdd(acc.sa2 + i * acc.A + j, w);
-                     else df_add2(c.sh[j], c.sl[j], h, l);
+                     c.s2[j] += dbl ? w : f2d(h) + f2d(l);
                      return;
                    }
+                   const int64_t i = (int64_t)(blockIdx.x & (acc.K - 1)) * acc.F + f;
                    atomicAdd(acc.sq + i * acc.A + j, qs);
                    if (dbl) atomicAdd(acc.sa2 + i * acc.A + j, w);
                    else add_pair(acc.sa2 + i * acc.A + j, h, l);
                  });
 }
 
-__device__ __forceinline__ void hot_flush(const FeatAcc& acc, HotCache& h) {
-  __syncwarp();
-  const int lane = threadIdx.x & 31;
-  if (h.fid >= 0 && lane < acc.A) {
-    const int64_t i = (int64_t)(blockIdx.x & (acc.K - 1)) * acc.F + h.fid;
-    atomicAdd(acc.sq + i * acc.A + lane, h.sq[lane]);
-    add_pair(acc.sa2 + i * acc.A + lane, h.sh[lane], h.sl[lane]);
+// The caches of a block's 8 warps into the accumulators, a feature's sums over the warps committed
+// once. All threads, after a barrier.
+__device__ __forceinline__ void hot_merge(const FeatAcc& acc, HotCache (&h)[8][kHotWays]) {
+  for (int i = threadIdx.x; i < kHotWays * 8 * acc.A; i += blockDim.x) {
+    const int j = i % acc.A, w = i / acc.A % 8, e = i / (8 * acc.A);
+    const long long f = h[w][e].fid;
+    bool first = f >= 0;
+    for (int k = 0; k < w; ++k) first &= h[k][e].fid != f;
+    if (!first) continue;
+    unsigned long long sq = 0ull;
+    double s2 = 0.0;
+    for (int k = w; k < 8; ++k)
+      if (h[k][e].fid == f) {
+        sq += h[k][e].sq[j];
+        s2 += h[k][e].s2[j];
+      }
+    const int64_t o = ((int64_t)(blockIdx.x & (acc.K - 1)) * acc.F + f) * acc.A + j;
+    atomicAdd(acc.sq + o, sq);
+    atomicAdd(acc.sa2 + o, s2);
   }
 }
 
