@@ -257,24 +257,33 @@ __device__ __forceinline__ void pred4(const DevPred& pr, const uint4& r, bool& b
   }
 }
 
-// Bits 0..7 of b to bits 0, 4, 8, .., 28.
-__device__ __forceinline__ uint32_t spread4(uint32_t b) {
-  b &= 0xFFu;
-  b = (b | (b << 12)) & 0x000F000Fu;
-  b = (b | (b << 6)) & 0x03030303u;
-  b = (b | (b << 3)) & 0x11111111u;
-  return b;
+// Eight lanes hold one 32-voxel row, four voxels each (lane 8r + q: voxels 4q .. 4q+3 of row
+// r, bits b0..b3). Each lane's four bits go to their place and three exchanges put the row
+// together (in all eight lanes); four ballots and spreading their bits took four times the
+// instructions. All lanes must call it.
+__device__ __forceinline__ uint32_t row_mask4(int lane, bool b0, bool b1, bool b2, bool b3) {
+  uint32_t w = ((b0 ? 1u : 0u) | (b1 ? 2u : 0u) | (b2 ? 4u : 0u) | (b3 ? 8u : 0u))
+               << (4 * (lane & 7));
+  w |= __shfl_xor_sync(0xFFFFFFFFu, w, 1);
+  w |= __shfl_xor_sync(0xFFFFFFFFu, w, 2);
+  w |= __shfl_xor_sync(0xFFFFFFFFu, w, 4);
+  return w;
 }
 
-// Eight lanes hold one 32-voxel row, four voxels each (lane 8r + q: voxels 4q .. 4q+3 of row
-// r, bits b0..b3). Four warp ballots put the row masks together; the value is meaningful in
-// lane 8r. All lanes must call it.
-__device__ __forceinline__ uint32_t row_mask4(int lane, bool b0, bool b1, bool b2, bool b3) {
-  const uint32_t B0 = __ballot_sync(0xFFFFFFFFu, b0), B1 = __ballot_sync(0xFFFFFFFFu, b1);
-  const uint32_t B2 = __ballot_sync(0xFFFFFFFFu, b2), B3 = __ballot_sync(0xFFFFFFFFu, b3);
-  const int sh = lane & 24;
-  return spread4(B0 >> sh) | (spread4(B1 >> sh) << 1) | (spread4(B2 >> sh) << 2) |
-         (spread4(B3 >> sh) << 3);
+// Window-linear index of the first voxel of row s of a tile (thread s's row), kNoRow outside the
+// window; a window has fewer than 2^31 voxel-timesteps. A thread forms its own row's once, and
+// the passes over the rows of its warp take them from its lanes (the tile and label passes are
+// bound by instruction issue: sixteen queries on 192^3, tile pass 6.33 -> 5.30 ms, labels 2.10 ->
+// 1.54 ms; 256^3 x 24, labels 0.33 -> 0.29 ms).
+constexpr uint32_t kNoRow = 0xFFFFFFFFu;
+__device__ __forceinline__ uint32_t row_start(const Geometry& g, const TileCoord& tc, int s) {
+  const int y = (tc.ty << g.lby) + (s & ((1 << g.lby) - 1));
+  const int z = (tc.tz << g.lbz) + ((s >> g.lby) & ((1 << g.lbz) - 1));
+  const int tw = (tc.tt << g.lbt) + (s >> (g.lby + g.lbz)) - g.toff;
+  if (y >= g.ny || z >= g.nz || tw < 0 || tw >= g.tw) return kNoRow;
+  return (((uint32_t)tw * (uint32_t)g.nz + (uint32_t)z) * (uint32_t)g.ny + (uint32_t)y) *
+             (uint32_t)g.nx +
+         (uint32_t)tc.xs * 32u;
 }
 
 struct TileSmem {
@@ -311,21 +320,21 @@ __device__ __forceinline__ void tile_body(const SegArgs& a, const int tile, cons
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const TileCoord tc = tile_coord(g, tile);
   const int BY = 1 << g.lby, BZ = 1 << g.lbz;
+  const uint32_t row = row_start(g, tc, tid);  // this thread's row
+  // its place in the row table
+  const uint32_t gs = row == kNoRow ? 0u : (g.nx & 31) == 0 ? row >> 5
+                                          : (row - (uint32_t)tc.xs * 32u) / (uint32_t)g.nx *
+                                                    (uint32_t)g.nxs + (uint32_t)tc.xs;
 
   // ---- phase 1: criterion, one 32-bit activity mask per row -------------------------------
+  const int64_t w0 = (int64_t)g.t0 * g.V;  // the window in the predicate arrays
   if constexpr (NP < 0) {
     // masks already formed by k_mask (kept in the row table's mask word)
-    const int sg = tid;
-    const int ly = sg & (BY - 1), lz = (sg >> g.lby) & (BZ - 1), lt = sg >> (g.lby + g.lbz);
-    const int y = tc.ty * BY + ly, z = tc.tz * BZ + lz, tw = (tc.tt << g.lbt) + lt - g.toff;
-    uint32_t mm = 0u;
-    if (y < g.ny && z < g.nz && tw >= 0 && tw < g.tw)
-      mm = __ldcg(reinterpret_cast<const uint32_t*>(a.seg) + 2 * seg_index(g, tw, z, y, tc.xs));
-    s_mask[sg] = mm;
+    s_mask[tid] = row != kNoRow ? __ldcg(reinterpret_cast<const uint32_t*>(a.seg + gs)) : 0u;
   } else if (VEC) {
     // 16-byte loads: lane = (row r of 4, x-quad q of 8); 4 rows per warp instruction.
     const int q = lane & 7, rsub = lane >> 3;
-    const int x4 = tc.xs * 32 + 4 * q;
+    const bool xin = tc.xs * 32 + 4 * q < g.nx;
     constexpr int U = NP <= 2 ? 4 : 2;
 #pragma unroll 1
     for (int it = 0; it < 8; it += U) {
@@ -333,15 +342,13 @@ __device__ __forceinline__ void tile_body(const SegArgs& a, const int tile, cons
       bool valid[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int sg = warp * 32 + 4 * (it + u) + rsub;
-        const int ly = sg & (BY - 1), lz = (sg >> g.lby) & (BZ - 1), lt = sg >> (g.lby + g.lbz);
-        const int y = tc.ty * BY + ly, z = tc.tz * BZ + lz, tw = (tc.tt << g.lbt) + lt - g.toff;
-        valid[u] = x4 < g.nx && y < g.ny && z < g.nz && tw >= 0 && tw < g.tw;
-        const int64_t off = (int64_t)(g.t0 + tw) * g.V + (int64_t)(z * g.ny + y) * g.nx + x4;
+        const uint32_t off = __shfl_sync(0xFFFFFFFFu, row, 4 * (it + u) + rsub);
+        valid[u] = xin && off != kNoRow;
 #pragma unroll
         for (int j = 0; j < NP; ++j)
           raw[u][j] = valid[u] ? __ldcs(reinterpret_cast<const uint4*>(
-                                     static_cast<const unsigned int*>(a.pred[j].base) + off))
+                                     static_cast<const unsigned int*>(a.pred[j].base) + w0 +
+                                     (off + 4u * q)))
                                : make_uint4(0, 0, 0, 0);
       }
 #pragma unroll
@@ -354,7 +361,7 @@ __device__ __forceinline__ void tile_body(const SegArgs& a, const int tile, cons
       }
     }
   } else {
-    const int x = tc.xs * 32 + lane;
+    const bool xin = tc.xs * 32 + lane < g.nx;
     constexpr int U = 8;
 #pragma unroll 1
     for (int i = 0; i < 32; i += U) {
@@ -362,14 +369,13 @@ __device__ __forceinline__ void tile_body(const SegArgs& a, const int tile, cons
       bool valid[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int sg = warp * 32 + i + u;
-        const int ly = sg & (BY - 1), lz = (sg >> g.lby) & (BZ - 1), lt = sg >> (g.lby + g.lbz);
-        const int y = tc.ty * BY + ly, z = tc.tz * BZ + lz, tw = (tc.tt << g.lbt) + lt - g.toff;
-        valid[u] = x < g.nx && y < g.ny && z < g.nz && tw >= 0 && tw < g.tw;
-        const int64_t off = (int64_t)(g.t0 + tw) * g.V + (int64_t)(z * g.ny + y) * g.nx + x;
+        const uint32_t off = __shfl_sync(0xFFFFFFFFu, row, i + u);
+        valid[u] = xin && off != kNoRow;
 #pragma unroll
         for (int j = 0; j < NP; ++j)
-          raw[u][j] = valid[u] ? __ldcs(static_cast<const unsigned int*>(a.pred[j].base) + off) : 0u;
+          raw[u][j] = valid[u] ? __ldcs(static_cast<const unsigned int*>(a.pred[j].base) + w0 +
+                                        (off + (uint32_t)lane))
+                               : 0u;
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
@@ -487,9 +493,7 @@ __device__ __forceinline__ void tile_body(const SegArgs& a, const int tile, cons
   }
   const uint32_t rbase = (uint32_t)tile * (uint32_t)a.maxr;
   const uint32_t cbase = (uint32_t)tile * (uint32_t)g.cmax;
-  const int y = tc.ty * BY + ly, z = tc.tz * BZ + lz, tw = (tc.tt << g.lbt) + lt - g.toff;
-  if (y < g.ny && z < g.nz && tw >= 0 && tw < g.tw) {
-    const int64_t gs = (((int64_t)tw * g.nz + z) * g.ny + y) * g.nxs + tc.xs;
+  if (row != kNoRow) {
     a.seg[gs] = make_uint2(m, rbase + rb);
     uint32_t bits = st;
     for (int j = 0; j < nr; ++j) {
@@ -501,7 +505,7 @@ __device__ __forceinline__ void tile_body(const SegArgs& a, const int tile, cons
       a.runcomp[rbase + r] = c;
       if (root == r) {
         a.cparent[c] = c;
-        a.cminli[c] = (int32_t)((((int64_t)tw * g.nz + z) * g.ny + y) * g.nx + tc.xs * 32 + x0);
+        a.cminli[c] = (int32_t)(row + (uint32_t)x0);
       }
     }
   }
@@ -887,76 +891,63 @@ __global__ void __launch_bounds__(256) k_flatten(const __grid_constant__ SegArgs
 // k_final: stream out the int32 labels
 // ---------------------------------------------------------------------------------------------
 template <bool SPATIAL, bool VEC>
-__device__ __forceinline__ void final_body(const SegArgs& a, const int tile, int32_t* s_lbl,
-                                           uint32_t* s_mask, uint32_t* s_rb) {
+__device__ __forceinline__ void final_body(const SegArgs& a, const int tile, int32_t* s_lbl) {
   constexpr int MAXR = kSegPerTile * (SPATIAL ? 16 : 32);
   const Geometry& g = a.g;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
   const TileCoord tc = tile_coord(g, tile);
-  const int BY = 1 << g.lby, BZ = 1 << g.lbz;
+  const uint32_t row = row_start(g, tc, tid);  // this thread's row, its mask and first run
   const int nrun = min(__ldcg(&a.tileinfo[tile].x), MAXR);
   const uint32_t rbase = (uint32_t)tile * (uint32_t)a.maxr;
+  uint32_t mask = 0u, rb = 0u;
+  if (nrun && row != kNoRow) {
+    const uint32_t gs = (g.nx & 31) == 0 ? row >> 5
+                                         : (row - (uint32_t)tc.xs * 32u) / (uint32_t)g.nx *
+                                                   (uint32_t)g.nxs + (uint32_t)tc.xs;
+    const uint2 e = __ldcg(a.seg + gs);
+    mask = e.x;
+    rb = e.y - rbase;
+  }
   for (int r = tid; r < nrun; r += 256) {
     const uint32_t c = __ldcg(a.runcomp + rbase + r);
     s_lbl[r] = __ldcg(a.cminli + __ldcg(a.cparent + c));
-  }
-  {
-    const int s = tid;
-    const int ly = s & (BY - 1), lz = (s >> g.lby) & (BZ - 1), lt = s >> (g.lby + g.lbz);
-    const int y = tc.ty * BY + ly, z = tc.tz * BZ + lz, tw = (tc.tt << g.lbt) + lt - g.toff;
-    uint32_t mm = 0, rr = 0;
-    if (nrun && y < g.ny && z < g.nz && tw >= 0 && tw < g.tw) {
-      const int64_t gs = seg_index(g, tw, z, y, tc.xs);
-      const uint2 e = __ldcg(a.seg + gs);
-      mm = e.x;
-      rr = e.y - rbase;
-    }
-    s_mask[s] = mm;
-    s_rb[s] = rr;
   }
   __syncthreads();
   if (VEC) {
     // 16-byte stores: lane = (row r of 4, x-quad q of 8)
     const int q = lane & 7, rsub = lane >> 3;
-    const int x4 = tc.xs * 32 + 4 * q;
-    if (x4 >= g.nx) return;
+    const bool xin = tc.xs * 32 + 4 * q < g.nx;
 #pragma unroll 2
     for (int it = 0; it < 8; ++it) {
-      const int sg = warp * 32 + 4 * it + rsub;
-      const int ly = sg & (BY - 1), lz = (sg >> g.lby) & (BZ - 1), lt = sg >> (g.lby + g.lbz);
-      const int y = tc.ty * BY + ly, z = tc.tz * BZ + lz, tw = (tc.tt << g.lbt) + lt - g.toff;
-      if (y >= g.ny || z >= g.nz || tw < 0 || tw >= g.tw) continue;
-      const uint32_t m = s_mask[sg];
+      const uint32_t off = __shfl_sync(0xFFFFFFFFu, row, 4 * it + rsub);
+      const uint32_t m = __shfl_sync(0xFFFFFFFFu, mask, 4 * it + rsub);
+      const uint32_t r0 = __shfl_sync(0xFFFFFFFFu, rb, 4 * it + rsub);
+      if (!xin || off == kNoRow) continue;
       int4 o = make_int4(-1, -1, -1, -1);
       if ((m >> (4 * q)) & 0xFu) {
         const uint32_t st = run_starts(m, SPATIAL);
-        const uint32_t rb = s_rb[sg];
         int v[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const int b = 4 * q + e;
-          v[e] = ((m >> b) & 1u) ? s_lbl[rb + run_index(st, b)] : -1;
+          v[e] = ((m >> b) & 1u) ? s_lbl[r0 + run_index(st, b)] : -1;
         }
         o = make_int4(v[0], v[1], v[2], v[3]);
       }
-      __stcs(reinterpret_cast<int4*>(a.labels + (int64_t)tw * g.V +
-                                     (int64_t)(z * g.ny + y) * g.nx + x4),
-             o);
+      __stcs(reinterpret_cast<int4*>(a.labels + (off + 4u * q)), o);
     }
     return;
   }
-  const int x = tc.xs * 32 + lane;
-  if (x >= g.nx) return;
+  const bool xin = tc.xs * 32 + lane < g.nx;
 #pragma unroll 4
   for (int i = 0; i < 32; ++i) {
-    const int sg = warp * 32 + i;
-    const int ly = sg & (BY - 1), lz = (sg >> g.lby) & (BZ - 1), lt = sg >> (g.lby + g.lbz);
-    const int y = tc.ty * BY + ly, z = tc.tz * BZ + lz, tw = (tc.tt << g.lbt) + lt - g.toff;
-    if (y >= g.ny || z >= g.nz || tw < 0 || tw >= g.tw) continue;
-    const uint32_t m = s_mask[sg];
+    const uint32_t off = __shfl_sync(0xFFFFFFFFu, row, i);
+    const uint32_t m = __shfl_sync(0xFFFFFFFFu, mask, i);
+    const uint32_t r0 = __shfl_sync(0xFFFFFFFFu, rb, i);
+    if (!xin || off == kNoRow) continue;
     int32_t lbl = -1;
-    if ((m >> lane) & 1u) lbl = s_lbl[s_rb[sg] + run_index(run_starts(m, SPATIAL), lane)];
-    __stcs(a.labels + (int64_t)tw * g.V + (int64_t)(z * g.ny + y) * g.nx + x, lbl);
+    if ((m >> lane) & 1u) lbl = s_lbl[r0 + run_index(run_starts(m, SPATIAL), lane)];
+    __stcs(a.labels + (off + (uint32_t)lane), lbl);
   }
 }
 
@@ -964,9 +955,7 @@ template <bool SPATIAL, bool VEC>
 __global__ void __launch_bounds__(256) k_final(const __grid_constant__ SegArgs a) {
   constexpr int MAXR = kSegPerTile * (SPATIAL ? 16 : 32);
   __shared__ int32_t s_lbl[MAXR];
-  __shared__ uint32_t s_mask[kSegPerTile];
-  __shared__ uint32_t s_rb[kSegPerTile];
-  final_body<SPATIAL, VEC>(a, blockIdx.x, s_lbl, s_mask, s_rb);
+  final_body<SPATIAL, VEC>(a, blockIdx.x, s_lbl);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -2120,13 +2109,11 @@ template <bool SPATIAL, bool VEC>
 __global__ void __launch_bounds__(256) k_final_batch(const __grid_constant__ BatchPlan b) {
   constexpr int MAXR = kSegPerTile * (SPATIAL ? 16 : 32);
   __shared__ int32_t s_lbl[MAXR];
-  __shared__ uint32_t s_mask[kSegPerTile];
-  __shared__ uint32_t s_rb[kSegPerTile];
   __shared__ __align__(16) SegArgs s_args;
   load_args(&s_args, b.qargs + blockIdx.y);
   __syncthreads();
   for (int tile = blockIdx.x; tile < s_args.g.ntiles; tile += gridDim.x) {
-    final_body<SPATIAL, VEC>(s_args, tile, s_lbl, s_mask, s_rb);
+    final_body<SPATIAL, VEC>(s_args, tile, s_lbl);
     __syncthreads();
   }
 }
@@ -2246,7 +2233,7 @@ __global__ void __launch_bounds__(256, 4) k_batch_fused(const __grid_constant__ 
     } else if (type == kFFlat) {
       flatten_body(s_args, (int)idx, &s_n);
     } else {
-      final_body<SPATIAL, VEC>(s_args, (int)idx, reinterpret_cast<int32_t*>(s_dyn), s_mask, s_rb);
+      final_body<SPATIAL, VEC>(s_args, (int)idx, reinterpret_cast<int32_t*>(s_dyn));
     }
     __syncthreads();
     if (threadIdx.x == 0 && type != kFFinal) {
