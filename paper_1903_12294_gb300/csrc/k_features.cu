@@ -42,6 +42,7 @@ struct FeatArgs {
   FeatAcc acc;
   RankArrays rk;
   double scale[MSF_MAX_ATTR];
+  const int32_t* flabel;  // [F] the features' labels (fast path)
   msf_feature* out;
 };
 
@@ -164,28 +165,8 @@ __global__ void __launch_bounds__(256) k_scan_down(const __grid_constant__ FeatA
 }
 
 __global__ void __launch_bounds__(256) k_feat_init(const __grid_constant__ FeatArgs a) {
-  const FeatAcc& c = a.acc;
-  const int64_t n = c.F * c.K;
-  const unsigned kmin0 = float_key(INFINITY), kmax0 = float_key(-INFINITY);
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    c.n_vox[i] = 0;
-    c.n_pts[i] = 0;
-    c.sf[i] = 0.0;
-    c.sf2[i] = 0.0;
-    c.fmin[i] = kmin0;
-    c.fmax[i] = kmax0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      c.bbmin[i * 4 + j] = 0x7FFFFFFF;
-      c.bbmax[i * 4 + j] = -1;
-      c.sc[i * 4 + j] = 0;
-    }
-    for (int k = 0; k < c.A; ++k) {
-      c.sq[i * c.A + k] = 0;
-      c.sa2[i * c.A + k] = 0.0;
-    }
-  }
+  acc_init(a.acc, (int64_t)blockIdx.x * blockDim.x + threadIdx.x,
+           (int64_t)gridDim.x * blockDim.x);
 }
 
 // Generic path: 64 consecutive 32-voxel rows (t, z, y, xs) per block, one warp per row at a time
@@ -254,69 +235,100 @@ __global__ void __launch_bounds__(256) k_pts(const __grid_constant__ FeatArgs a)
   hot_merge(a.acc, s_hot);
 }
 
-__global__ void __launch_bounds__(256) k_records(const __grid_constant__ FeatArgs a) {
-  const int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// x / n from r = 1 / n: one correction step with the exact residual, for several quotients by one
+// n (an fp64 division is a chain of operations on this part's narrow pipe).
+__device__ __forceinline__ double div_by(double x, double n, double r) {
+  const double q = __dmul_rn(x, r);
+  return isfinite(q) ? __fma_rn(__fma_rn(-q, n, x), r, q) : q;
+}
+
+// One lane per (feature, copy): the K copies of a feature lie in neighbouring lanes and are summed
+// by exchanges (one thread per feature walked them one after the other, 26 us of a small step).
+// The records go through shared memory so that the block stores them as one run of words (each
+// thread storing its own 312 bytes took 0.27 ms for 584K features, now 0.21 ms).
+constexpr int kRecNT = 128;
+constexpr int kRecWords = (int)(sizeof(msf_feature) / 8);
+static_assert(sizeof(msf_feature) == 8 * kRecWords, "records are whole 8-byte words");
+
+__global__ void __launch_bounds__(kRecNT) k_records(const __grid_constant__ FeatArgs a) {
+  __shared__ __align__(16) unsigned long long s_rec[kRecNT * kRecWords];
+  constexpr unsigned W = 0xFFFFFFFFu;
   const FeatAcc& c = a.acc;
-  if (f >= c.F) return;
-  // sum the K copies
-  unsigned long long nv = 0, np = 0, sc[4] = {0, 0, 0, 0};
-  double sf = 0.0, sf2 = 0.0;
-  unsigned kmin = 0xFFFFFFFFu, kmax = 0u;
-  int bmin[4] = {0x7FFFFFFF, 0x7FFFFFFF, 0x7FFFFFFF, 0x7FFFFFFF}, bmax[4] = {-1, -1, -1, -1};
-  unsigned long long sq[MSF_MAX_ATTR] = {};
-  double sa2[MSF_MAX_ATTR] = {};
-  for (int k = 0; k < c.K; ++k) {
-    const int64_t i = (int64_t)k * c.F + f;
-    nv += c.n_vox[i];
-    np += c.n_pts[i];
-    sf += c.sf[i];
-    sf2 += c.sf2[i];
-    kmin = min(kmin, c.fmin[i]);
-    kmax = max(kmax, c.fmax[i]);
-    for (int j = 0; j < 4; ++j) {
-      bmin[j] = min(bmin[j], c.bbmin[i * 4 + j]);
-      bmax[j] = max(bmax[j], c.bbmax[i * 4 + j]);
-      sc[j] += c.sc[i * 4 + j];
-    }
-    for (int j = 0; j < a.A; ++j) {
-      sq[j] += c.sq[i * a.A + j];
-      sa2[j] += c.sa2[i * a.A + j];
-    }
-  }
-  msf_feature o;
-  memset(&o, 0, sizeof(o));
-  const double n = (double)nv;
+  const int per = kRecNT / c.K;  // features per block (K: a power of two, at most 16)
+  const int fl = threadIdx.x / c.K, k = threadIdx.x % c.K;
+  const int64_t f = (int64_t)blockIdx.x * per + fl;
+  const bool in = f < c.F;
+  const int64_t i = in ? (int64_t)k * c.F + f : 0;
+  auto sum = [&](unsigned long long v) {
+    v = in ? v : 0ull;
+    for (int o = c.K >> 1; o; o >>= 1) v += __shfl_xor_sync(W, v, o);
+    return v;
+  };
+  auto sumd = [&](double v) {
+    v = in ? v : 0.0;
+    for (int o = c.K >> 1; o; o >>= 1) v += __shfl_xor_sync(W, v, o);
+    return v;
+  };
+  auto least = [&](auto v) {
+    for (int o = c.K >> 1; o; o >>= 1) v = min(v, __shfl_xor_sync(W, v, o));
+    return v;
+  };
+  auto most = [&](auto v) {
+    for (int o = c.K >> 1; o; o >>= 1) v = max(v, __shfl_xor_sync(W, v, o));
+    return v;
+  };
+  const unsigned long long nv = sum(c.n_vox[i]), np = sum(c.n_pts[i]);
+  const double sf = sumd(c.sf[i]), sf2 = sumd(c.sf2[i]);
+  const unsigned kmin = least(c.fmin[i]), kmax = most(c.fmax[i]);
+  const int4 b0 = reinterpret_cast<const int4*>(c.bbmin)[i];
+  const int4 b1 = reinterpret_cast<const int4*>(c.bbmax)[i];
+  const int bmin[4] = {least(b0.x), least(b0.y), least(b0.z), least(b0.w)};
+  const int bmax[4] = {most(b1.x), most(b1.y), most(b1.z), most(b1.w)};
+  msf_feature& o = *reinterpret_cast<msf_feature*>(s_rec + fl * kRecWords);
+  if (k == 0)
+    for (int j = 0; j < kRecWords; ++j) s_rec[fl * kRecWords + j] = 0ull;
+  const double n = (double)nv, rn = __drcp_rn(n), npd = (double)np;
   for (int j = 0; j < 4; ++j) {
-    o.bbox_min[j] = bmin[j];
-    o.bbox_max[j] = bmax[j];
-    o.centroid[j] = (double)sc[j] / n;
+    const unsigned long long sc = sum(c.sc[i * 4 + j]);
+    if (k == 0) {
+      o.bbox_min[j] = bmin[j];
+      o.bbox_max[j] = bmax[j];
+      o.centroid[j] = div_by((double)sc, n, rn);
+    }
   }
-  o.label = -1;  // set by k_labels
-  o.n_attr = a.A;
-  o.n_vox = (int64_t)nv;
-  o.n_pts = (int64_t)np;
-  o.sum_field = sf;
-  o.mean_field = sf / n;
-  const double var = sf2 / n - o.mean_field * o.mean_field;
-  o.std_field = sqrt(var > 0.0 ? var : 0.0);
-  o.min_field = key_float(kmin);
-  o.max_field = key_float(kmax);
+  if (k == 0) {
+    o.label = a.flabel ? (in ? a.flabel[f] : 0) : -1;  // -1: set by k_labels
+    o.n_attr = a.A;
+    o.n_vox = (int64_t)nv;
+    o.n_pts = (int64_t)np;
+    o.sum_field = sf;
+    o.mean_field = sf / n;
+    const double var = sf2 / n - o.mean_field * o.mean_field;
+    o.std_field = sqrt(var > 0.0 ? var : 0.0);
+    o.min_field = key_float(kmin);
+    o.max_field = key_float(kmax);
+  }
   const double qnan = __longlong_as_double(0x7ff8000000000000ll);
   for (int j = 0; j < a.A; ++j) {
-    const long long s = (long long)sq[j];
+    const long long s = (long long)sum(c.sq[i * a.A + j]);
+    const double sa2 = sumd(c.sa2[i * a.A + j]);
+    if (k) continue;
     o.sumq[j] = s;
-    if (o.n_pts == 0) {
+    if (np == 0) {
       o.mean_attr[j] = qnan;
       o.std_attr[j] = qnan;
     } else {
-      const double npd = (double)o.n_pts;
       const double m = (double)s / (npd * a.scale[j]);
       o.mean_attr[j] = m;
-      const double v = sa2[j] / npd - m * m;
+      const double v = sa2 / npd - m * m;
       o.std_attr[j] = sqrt(v > 0.0 ? v : 0.0);
     }
   }
-  a.out[f] = o;
+  __syncthreads();
+  const int64_t w0 = (int64_t)blockIdx.x * per * kRecWords;
+  const int nw = (int)min((int64_t)per, c.F - (int64_t)blockIdx.x * per) * kRecWords;
+  unsigned long long* out = reinterpret_cast<unsigned long long*>(a.out) + w0;
+  for (int j = threadIdx.x; j < nw; j += kRecNT) out[j] = s_rec[j];
 }
 
 // label of feature f = position of the f-th set bit
@@ -383,13 +395,11 @@ int features_run(msf_ctx* ctx, const msf_criteria* crit, const int32_t* labels,
   a.counters = ctx->seg.counters.as<unsigned long long>() + 4;  // [0..3] belong to msf_segment
   a.rk = RankArrays{a.rootbits, a.wordrank, a.N};
   cudaStream_t s = ctx->stream;
-  MSF_CUDA_TRY(cudaMemsetAsync(a.counters, 0, 2 * sizeof(unsigned long long), s));
   unsigned long long F = 0;
   if (fast) {
-    MSF_CUDA_TRY(cudaMemsetAsync(a.rootbits, 0, sizeof(uint32_t) * a.nwords, s));
-    MSF_TRY(seg_mark_roots(ctx, a.rootbits, a.counters));
     F = (unsigned long long)ctx->last.n_features;
   } else {
+    MSF_CUDA_TRY(cudaMemsetAsync(a.counters, 0, 2 * sizeof(unsigned long long), s));
     if (!labels) return MSF_ERR_INVALID_ARG;
     {
       ScopedKernel k(ctx, "k_rootbits");
@@ -419,7 +429,7 @@ int features_run(msf_ctx* ctx, const msf_criteria* crit, const int32_t* labels,
   auto r256 = [](size_t n) { return (n + 255) & ~size_t(255); };
   const size_t bytes = 4 * r256(f8) + r256(f8 * 4) + 2 * r256(f8 * Af) +
                        2 * r256(sizeof(unsigned) * FK) + 2 * r256(sizeof(int) * FK * 4) +
-                       r256(sizeof(msf_feature) * F);
+                       r256(sizeof(int32_t) * F) + r256(sizeof(msf_feature) * F);
   MSF_TRY(S.acc.ensure(bytes));
   char* p = S.acc.as<char>();
   auto carve = [&](size_t n) {
@@ -438,28 +448,39 @@ int features_run(msf_ctx* ctx, const msf_criteria* crit, const int32_t* labels,
   a.acc.fmax = reinterpret_cast<unsigned*>(carve(sizeof(unsigned) * FK));
   a.acc.bbmin = reinterpret_cast<int*>(carve(sizeof(int) * FK * 4));
   a.acc.bbmax = reinterpret_cast<int*>(carve(sizeof(int) * FK * 4));
+  int32_t* flabel = reinterpret_cast<int32_t*>(carve(sizeof(int32_t) * F));
+  a.flabel = fast ? flabel : nullptr;
   a.out = out_kind == MSF_DEVICE ? out
                                  : reinterpret_cast<msf_feature*>(carve(sizeof(msf_feature) * F));
-  const unsigned fb = (unsigned)((F + 255) / 256);
-  {
-    ScopedKernel k(ctx, "k_scan_reduce");
-    k_scan_reduce<<<(unsigned)nblk, 256, 0, s>>>(a);
-  }
-  {
-    ScopedKernel k(ctx, "k_scan_top");
-    k_scan_top<<<1, 1024, 0, s>>>(a.blocksums, (int)nblk);
-  }
-  {
-    ScopedKernel k(ctx, "k_scan_down");
-    k_scan_down<<<(unsigned)nblk, 256, 0, s>>>(a);
-  }
-  {
-    ScopedKernel k(ctx, "k_feat_init");
-    const int64_t nb = (FK + 255) / 256;
-    k_feat_init<<<(unsigned)std::min<int64_t>(nb, (int64_t)ctx->sm_count * 16), 256, 0, s>>>(a);
+  const unsigned fb = (unsigned)((F * K + kRecNT - 1) / kRecNT);
+  const bool ranked = fast && a.nwords <= kRankWords;
+  if (ranked) {
+    MSF_TRY(seg_feature_ranks(ctx, a.nwords, a.acc, flabel));
+  } else {
+    if (fast) {
+      MSF_CUDA_TRY(cudaMemsetAsync(a.rootbits, 0, sizeof(uint32_t) * a.nwords, s));
+      MSF_TRY(seg_mark_roots(ctx, a.rootbits));
+    }
+    {
+      ScopedKernel k(ctx, "k_scan_reduce");
+      k_scan_reduce<<<(unsigned)nblk, 256, 0, s>>>(a);
+    }
+    {
+      ScopedKernel k(ctx, "k_scan_top");
+      k_scan_top<<<1, 1024, 0, s>>>(a.blocksums, (int)nblk);
+    }
+    {
+      ScopedKernel k(ctx, "k_scan_down");
+      k_scan_down<<<(unsigned)nblk, 256, 0, s>>>(a);
+    }
+    {
+      ScopedKernel k(ctx, "k_feat_init");
+      const int64_t nb = (FK + 255) / 256;
+      k_feat_init<<<(unsigned)std::min<int64_t>(nb, (int64_t)ctx->sm_count * 16), 256, 0, s>>>(a);
+    }
   }
   if (fast) {
-    MSF_TRY(seg_feature_stats(ctx, a.rk, a.acc));
+    MSF_TRY(seg_feature_stats(ctx, a.rk, a.acc, flabel, ranked));
   } else {
     {
       ScopedKernel k(ctx, "k_vox");
@@ -474,15 +495,16 @@ int features_run(msf_ctx* ctx, const msf_criteria* crit, const int32_t* labels,
   }
   {
     ScopedKernel k(ctx, "k_records");
-    k_records<<<fb, 256, 0, s>>>(a);
+    k_records<<<fb, kRecNT, 0, s>>>(a);
   }
-  {
+  if (!fast) {
     ScopedKernel k(ctx, "k_labels");
     k_labels<<<(unsigned)((a.nwords + 255) / 256), 256, 0, s>>>(a);
   }
   MSF_CUDA_TRY(cudaGetLastError());
   unsigned long long bad = 0;
-  MSF_CUDA_TRY(cudaMemcpyAsync(&bad, a.counters + 1, sizeof(bad), cudaMemcpyDeviceToHost, s));
+  if (!fast)  // (the retained segmentation's labels are canonical)
+    MSF_CUDA_TRY(cudaMemcpyAsync(&bad, a.counters + 1, sizeof(bad), cudaMemcpyDeviceToHost, s));
   if (out_kind == MSF_HOST)
     MSF_CUDA_TRY(cudaMemcpyAsync(out, a.out, sizeof(msf_feature) * F, cudaMemcpyDeviceToHost, s));
   MSF_CUDA_TRY(cudaStreamSynchronize(s));

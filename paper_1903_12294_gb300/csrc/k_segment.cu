@@ -1371,16 +1371,78 @@ __global__ void __launch_bounds__(256) k_mark_roots(const __grid_constant__ SegA
   }
 }
 
-// Feature rank of every component (through its root's label).
+// Feature rank of every component (through its root's label), and the features' labels.
 __global__ void __launch_bounds__(256) k_comp_fid(const __grid_constant__ SegArgs a,
-                                                  RankArrays rk, int32_t* cfid) {
+                                                  RankArrays rk, int32_t* cfid,
+                                                  int32_t* flabel) {
   const int tile = blockIdx.x;
   const int nc = min(a.tileinfo[tile].y, a.g.cmax);
   const uint32_t cbase = (uint32_t)tile * (uint32_t)a.g.cmax;
   for (int k = threadIdx.x; k < nc; k += blockDim.x) {
     const uint32_t c = cbase + k;
-    cfid[c] = (int32_t)feature_rank(rk, __ldg(a.cminli + __ldg(a.cparent + c)));
+    const uint32_t r = __ldg(a.cparent + c);
+    const int32_t lbl = __ldg(a.cminli + r);
+    const int32_t f = (int32_t)feature_rank(rk, lbl);
+    cfid[c] = f;
+    if (r == c) flabel[f] = lbl;
   }
+}
+
+// The same for a small window in one launch: block 0 sets the label bits in shared memory, counts
+// them and ranks every component; the other blocks empty the accumulators. A small step is a
+// chain of launches of a few microseconds each, and clearing the bits, marking, three scans,
+// clearing and ranking were seven of them (32^3 x 8: 351 us the step, now 304 us).
+__global__ void __launch_bounds__(1024) k_feat_ranks(const __grid_constant__ SegArgs a,
+                                                     FeatAcc acc, int32_t* cfid, int32_t* flabel,
+                                                     int nwords) {
+  extern __shared__ uint32_t s_bits[];  // [nwords]
+  __shared__ uint32_t s_base[1024];     // label bits before the thread's words
+  __shared__ uint32_t s_warp[32];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  if (blockIdx.x > 0) {
+    acc_init(acc, (int64_t)(blockIdx.x - 1) * 1024 + tid, (int64_t)(gridDim.x - 1) * 1024);
+    return;
+  }
+  for (int i = tid; i < nwords; i += 1024) s_bits[i] = 0u;
+  __syncthreads();
+  auto components = [&](auto&& f) {  // 64 threads per tile
+    for (int i = tid; i < a.g.ntiles * 64; i += 1024) {
+      const int tile = i >> 6;
+      const int nc = min(__ldg(&a.tileinfo[tile].y), a.g.cmax);
+      for (int k = i & 63; k < nc; k += 64) f((uint32_t)tile * (uint32_t)a.g.cmax + k);
+    }
+  };
+  components([&](uint32_t c) {
+    if (__ldg(a.cparent + c) != c) return;
+    const int32_t lbl = __ldg(a.cminli + c);
+    atomicOr(s_bits + (lbl >> 5), 1u << (lbl & 31));
+  });
+  __syncthreads();
+  int lw = 0;  // 2^lw words per thread
+  while ((1024 << lw) < nwords) ++lw;
+  uint32_t n = 0;
+  for (int i = tid << lw; i < min((tid + 1) << lw, nwords); ++i) n += __popc(s_bits[i]);
+  uint32_t x = n;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) s_warp[w] = x;
+  __syncthreads();
+  uint32_t before = 0;
+  for (int i = 0; i < w; ++i) before += s_warp[i];
+  s_base[tid] = before + x - n;
+  __syncthreads();
+  components([&](uint32_t c) {
+    const uint32_t r = __ldg(a.cparent + c);
+    const int32_t lbl = __ldg(a.cminli + r);
+    const int wi = lbl >> 5, t = wi >> lw;
+    uint32_t f = s_base[t] + __popc(s_bits[wi] & ((1u << (lbl & 31)) - 1u));
+    for (int i = t << lw; i < wi; ++i) f += __popc(s_bits[i]);
+    cfid[c] = (int32_t)f;
+    if (r == c) flabel[f] = lbl;
+  });
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1772,8 +1834,7 @@ static void launch_feat_points(const SegArgs& a, const FeatAcc& acc, const int32
   }
 }
 
-int seg_mark_roots(msf_ctx* ctx, uint32_t* rootbits, unsigned long long* counter) {
-  (void)counter;
+int seg_mark_roots(msf_ctx* ctx, uint32_t* rootbits) {
   const SegState& L = ctx->last;
   SegArgs a;
   MSF_TRY(seg_args(ctx, L.g, L.crit.edges & MSF_EDGE_SPATIAL, &a));
@@ -1783,7 +1844,24 @@ int seg_mark_roots(msf_ctx* ctx, uint32_t* rootbits, unsigned long long* counter
   return MSF_OK;
 }
 
-int seg_feature_stats(msf_ctx* ctx, const RankArrays& rk, const FeatAcc& acc) {
+int seg_feature_ranks(msf_ctx* ctx, int64_t nwords, const FeatAcc& acc, int32_t* flabel) {
+  SegState& L = ctx->last;
+  SegArgs a;
+  MSF_TRY(seg_args(ctx, L.g, L.crit.edges & MSF_EDGE_SPATIAL, &a));
+  MSF_TRY(L.cfid.ensure(sizeof(int32_t) * (size_t)L.g.ntiles * L.g.cmax));
+  static std::atomic<uint64_t> attr_set{0};
+  ensure_smem_attr(k_feat_ranks, sizeof(uint32_t) * kRankWords, attr_set);
+  const int64_t init = (acc.F * acc.K + 1023) / 1024;
+  ScopedKernel k(ctx, "k_feat_ranks");
+  k_feat_ranks<<<(unsigned)(1 + std::min<int64_t>(init, ctx->sm_count)), 1024,
+                 sizeof(uint32_t) * nwords, ctx->stream>>>(a, acc, L.cfid.as<int32_t>(), flabel,
+                                                           (int)nwords);
+  MSF_CUDA_TRY(cudaGetLastError());
+  return MSF_OK;
+}
+
+int seg_feature_stats(msf_ctx* ctx, const RankArrays& rk, const FeatAcc& acc, int32_t* flabel,
+                      bool ranked) {
   SegState& L = ctx->last;
   const Geometry& g = L.g;
   const bool spatial = L.crit.edges & MSF_EDGE_SPATIAL;
@@ -1796,9 +1874,9 @@ int seg_feature_stats(msf_ctx* ctx, const RankArrays& rk, const FeatAcc& acc) {
   int32_t* cfid = L.cfid.as<int32_t>();
   cudaStream_t s = ctx->stream;
   const Dataset& d = ctx->ds;
-  {
+  if (!ranked) {
     ScopedKernel k(ctx, "k_comp_fid");
-    k_comp_fid<<<g.ntiles, 256, 0, s>>>(a, rk, cfid);
+    k_comp_fid<<<g.ntiles, 256, 0, s>>>(a, rk, cfid, flabel);
   }
   // voxel and point statistics only add into the accumulators: the point pass runs beside the
   // voxel pass on the auxiliary stream

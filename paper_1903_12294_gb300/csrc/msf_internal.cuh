@@ -783,6 +783,30 @@ struct VoxTable {
 // Point samples (one per lane in `ok`): lanes of the same feature reduce their exact
 // fixed-point attribute values and double-float squares; the group's first lane commits.
 // Every lane of the warp must call this.
+// empty accumulators i, i + stride, ..
+__device__ __forceinline__ void acc_init(const FeatAcc& c, int64_t i0, int64_t stride) {
+  const int64_t n = c.F * c.K;
+  const unsigned kmin0 = float_key(INFINITY), kmax0 = float_key(-INFINITY);
+  for (int64_t i = i0; i < n; i += stride) {
+    c.n_vox[i] = 0;
+    c.n_pts[i] = 0;
+    c.sf[i] = 0.0;
+    c.sf2[i] = 0.0;
+    c.fmin[i] = kmin0;
+    c.fmax[i] = kmax0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      c.bbmin[i * 4 + j] = 0x7FFFFFFF;
+      c.bbmax[i * 4 + j] = -1;
+      c.sc[i * 4 + j] = 0;
+    }
+    for (int k = 0; k < c.A; ++k) {
+      c.sq[i * c.A + k] = 0;
+      c.sa2[i * c.A + k] = 0.0;
+    }
+  }
+}
+
 // 2^x as fp32 for -126 <= x <= 127, built from the bits.
 __device__ __forceinline__ float pow2f(int x) { return __uint_as_float((uint32_t)(x + 127) << 23); }
 
@@ -1041,8 +1065,14 @@ int segment_field_fixed(const Geometry& g, int npred, const DevPred& pred, uint3
 
 // fast feature path (k_segment.cu): marks the feature labels of the retained segmentation in
 // rootbits and counts them; then, after the ranks exist, reduces voxel and point statistics.
-int seg_mark_roots(msf_ctx* ctx, uint32_t* rootbits, unsigned long long* counter);
-int seg_feature_stats(msf_ctx* ctx, const RankArrays& rk, const FeatAcc& acc);
+// With both, flabel [F] receives the features' labels. Windows of up to kRankWords words of bits
+// (32 voxel-timesteps each) take seg_feature_ranks instead of the bits, ranks and the empty
+// accumulators' own launches; seg_feature_stats then has its features' ranks (ranked).
+constexpr int64_t kRankWords = 49152;
+int seg_mark_roots(msf_ctx* ctx, uint32_t* rootbits);
+int seg_feature_ranks(msf_ctx* ctx, int64_t nwords, const FeatAcc& acc, int32_t* flabel);
+int seg_feature_stats(msf_ctx* ctx, const RankArrays& rk, const FeatAcc& acc, int32_t* flabel,
+                      bool ranked);
 bool seg_state_matches(const msf_ctx* ctx, const msf_criteria* crit, const void* labels);
 int validate_criteria(const msf_ctx* ctx, const msf_criteria* c);
 int make_geometry(const msf_ctx* ctx, const msf_criteria* c, Geometry* g);
