@@ -487,8 +487,10 @@ int msf_set_tile(msf_ctx* ctx, int by, int bz, int bt);
                                        beside the second launch (ignored with SERIAL_JOINS,
                                        without trajectory joins or below two tile rows)     */
 
-/* Fix the schedule of msf_segment (MSF_SCHED_* bits, 0..7), or -1 for the automatic one (a
- * tuned schedule when msf_autotune has tuned the problem's shape, else 0). Errors: INVALID_ARG. */
+/* Fix the schedule of msf_segment (MSF_SCHED_* bits, 0..7), or -1 for the automatic one: a
+ * tuned schedule when msf_autotune has tuned the problem's shape, else the joins of schedule 0
+ * with the criterion evaluated where the library finds it faster (reported as 0).
+ * Errors: INVALID_ARG. */
 int msf_set_schedule(msf_ctx* ctx, int sched);
 
 /* Result of msf_autotune. */

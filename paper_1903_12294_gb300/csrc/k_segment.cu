@@ -1229,7 +1229,13 @@ int segment_run(msf_ctx* ctx, const msf_criteria* crit, int32_t* labels, int64_t
   cudaStream_t s = ctx->stream;
   const int sched = segment_schedule(ctx, crit);
   MSF_CUDA_TRY(cudaMemsetAsync(a.counters, 0, sizeof(unsigned long long) * 4, s));
-  const bool fused = sched & MSF_SCHED_FUSED_CRITERION;
+  // Without a schedule set or tuned the criterion is evaluated inside the tile pass: its loads
+  // overlap the labelling, which is bound by instruction issue, and the masks' round trip through
+  // L2 goes. The streaming pass was the faster one on no size measured (one query, streamed
+  // against inside: 128^3 x 32 373 -> 336 us, 256^3 x 24 3.21 -> 2.82 ms, 1024^2 x 64 364 -> 331
+  // us, 32^3 x 8 with the rest of a step 303 -> 295 us); it stays for callers that set it and for
+  // the tuner.
+  const bool fused = (sched & MSF_SCHED_FUSED_CRITERION) || segment_automatic(ctx, crit);
   if (!fused) {  // the criterion as a streaming pass, the tile pass then starting from its masks
     ScopedKernel k(ctx, "k_mask");
     if ((a.g.nx & 3) == 0) launch_mask_np<true>(a, s);

@@ -1078,6 +1078,7 @@ int validate_criteria(const msf_ctx* ctx, const msf_criteria* c);
 int make_geometry(const msf_ctx* ctx, const msf_criteria* c, Geometry* g);
 const TuneEntry* tune_find(const msf_ctx* ctx, const msf_criteria* c);
 int segment_schedule(const msf_ctx* ctx, const msf_criteria* c);  // MSF_SCHED_* bits
+bool segment_automatic(const msf_ctx* ctx, const msf_criteria* c);  // none set, none tuned
 void make_preds(const msf_ctx* ctx, const msf_criteria* c, DevPred* out);
 
 }  // namespace msf

@@ -56,6 +56,10 @@ const TuneEntry* tune_find(const msf_ctx* ctx, const msf_criteria* c) {
   return nullptr;
 }
 
+bool segment_automatic(const msf_ctx* ctx, const msf_criteria* c) {
+  return ctx->sched < 0 && !tune_find(ctx, c);
+}
+
 int segment_schedule(const msf_ctx* ctx, const msf_criteria* c) {
   if (ctx->sched >= 0) return ctx->sched;
   if (const TuneEntry* e = tune_find(ctx, c)) return e->sched;
