@@ -21,9 +21,10 @@
 // Point samples may come on a finer time grid than the field (point step j falls in field step
 // fstep[j]); the records of all point steps of a field step go to that step's buckets.
 //   k_bin_reduce   one CTA per (bucket, field step): its records arrive by bulk copy while the
-//                  counters are cleared; a counting sort by voxel in shared memory; counts with
-//                  NaN means stored for every voxel, then the sums and means of the non-empty
-//                  voxels (one lane each) stored over them
+//                  counters are cleared and go to registers; counts by shared-memory atomics; the
+//                  means form in shared memory, one thread per record, and every voxel's count
+//                  and means are stored once; the voxel pairs of the records in their order, for
+//                  the trajectory joins
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -62,7 +63,7 @@ struct BinArgs {
   uint32_t* cursor;             // [T][nb] next free slot, from offs, one per kCurStride words
   uint2* rec_vn;                // [P*Tp] the sample's voxel, and the same point's voxel at the
                                 // next point step (-1 at the last or outside the grid)
-  float* rec_a;                 // [P*Tp][rec_aw(A)] attribute values (+4 slack)
+  uint32_t* rec;                // [P*Tp][rec_words(A)] attribute values and the same voxel pair
   unsigned* err;                // bounded waits that gave up
   uint32_t* ovf;                // items (t * nb + bucket) left to the wide reduce
   uint32_t* novf;               // their number
@@ -195,19 +196,23 @@ __global__ void __launch_bounds__(256) k_bin_keys(const __grid_constant__ BinArg
 // ---------------------------------------------------------------------------------------------
 // pass 2: records in bucket order (and the attribute maxima)
 // ---------------------------------------------------------------------------------------------
-// A record is the sample's voxel with the same point's voxel at the next point step (rec_vn, 8
-// bytes: what a trajectory link joins) and its attributes (rec_a, A values padded to 1, 2, 4 or
-// 8 words so that one vector store writes them). The block reads its samples in order
-// (coalesced keys and attributes, several per thread in flight) and sends each to the next free
-// slot of its bucket, taken from one global cursor per (field step, bucket). Records thus fill
+// A record is the sample's attributes, its voxel and the same point's voxel at the next point step
+// (what a trajectory link joins), in one, two or three 16-byte units so that it is written by one
+// store (of 16 or 32 bytes; three for seven or eight attributes). The block reads its samples in
+// order (coalesced keys and attributes, several per thread in flight) and sends each to the next
+// free slot of its bucket, taken from one global cursor per (field step, bucket). The pass is
+// bound by its scattered requests to L2, half of which cross to the other die: a slot atomic and
+// a store per sample (voxel pair and attributes stored apart, 8M particles x 24 steps, A = 4: 4.59
+// ms; together 2.80 ms, although a record then has 32 bytes instead of 24). Records thus fill
 // every bucket's range front to back in the order they arrive from all blocks, so a partly
 // written sector is completed within microseconds while it is still in L2 (per-block slot
 // ranges would leave one partial sector per block and bucket open for a block's whole life and
-// push them out to DRAM half-written). The order within a bucket changes nothing downstream:
-// counts and fixed-point sums are exact.
-__host__ __device__ constexpr int rec_aw(int A) {
-  return A <= 0 ? 0 : A == 1 ? 1 : A == 2 ? 2 : A <= 4 ? 4 : 8;
-}
+// push them out to DRAM half-written: ranks from the keys pass instead of the slot atomics took
+// 7.6 ms). The order within a bucket changes nothing downstream: counts and fixed-point sums are
+// exact.
+__host__ __device__ constexpr int rec_words(int A) { return A <= 2 ? 4 : A <= 6 ? 8 : 12; }
+// first word of the voxel pair (the attributes come first)
+__host__ __device__ constexpr int rec_pair(int A) { return A <= 2 ? 2 : A <= 4 ? 4 : A <= 6 ? 6 : 8; }
 
 constexpr int kPlaceNT = 512;                  // threads per block of the place pass
 constexpr int kPlacePer = 4;                   // samples per thread in flight
@@ -217,29 +222,28 @@ constexpr int kCurStride = 32;                 // words between two buckets' cur
                                                // 128-byte line, so that the slot atomics of
                                                // neighbouring buckets do not queue on one line
 
-template <int A>
-__device__ __forceinline__ float attr_or_zero(const float (&av)[A > 0 ? A : 1], int a) {
-  return a < A ? av[a < A ? a : 0] : 0.f;
+__device__ __forceinline__ void store32(uint32_t* p, const uint32_t (&w)[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(w[0]),
+               "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+               : "memory");
 }
 
 template <int A>
 __device__ __forceinline__ void put_record(const BinArgs& b, uint32_t slot, int32_t k, int32_t kn,
                                            const float (&av)[A > 0 ? A : 1]) {
-  constexpr int AW = rec_aw(A);
-  b.rec_vn[slot] = make_uint2((uint32_t)k, (uint32_t)kn);
-  float* dst = b.rec_a + (size_t)slot * AW;
-  if constexpr (AW == 1) {
-    dst[0] = av[0];
-  } else if constexpr (AW == 2) {
-    *reinterpret_cast<float2*>(dst) = make_float2(av[0], attr_or_zero<A>(av, 1));
-  } else if constexpr (AW == 4) {
-    *reinterpret_cast<float4*>(dst) = make_float4(av[0], attr_or_zero<A>(av, 1),
-                                                  attr_or_zero<A>(av, 2), attr_or_zero<A>(av, 3));
-  } else if constexpr (AW == 8) {
-    *reinterpret_cast<float4*>(dst) = make_float4(av[0], attr_or_zero<A>(av, 1),
-                                                  attr_or_zero<A>(av, 2), attr_or_zero<A>(av, 3));
-    *reinterpret_cast<float4*>(dst + 4) = make_float4(attr_or_zero<A>(av, 4), attr_or_zero<A>(av, 5),
-                                                      attr_or_zero<A>(av, 6), attr_or_zero<A>(av, 7));
+  constexpr int RW = rec_words(A), VO = rec_pair(A);
+  uint32_t w[RW];
+#pragma unroll
+  for (int i = 0; i < RW; ++i) w[i] = i < A ? __float_as_uint(av[i < A ? i : 0]) : 0u;
+  w[VO] = (uint32_t)k;
+  w[VO + 1] = (uint32_t)kn;
+  uint32_t* dst = b.rec + (size_t)slot * RW;
+  if constexpr (RW == 8) {
+    store32(dst, w);
+  } else {
+#pragma unroll
+    for (int i = 0; i < RW; i += 4)
+      *reinterpret_cast<uint4*>(dst + i) = make_uint4(w[i], w[i + 1], w[i + 2], w[i + 3]);
   }
 }
 
@@ -340,14 +344,13 @@ __global__ void __launch_bounds__(kPlaceNT) k_bin_place(const __grid_constant__ 
 // ---------------------------------------------------------------------------------------------
 // pass 3: per (bucket, timestep) counts, sums, means
 // ---------------------------------------------------------------------------------------------
-// Bulk copies of records [a0, a0 + n) (a0 and n multiples of 4) into a staging area.
+// Bulk copy of records [a0, a0 + n) into a staging area (a record is whole 16-byte units).
 template <int A>
 __device__ __forceinline__ void reduce_issue(const BinArgs& b, uint32_t a0, uint32_t n,
-                                             uint2* s_stv, float* s_sta, uint64_t* bar) {
-  constexpr int AW = rec_aw(A);
-  mbar_expect_tx(bar, 4u * n * (2 + AW));
-  bulk_g2s(s_stv, b.rec_vn + a0, 8u * n, bar);
-  if (AW) bulk_g2s(s_sta, b.rec_a + (size_t)a0 * AW, 4u * n * AW, bar);
+                                             uint32_t* s_st, uint64_t* bar) {
+  constexpr int RW = rec_words(A);
+  mbar_expect_tx(bar, 4u * n * RW);
+  bulk_g2s(s_st, b.rec + (size_t)a0 * RW, 4u * n * RW, bar);
 }
 
 // record range [r0, r1) of the item (field step t, bucket): the slots of its point steps
@@ -369,122 +372,114 @@ __device__ __forceinline__ void item_scale(const BinArgs& b, int a, int* s_k, fl
   s_f2[a] = pow2f(-(k - k / 2));
 }
 
-// The staged attribute values of record q, as AW words.
+// The staged record q: attribute values and the voxel pair.
 template <int A>
-__device__ __forceinline__ void staged_attrs(const float* s_sta, int q, float (&v)[A > 0 ? A : 1]) {
-  constexpr int AW = rec_aw(A);
-  if constexpr (AW == 1) {
-    v[0] = s_sta[q];
-  } else if constexpr (AW == 2) {
-    const float2 x = reinterpret_cast<const float2*>(s_sta)[q];
-    v[0] = x.x;
-    if (A > 1) v[A > 1 ? 1 : 0] = x.y;
-  } else if constexpr (AW == 4) {
-    const float4 x = reinterpret_cast<const float4*>(s_sta)[q];
-    const float w[4] = {x.x, x.y, x.z, x.w};
+__device__ __forceinline__ uint2 staged_record(const uint32_t* s_st, int q,
+                                               float (&v)[A > 0 ? A : 1]) {
+  constexpr int RW = rec_words(A), VO = rec_pair(A);
+  uint32_t w[RW];
 #pragma unroll
-    for (int a = 0; a < A; ++a) v[a] = w[a];
-  } else if constexpr (AW == 8) {
-    const float4 x = reinterpret_cast<const float4*>(s_sta)[2 * q];
-    const float4 y = reinterpret_cast<const float4*>(s_sta)[2 * q + 1];
-    const float w[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
-#pragma unroll
-    for (int a = 0; a < A; ++a) v[a] = w[a];
+  for (int i = 0; i < RW; i += 4) {
+    const uint4 x = reinterpret_cast<const uint4*>(s_st)[(q * RW + i) / 4];
+    w[i] = x.x, w[i + 1] = x.y, w[i + 2] = x.z, w[i + 3] = x.w;
   }
+#pragma unroll
+  for (int a = 0; a < A; ++a) v[a] = __uint_as_float(w[a]);
+  return make_uint2(w[VO], w[VO + 1]);
 }
 
-// Count, NaN mean (and zero sum) of four consecutive voxels v.. of field step t; the tail of a
-// grid whose voxel count is not a multiple of four takes scalar stores.
-template <int A, bool KEEP>
-__device__ __forceinline__ void store_empty4(const BinArgs& b, int t, int64_t v, int nleft,
-                                             uint4 c4) {
-  const float qnan = __int_as_float(0x7fc00000);
-  if ((b.V & 3) == 0) {  // v is then a multiple of four and all four exist
-    __stcs(reinterpret_cast<uint4*>(b.count + (int64_t)t * b.V + v), c4);
-#pragma unroll
-    for (int a = 0; a < A; ++a) {
-      const int64_t o = ((int64_t)a * b.T + t) * b.V + v;
-      __stcs(reinterpret_cast<float4*>(b.mean + o), make_float4(qnan, qnan, qnan, qnan));
-      if (KEEP) {
-        __stcs(reinterpret_cast<longlong2*>(b.sumq + o), make_longlong2(0, 0));
-        __stcs(reinterpret_cast<longlong2*>(b.sumq + o + 2), make_longlong2(0, 0));
-      }
-    }
-  } else {
-    const uint32_t cc[4] = {c4.x, c4.y, c4.z, c4.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      if (e >= nleft) break;
-      __stcs(b.count + (int64_t)t * b.V + v + e, (int)cc[e]);
-#pragma unroll
-      for (int a = 0; a < A; ++a) {
-        const int64_t o = ((int64_t)a * b.T + t) * b.V + v + e;
-        __stcs(b.mean + o, qnan);
-        if (KEEP) __stcs(b.sumq + o, 0ll);
-      }
-    }
-  }
+// One block per item (field step t, bucket): the bucket's records (at most red_stage(A) of them,
+// a few per thread) arrive by bulk copy while the voxel counters are cleared and go to registers,
+// their attributes quantised; the staging area then becomes the bucket's means. A record's
+// shared-memory atomic on its voxel's counter (two 16-bit counters per word) counts the voxel's
+// records and gives the record its place among them. What a voxel needs depends on its count:
+//   1   the record's thread forms the mean: (float)sum / 1 is the quantised value itself;
+//   2   the second record leaves its quantised values in the voxel's mean, the first adds its
+//       own: both are exact in fp32, so one fp32 addition rounds their exact sum once, as
+//       converting the int64 sum does;
+//   3+  exact int64 sums in a compact list of such voxels (two 32-bit atomics with the carry),
+//       then the fp32 mean chain, one thread per voxel.
+// Then the block streams counts and means out, four voxels per thread with 16-byte stores, NaN
+// where there are no records (storing NaN everywhere and the means over it, one 4-byte store per
+// non-empty voxel and attribute, issued twice the stores; sorting the records by voxel first and
+// quantising in the divergent parts made it 16,000 instructions a bucket). 8M records x 24 steps,
+// 256^3 voxels, A = 4: 4.17 ms before, 3.47 ms now. A bucket with more records than the staging
+// area holds is listed for k_bin_reduce_wide and left to it.
+__host__ __device__ constexpr int red_stage(int A) { return A <= 6 ? 2048 : 1536; }
+
+// The quantised value of v as fp32, q = round_half_even(v * 2^k): exact (a 24-bit mantissa shifted
+// left, or an integer below 2^24), so it is formed in fp32: v * 2^k is exact (two power-of-two
+// factors u1, u2; a product too small for a normal fp32 is below one half either way), rounding
+// it to an integer (half to even) is the quantisation, and adding +0 turns a negative zero into
+// the positive zero the integer path gives. Non-finite v gives 0.
+__device__ __forceinline__ float quantised(float v, float u1, float u2) {
+  return isfinite(v) ? __fadd_rn(rintf(__fmul_rn(__fmul_rn(v, u1), u2)), 0.0f) : 0.0f;
 }
 
-// One block per item (field step t, bucket): the bucket's records (at most kRedStage of them)
-// arrive by bulk copy while the voxel counters are cleared; the block counts the records per
-// voxel (32-bit shared atomics), turns the counts into each voxel's range by a block scan, and
-// sorts the records into those ranges (an index permutation). The scan's pass, four voxels per
-// thread, also stores every voxel's count with a NaN mean (16-byte stores) and lists the
-// non-empty voxels block-wide, those with one record apart from the others; the block's threads
-// then take the listed voxels one each, so that means and fixed-point sums are formed only where
-// there are samples, with all lanes busy, and stored over the NaN (ordered after it by the block
-// barrier). A bucket with more records than the staging area holds is listed for
-// k_bin_reduce_wide and left to it.
-constexpr int kRedStage = 2048;  // records staged per bucket (plus alignment slack)
+// an integer held in fp32, as int64 (integer operations: the hardware conversion issues on the
+// narrow fp64 pipe)
+__device__ __forceinline__ long long exact_ll(float q) {
+  const uint32_t b = __float_as_uint(q);
+  const int e = (int)((b >> 23) & 0xFFu) - 150;
+  if (e < -23) return 0;  // zero
+  const long long m = (long long)((b & 0x7FFFFFu) | 0x800000u);
+  const long long u = e >= 0 ? m << e : m >> -e;
+  return (b >> 31) ? -u : u;
+}
 
 template <int A, bool KEEP>
 __global__ void __launch_bounds__(kBinNT, A <= 4 ? 3 : 2) k_bin_reduce(const __grid_constant__ BinArgs b) {
-  constexpr int AW = rec_aw(A);
-  constexpr int SS = kRedStage + 8;                                      // staged records
+  constexpr int A1 = A > 0 ? A : 1;
+  constexpr int SS = red_stage(A), PER = SS / kBinNT, MANY = SS / 3;
   extern __shared__ __align__(16) uint32_t s_red[];
   const int R = 1 << b.logR;
-  float* s_sta = reinterpret_cast<float*>(s_red);                       // [SS][AW] values
-  uint2* s_stv = reinterpret_cast<uint2*>(s_red + SS * AW);              // [SS] voxel pairs
-  uint32_t* s_pos = s_red + SS * (AW + 2);                               // [R] counts, then ends
-  uint16_t* s_idx = reinterpret_cast<uint16_t*>(s_pos + R);              // [SS] sorted records
-  uint16_t* s_list1 = s_idx + SS;                                        // [R] one-record voxels
-  uint16_t* s_list2 = s_list1 + R;                                       // [R] the others
+  uint32_t* s_cnt = s_red;                              // [R] 16-bit counters, two per word
+  uint32_t* s_area = s_red + R / 2;                     // staged records, then
+  float* s_mean = reinterpret_cast<float*>(s_area);     // [A][R] and
+  uint32_t* s_sum = s_area + A * R;                     // [MANY][A] low, high
   __shared__ __align__(8) uint64_t s_bar;
-  __shared__ int2 s_warp2[kBinNT / 32];
-  __shared__ int s_k[A > 0 ? A : 1];
-  __shared__ float s_f1[A > 0 ? A : 1], s_f2[A > 0 ? A : 1];
+  __shared__ uint16_t s_many[MANY];
+  __shared__ int s_nmany;
+  __shared__ float4 s_sc[A1];  // 2^k as two factors, 2^-k as two factors
   const int bucket = blockIdx.x, t = blockIdx.y;  // t: the field step
   uint32_t r0, r1;
   item_range(b, t, bucket, r0, r1);
-  if (r1 - r0 > (uint32_t)kRedStage) {  // too many records to stage: the wide pass takes it
+  if (r1 - r0 > (uint32_t)SS) {  // too many records to stage: the wide pass takes it
     if (threadIdx.x == 0) b.ovf[atomicAdd(b.novf, 1u)] = (uint32_t)t * (uint32_t)b.nb + bucket;
     return;
   }
-  const uint32_t s0 = r0 & ~3u, e1 = (r1 + 3u) & ~3u;
-  const bool any = r1 > r0;
+  const int n = (int)(r1 - r0);
   if (threadIdx.x == 0) {
     mbar_init(&s_bar, 1);
-    if (any) reduce_issue<A>(b, s0, e1 - s0, s_stv, s_sta, &s_bar);
+    if (n) reduce_issue<A>(b, r0, (uint32_t)n, s_area, &s_bar);
     // the records of the item one wave of blocks later, into L2 (its block then copies from
     // there instead of from DRAM)
     const int64_t nxt = (int64_t)t * b.nb + bucket + b.pf_ahead;
     if (nxt < (int64_t)b.T * b.nb) {
       uint32_t q0, q1;
       item_range(b, (int)(nxt / b.nb), (int)(nxt % b.nb), q0, q1);
-      if (q1 > q0 && q1 - q0 <= (uint32_t)kRedStage) {
-        const uint32_t p0 = q0 & ~3u, p1 = (q1 + 3u) & ~3u;
-        prefetch_l2(b.rec_vn + p0, 8u * (p1 - p0));
-        if (rec_aw(A)) prefetch_l2(b.rec_a + (size_t)p0 * rec_aw(A), 4u * rec_aw(A) * (p1 - p0));
-      }
+      if (q1 > q0 && q1 - q0 <= (uint32_t)SS)
+        prefetch_l2(b.rec + (size_t)q0 * rec_words(A), 4u * rec_words(A) * (q1 - q0));
     }
+    s_nmany = 0;
   }
-  if ((int)threadIdx.x < A) item_scale(b, threadIdx.x, s_k, s_f1, s_f2);
-  for (int q = threadIdx.x; q < R / 4; q += kBinNT)
-    reinterpret_cast<uint4*>(s_pos)[q] = make_uint4(0u, 0u, 0u, 0u);
+  if ((int)threadIdx.x < A) {
+    const int k = scale_exponent_bits(b.absmax[threadIdx.x], (long long)b.scale_n);
+    s_sc[threadIdx.x] = make_float4(pow2f(k / 2), pow2f(k - k / 2), pow2f(-(k / 2)),
+                                    pow2f(-(k - k / 2)));
+  }
+  for (int q = threadIdx.x; q < R / 8; q += kBinNT)
+    reinterpret_cast<uint4*>(s_cnt)[q] = make_uint4(0u, 0u, 0u, 0u);
+  const int64_t vbase = (int64_t)bucket << b.logR;
+  const int nv = (int)min((int64_t)R, b.V - vbase);
+  auto keep = [&](int a, int v, long long sum) {  // the int64 sum of a non-empty voxel
+    if (KEEP) b.sumq[((int64_t)a * b.T + t) * b.V + vbase + v] = sum;
+  };
+  if (KEEP)  // zero sums; those of the non-empty voxels are stored over them behind a barrier
+    for (int a = 0; a < A; ++a)
+      for (int q = threadIdx.x; q < nv; q += kBinNT) keep(a, q, 0ll);
   __syncthreads();
-  const int m = (int)(e1 - s0);
-  if (any) {
+  if (n) {
     const bool ok = mbar_wait(&s_bar, 0, b.wait_cycles);
     if (__syncthreads_or(!ok)) {  // the copy did not arrive in time
       if (threadIdx.x == 0) {
@@ -493,154 +488,132 @@ __global__ void __launch_bounds__(kBinNT, A <= 4 ? 3 : 2) k_bin_reduce(const __g
       }
       return;
     }
-    for (int q = threadIdx.x; q < m; q += kBinNT) {
-      const uint32_t r = s0 + (uint32_t)q;
-      if (r < r0 || r >= r1) continue;  // alignment slack of the neighbouring buckets
-      atomicAdd(s_pos + (s_stv[q].x & (uint32_t)(R - 1)), 1u);
+    int v[PER], place[PER];
+    float x[PER][A1];  // quantised attributes
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int q = (int)threadIdx.x + kBinNT * i;
+      v[i] = -1;
+      place[i] = 0;
+      if (q < n) {
+        const uint2 vn = staged_record<A>(s_area, q, x[i]);
+        __stcs(b.rec_vn + r0 + q, vn);
+        v[i] = (int)(vn.x & (uint32_t)(R - 1));
+        const int sh = (v[i] & 1) << 4;
+        place[i] = (int)((atomicAdd(s_cnt + (v[i] >> 1), 1u << sh) >> sh) & 0xFFFFu);
+#pragma unroll
+        for (int a = 0; a < A; ++a) {
+          const float2 up = *reinterpret_cast<const float2*>(&s_sc[a]);
+          x[i][a] = quantised(x[i][a], up.x, up.y);
+        }
+      }
+    }
+    __syncthreads();  // the counts are complete, the staging area is read
+    if constexpr (A > 0) {
+      auto mean_of = [&](int a, float m) { return __fmul_rn(__fmul_rn(m, s_sc[a].z), s_sc[a].w); };
+      int c[PER];
+#pragma unroll
+      for (int i = 0; i < PER; ++i) {
+        c[i] = 0;
+        if (v[i] < 0) continue;
+        c[i] = (int)((s_cnt[v[i] >> 1] >> ((v[i] & 1) << 4)) & 0xFFFFu);
+        if (c[i] <= 2 && place[i] == c[i] - 1) {
+#pragma unroll
+          for (int a = 0; a < A; ++a) {
+            s_mean[a * R + v[i]] = c[i] == 1 ? mean_of(a, x[i][a]) : x[i][a];
+            if (c[i] == 1) keep(a, v[i], exact_ll(x[i][a]));
+          }
+        } else if (c[i] > 2 && place[i] == 0) {
+          const int slot = atomicAdd(&s_nmany, 1);
+          s_many[slot] = (uint16_t)v[i];
+          s_mean[v[i]] = __int_as_float(slot);
+#pragma unroll
+          for (int a = 0; a < A; ++a)
+            *reinterpret_cast<uint2*>(s_sum + 2 * (slot * A + a)) = make_uint2(0u, 0u);
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < PER; ++i) {
+        if (c[i] == 2 && place[i] == 0) {
+#pragma unroll
+          for (int a = 0; a < A; ++a) {
+            const float q1 = s_mean[a * R + v[i]];
+            s_mean[a * R + v[i]] = mean_of(a, __fmul_rn(__fadd_rn(x[i][a], q1), 0.5f));
+            keep(a, v[i], exact_ll(x[i][a]) + exact_ll(q1));
+          }
+        } else if (c[i] > 2) {
+          const int slot = __float_as_int(s_mean[v[i]]);
+#pragma unroll
+          for (int a = 0; a < A; ++a) {
+            const unsigned long long q = (unsigned long long)exact_ll(x[i][a]);
+            uint32_t* p = s_sum + 2 * (slot * A + a);
+            const uint32_t lo = (uint32_t)q, old = atomicAdd(p, lo);
+            atomicAdd(p + 1, (uint32_t)(q >> 32) + (old + lo < old ? 1u : 0u));
+          }
+        }
+      }
+      __syncthreads();
+      for (int i = threadIdx.x; i < s_nmany; i += kBinNT) {
+        const int u = s_many[i];
+        const int m = (int)((s_cnt[u >> 1] >> ((u & 1) << 4)) & 0xFFFFu);
+#pragma unroll
+        for (int a = 0; a < A; ++a) {
+          const uint2 w = *reinterpret_cast<const uint2*>(s_sum + 2 * (i * A + a));
+          const long long sum = (long long)(((unsigned long long)w.y << 32) | w.x);
+          s_mean[a * R + u] = mean_of(a, div_count(i64_to_f32_rn(sum), m));
+          keep(a, u, sum);
+        }
+      }
+      __syncthreads();
     }
   }
-  __syncthreads();
-  // One pass of four consecutive voxels per thread: the range starts (an exclusive block scan of
-  // the counts, in place), the voxels with one record and those with more listed block-wide
-  // (their places from the same scan), and every voxel's count stored with a NaN mean.
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t vbase = (int64_t)bucket << b.logR;
-  const int nv = (int)min((int64_t)R, b.V - vbase);
-  int carry = 0, carry1 = 0, carry2 = 0;
-  for (int base = 0; base < R; base += 4 * kBinNT) {
-    const int q = base + 4 * (int)threadIdx.x;
-    uint4 c4 = make_uint4(0u, 0u, 0u, 0u);
-    if (q < R) c4 = *reinterpret_cast<const uint4*>(s_pos + q);
-    const int tot = (int)(c4.x + c4.y + c4.z + c4.w);
-    const int n1 = (c4.x == 1u) + (c4.y == 1u) + (c4.z == 1u) + (c4.w == 1u);
-    const int n2 = (c4.x > 1u) + (c4.y > 1u) + (c4.z > 1u) + (c4.w > 1u);
-    int x = tot, y12 = n1 | (n2 << 16);
+  const float qnan = __int_as_float(0x7fc00000);
+  for (int q = 4 * (int)threadIdx.x; q < nv; q += 4 * kBinNT) {
+    const uint2 w = *reinterpret_cast<const uint2*>(s_cnt + q / 2);
+    const uint4 c4 = make_uint4(w.x & 0xFFFFu, w.x >> 16, w.y & 0xFFFFu, w.y >> 16);
+    const int64_t o = (int64_t)t * b.V + vbase + q;
+    if ((b.V & 3) == 0) {  // nv is then a multiple of four
+      __stcs(reinterpret_cast<uint4*>(b.count + o), c4);
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int u = __shfl_up_sync(0xFFFFFFFFu, x, o);
-      const int v = __shfl_up_sync(0xFFFFFFFFu, y12, o);
-      if (lane >= o) {
-        x += u;
-        y12 += v;
+      for (int a = 0; a < A; ++a) {
+        const float4 m4 = *reinterpret_cast<const float4*>(s_mean + a * R + q);
+        __stcs(reinterpret_cast<float4*>(b.mean + (int64_t)a * b.T * b.V + o),
+               make_float4(c4.x ? m4.x : qnan, c4.y ? m4.y : qnan, c4.z ? m4.z : qnan,
+                           c4.w ? m4.w : qnan));
       }
-    }
-    if (lane == 31) s_warp2[w] = make_int2(x, y12);
-    __syncthreads();
-    // the warps' totals, scanned by every warp (16 lanes)
-    int2 wt = lane < kBinNT / 32 ? s_warp2[lane] : make_int2(0, 0);
-#pragma unroll
-    for (int o = 1; o < kBinNT / 32; o <<= 1) {
-      const int u = __shfl_up_sync(0xFFFFFFFFu, wt.x, o);
-      const int v = __shfl_up_sync(0xFFFFFFFFu, wt.y, o);
-      if (lane >= o) {
-        wt.x += u;
-        wt.y += v;
-      }
-    }
-    const int all = __shfl_sync(0xFFFFFFFFu, wt.x, kBinNT / 32 - 1);
-    const int all12 = __shfl_sync(0xFFFFFFFFu, wt.y, kBinNT / 32 - 1);
-    const int wx = w ? __shfl_sync(0xFFFFFFFFu, wt.x, w - 1) : 0;
-    const int wy = w ? __shfl_sync(0xFFFFFFFFu, wt.y, w - 1) : 0;
-    const int run = carry + x - tot + wx;
-    const int e12 = y12 - (n1 | (n2 << 16)) + wy;  // exclusive, both fields
-    int p1 = carry1 + (e12 & 0xFFFF), p2 = carry2 + (e12 >> 16);
-    if (q < R) {
-      *reinterpret_cast<uint4*>(s_pos + q) =
-          make_uint4((uint32_t)run, (uint32_t)run + c4.x, (uint32_t)run + c4.x + c4.y,
-                     (uint32_t)run + c4.x + c4.y + c4.z);
+    } else {
       const uint32_t cc[4] = {c4.x, c4.y, c4.z, c4.w};
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        if (cc[e] == 1u) s_list1[p1++] = (uint16_t)(q + e);
-        else if (cc[e] > 1u) s_list2[p2++] = (uint16_t)(q + e);
-      }
-      if (q < nv) store_empty4<A, KEEP>(b, t, vbase + q, nv - q, c4);
-    }
-    carry += all;
-    carry1 += all12 & 0xFFFF;
-    carry2 += all12 >> 16;
-    __syncthreads();
-  }
-  const int N1 = carry1, N2 = carry2;
-  // sort: each record to the next place of its voxel's range (s_pos becomes the range ends, so
-  // voxel u's records sit at [u ? s_pos[u - 1] : 0, s_pos[u]))
-  if (any)
-    for (int q = threadIdx.x; q < m; q += kBinNT) {
-      const uint32_t r = s0 + (uint32_t)q;
-      if (r < r0 || r >= r1) continue;
-      const uint32_t pos = atomicAdd(s_pos + (s_stv[q].x & (uint32_t)(R - 1)), 1u);
-      s_idx[pos] = (uint16_t)q;
-    }
-  __syncthreads();  // the ranges, and the NaN stores before the means over them
-  if constexpr (A > 0) {
-    int kq[A];
+        if (q + e >= nv) break;
+        __stcs(b.count + o + e, (int)cc[e]);
 #pragma unroll
-    for (int a = 0; a < A; ++a) kq[a] = s_k[a];
-    // One record: its mean is its value quantised and scaled back. (float)sum / 1 of the
-    // general chain is the quantised value itself, which fp32 holds exactly (a 24-bit mantissa
-    // shifted left, or an integer below 2^24), so it is formed in fp32: v * 2^k is exact (two
-    // power-of-two factors; a product too small for a normal fp32 is below one half either
-    // way), rounding it to an integer (half to even) is the quantisation, and adding +0 turns
-    // a negative zero into the positive zero the integer path gives.
-    for (int i = threadIdx.x; i < N1; i += kBinNT) {
-      const int u = s_list1[i];
-      float vv[A];
-      staged_attrs<A>(s_sta, s_idx[s_pos[u] - 1u], vv);
-#pragma unroll
-      for (int a = 0; a < A; ++a) {
-        const int k = kq[a];
-        const int64_t o = ((int64_t)a * b.T + t) * b.V + vbase + u;
-        const float qv =
-            isfinite(vv[a])
-                ? __fadd_rn(rintf(__fmul_rn(__fmul_rn(vv[a], pow2f(k / 2)), pow2f(k - k / 2))), 0.0f)
-                : 0.0f;
-        __stcs(b.mean + o, __fmul_rn(__fmul_rn(qv, pow2f(-(k / 2))), pow2f(-(k - k / 2))));
-        if (KEEP) __stcs(b.sumq + o, quantise(vv[a], k));
-      }
-    }
-    // More records: exact fixed-point sums, then the fp32 mean chain.
-    for (int i = threadIdx.x; i < N2; i += kBinNT) {
-      const int u = s_list2[i];
-      const uint32_t e = s_pos[u], st = u ? s_pos[u - 1] : 0u;
-      long long sum[A];
-#pragma unroll
-      for (int a = 0; a < A; ++a) sum[a] = 0;
-      for (uint32_t y = st; y < e; ++y) {
-        float vv[A];
-        staged_attrs<A>(s_sta, s_idx[y], vv);
-#pragma unroll
-        for (int a = 0; a < A; ++a) sum[a] += quantise(vv[a], kq[a]);
-      }
-      const int c = (int)(e - st);
-#pragma unroll
-      for (int a = 0; a < A; ++a) {
-        const int k = kq[a];
-        const int64_t o = ((int64_t)a * b.T + t) * b.V + vbase + u;
-        __stcs(b.mean + o, __fmul_rn(__fmul_rn(div_count(i64_to_f32_rn(sum[a]), c),
-                                               pow2f(-(k / 2))), pow2f(-(k - k / 2))));
-        if (KEEP) __stcs(b.sumq + o, sum[a]);
+        for (int a = 0; a < A; ++a)
+          __stcs(b.mean + (int64_t)a * b.T * b.V + o + e, cc[e] ? s_mean[a * R + q + e] : qnan);
       }
     }
   }
 }
 
 // Buckets with more records than k_bin_reduce stages (listed by it): the records arrive in
-// pieces of R; counts and fixed-point sums accumulate in shared memory (sums [A][R] u64,
-// counts [R] u32, then the staging buffer of R records, reused for the means [A][R] f32 and the
-// non-empty lists once the records are in). After the records, every warp owns 128 voxels (four
+// pieces of wide_piece; counts and fixed-point sums accumulate in shared memory (sums [A][R] u64,
+// counts [R] u32, then the staging buffer, reused for the means [A][R] f32 and the non-empty
+// lists once the records are in). After the records, every warp owns 128 voxels (four
 // per lane): it lists its non-empty ones, forms their means and stores its outputs. Blocks take
 // listed items in turn.
+__host__ __device__ constexpr int wide_piece(int A) { return A <= 6 ? 2048 : 1024; }
+
 template <int A, bool KEEP>
 __global__ void __launch_bounds__(kBinNT, 1) k_bin_reduce_wide(const __grid_constant__ BinArgs b) {
-  constexpr int AW = rec_aw(A);
+  constexpr uint32_t PW = wide_piece(A);
   extern __shared__ __align__(16) unsigned long long s_dyn64[];
   const int R = 1 << b.logR;
   unsigned long long* s_sum = s_dyn64;                                    // [A][R]
   uint32_t* s_cnt = reinterpret_cast<uint32_t*>(s_dyn64 + (size_t)A * R);  // [R]
-  float* s_sta = reinterpret_cast<float*>(s_cnt + R);                     // [R][AW] values
-  uint2* s_stv = reinterpret_cast<uint2*>(s_sta + (size_t)AW * R);       // [R] voxel pairs
-  float* s_mean = s_sta;                                                  // after the records
-  uint32_t* s_list = reinterpret_cast<uint32_t*>(s_sta) + (size_t)A * R;
+  uint32_t* s_st = s_cnt + R;                                             // [PW] records
+  float* s_mean = reinterpret_cast<float*>(s_st);                         // after the records
+  uint32_t* s_list = s_st + (size_t)A * R;
   __shared__ __align__(8) uint64_t s_bar;
   __shared__ int s_k[A > 0 ? A : 1];
   __shared__ float s_f1[A > 0 ? A : 1], s_f2[A > 0 ? A : 1];
@@ -654,11 +627,10 @@ __global__ void __launch_bounds__(kBinNT, 1) k_bin_reduce_wide(const __grid_cons
   const int bucket = (int)(itm % (uint32_t)b.nb), t = (int)(itm / (uint32_t)b.nb);
   uint32_t r0, r1;
   item_range(b, t, bucket, r0, r1);
-  const uint32_t s0 = r0 & ~3u, e1 = (r1 + 3u) & ~3u;
-  const int npiece = r1 > r0 ? (int)((e1 - s0 + (uint32_t)R - 1) / (uint32_t)R) : 0;
+  const int npiece = (int)((r1 - r0 + PW - 1) / PW);
   if (threadIdx.x == 0 && npiece) {
     fence_proxy_async_smem();
-    reduce_issue<A>(b, s0, min((uint32_t)R, e1 - s0), s_stv, s_sta, &s_bar);
+    reduce_issue<A>(b, r0, min(PW, r1 - r0), s_st, &s_bar);
   }
   {
     uint4* z = reinterpret_cast<uint4*>(s_dyn64);
@@ -675,15 +647,14 @@ __global__ void __launch_bounds__(kBinNT, 1) k_bin_reduce_wide(const __grid_cons
       }
       return;
     }
-    const uint32_t a0 = s0 + (uint32_t)piece * (uint32_t)R;
-    const int m = (int)min((uint32_t)R, e1 - a0);
+    const uint32_t a0 = r0 + (uint32_t)piece * PW;
+    const int m = (int)min(PW, r1 - a0);
     for (int q = threadIdx.x; q < m; q += kBinNT) {
-      const uint32_t r = a0 + (uint32_t)q;
-      if (r < r0 || r >= r1) continue;  // alignment slack of the neighbouring buckets
-      const uint32_t v = s_stv[q].x & (uint32_t)(R - 1);  // voxel within the bucket
-      atomicAdd(s_cnt + v, 1u);
       float vv[A > 0 ? A : 1];
-      staged_attrs<A>(s_sta, q, vv);
+      const uint2 vn = staged_record<A>(s_st, q, vv);
+      __stcs(b.rec_vn + a0 + q, vn);
+      const uint32_t v = vn.x & (uint32_t)(R - 1);  // voxel within the bucket
+      atomicAdd(s_cnt + v, 1u);
 #pragma unroll
       for (int a = 0; a < A; ++a)
         atomicAdd(s_sum + (size_t)a * R + v, (unsigned long long)quantise(vv[a], s_k[a]));
@@ -691,8 +662,8 @@ __global__ void __launch_bounds__(kBinNT, 1) k_bin_reduce_wide(const __grid_cons
     __syncthreads();
     if (piece + 1 < npiece && threadIdx.x == 0) {
       fence_proxy_async_smem();  // the reads above before the next copy overwrites them
-      const uint32_t a1 = a0 + (uint32_t)R;
-      reduce_issue<A>(b, a1, min((uint32_t)R, e1 - a1), s_stv, s_sta, &s_bar);
+      const uint32_t a1 = a0 + PW;
+      reduce_issue<A>(b, a1, min(PW, r1 - a1), s_st, &s_bar);
     }
   }
   const float qnan = __int_as_float(0x7fc00000);
@@ -771,16 +742,18 @@ __global__ void __launch_bounds__(kBinNT, 1) k_bin_reduce_wide(const __grid_cons
   }  // items
 }
 
-// Bucket width: 2048 voxels (the sorted reduce stages records, not per-voxel sums, so the
-// width does not depend on the attribute count), wider when the grid has more buckets than the
-// shared-memory histograms hold and the wide pass's sums still fit.
+// Bucket width: 2048 voxels, wider when the grid has more buckets than the shared-memory
+// histograms hold and the wide pass's sums still fit.
 static size_t reduce_smem(int A, int logR) {
-  const size_t R = (size_t)1 << logR, SS = kRedStage + 8;
-  return 4 * SS * (2 + (size_t)rec_aw(A)) + 4 * R + 2 * SS + 4 * R;
+  const size_t R = (size_t)1 << logR, SS = red_stage(A);
+  const size_t staged = 4 * SS * rec_words(A);
+  const size_t means = 4 * R * A + 8 * (SS / 3) * A;  // and the int64 sums
+  return 2 * R + std::max(staged, means);
 }
 static size_t reduce_wide_smem(int A, int logR) {
   const size_t R = (size_t)1 << logR;
-  return R * (8 * (size_t)A + 4 + 4 * (2 + (size_t)rec_aw(A)));
+  const size_t staged = 4 * (size_t)wide_piece(A) * rec_words(A);
+  return R * (8 * (size_t)A + 4) + std::max(staged, 4 * R * A + 4 * R);
 }
 
 static int bucket_log2(int A, int64_t V) {
@@ -894,17 +867,15 @@ int bin_run(msf_ctx* ctx, unsigned flags) {
   const int64_t TB = (int64_t)d.T * b.nb;
   const int64_t NR = d.P * (int64_t)d.Tp;
   const int Af = d.A > 0 ? d.A : 1;
-  const int AW = rec_aw(d.A);
+  const int RW = rec_words(d.A);
   if (NR >= ((int64_t)1 << 32) || TB >= ((int64_t)1 << 31) ||
       (d.P + kPlaceChunk - 1) / kPlaceChunk > 0x7FFFFFFF)
     return MSF_ERR_TOO_LARGE;
   MSF_TRY(S.hist.ensure(sizeof(uint32_t) * TB));
   MSF_TRY(S.offs.ensure(sizeof(uint32_t) * (TB + d.T)));
   MSF_TRY(S.cursor.ensure(sizeof(uint32_t) * kCurStride * TB));
-  // records: voxels [NR] and attributes [NR][AW], with room for the rounded-up bulk copies
-  const int64_t NRp = (NR + 3) & ~(int64_t)3;
-  MSF_TRY(S.rec_vn.ensure(sizeof(uint2) * (NRp + 4)));
-  MSF_TRY(S.rec_a.ensure(sizeof(float) * ((NRp + 4) * (AW > 0 ? AW : 1))));
+  MSF_TRY(S.rec_vn.ensure(sizeof(uint2) * std::max<int64_t>(NR, 1)));
+  MSF_TRY(S.rec.ensure(sizeof(uint32_t) * RW * std::max<int64_t>(NR, 1)));
   MSF_TRY(S.absmax.ensure(sizeof(unsigned) * MSF_MAX_ATTR));
   MSF_TRY(S.outside.ensure(sizeof(unsigned long long) * d.Tp));
   MSF_TRY(S.total.ensure(sizeof(uint32_t) * 4));  // [2] error word, [3] wide items
@@ -920,7 +891,7 @@ int bin_run(msf_ctx* ctx, unsigned flags) {
   b.offs = S.offs.as<uint32_t>();
   b.cursor = S.cursor.as<uint32_t>();
   b.rec_vn = S.rec_vn.as<uint2>();
-  b.rec_a = S.rec_a.as<float>();
+  b.rec = S.rec.as<uint32_t>();
   b.wait_cycles = ctx->wait_cycles;
   b.pf_ahead = ctx->sm_count * (d.A <= 4 ? 3 : 2);  // resident reduce blocks
   b.err = S.total.as<uint32_t>() + 2;
@@ -988,7 +959,7 @@ int bin_run(msf_ctx* ctx, unsigned flags) {
   S.rec_valid = d.P > 0;
   S.rec_logR = b.logR;
   S.rec_nb = b.nb;
-  S.rec_aw = AW;
+  S.rec_words = RW;
   for (int a = 0; a < d.A; ++a) {
     float m;
     memcpy(&m, &hmax[a], sizeof(float));

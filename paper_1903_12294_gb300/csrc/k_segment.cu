@@ -729,17 +729,17 @@ constexpr uint32_t kRecChunkMax = 32768, kRecChunkMin = 1024;
 
 struct RecView {
   const uint2* rec_vn;    // [records] voxel, the point's voxel at the next point step (or -1)
-  const float* rec_a;     // [records][aw] attributes
+  const float* rec;       // [records][rw] attributes first
   const uint32_t* offs;   // [T][nb + 1] first record of each (field step, bucket); [t][nb]
                           // ends field step t's records
-  int nb, aw;
+  int nb, rw;
   uint32_t chunk;         // records per block
 };
 
 static RecView rec_view(const msf_ctx* ctx) {
   const BinScratch& B = ctx->bin;
-  return RecView{B.rec_vn.as<uint2>(), B.rec_a.as<float>(), B.offs.as<uint32_t>(), B.rec_nb,
-                 B.rec_aw, kRecChunkMax};
+  return RecView{B.rec_vn.as<uint2>(), B.rec.as<float>(), B.offs.as<uint32_t>(), B.rec_nb,
+                 B.rec_words, kRecChunkMax};
 }
 
 // Records per block for a pass of `steps` block rows (field steps, or batch items) over at most
@@ -1773,12 +1773,13 @@ constexpr size_t feat_vox_smem() {
 // samples are those of every point step falling in the window's field steps that binning placed
 // inside the grid: the same as the per-point pass takes. Block (x, y) takes records
 // [x * chunk, (x + 1) * chunk) of window field step y.
-// AW: attribute words of a record.
-template <bool SPATIAL, int AW>
+// RW: words of a record (4, 8 or 12, the first 2, 6 or 8 attributes).
+template <bool SPATIAL, int RW>
 __global__ void __launch_bounds__(256) k_feat_points_rec(const __grid_constant__ SegArgs a,
                                                          FeatAcc acc,
                                                          const int32_t* __restrict__ cfid,
                                                          const __grid_constant__ RecView rv) {
+  constexpr int AM = RW == 4 ? 2 : RW == 8 ? 6 : 8;
   __shared__ uint2 s_buf[8][kRecBuf];   // per warp: (voxel, record) of its members
   __shared__ HotCache s_hot[8][kHotWays];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1789,22 +1790,17 @@ __global__ void __launch_bounds__(256) k_feat_points_rec(const __grid_constant__
   const uint32_t step0 = step_seg0(a.g, tw);
   auto take = [&](bool ok, uint2 e) {  // 32 members (fewer at the end)
     int64_t fid = -1;
-    float v[AW] = {};
+    float v[AM] = {};
     if (ok) {
-      const float* p = rv.rec_a + (size_t)e.y * AW;
-      if constexpr (AW >= 4) {
+      const float* p = rv.rec + (size_t)e.y * RW;
 #pragma unroll
-        for (int q = 0; q < AW; q += 4) {
-          const float4 x = __ldg(reinterpret_cast<const float4*>(p + q));
-          v[q] = x.x, v[q + 1] = x.y, v[q + 2] = x.z, v[q + 3] = x.w;
-        }
-      } else {
-#pragma unroll
-        for (int q = 0; q < AW; ++q) v[q] = __ldg(p + q);
+      for (int q = 0; q < AM; q += 2) {
+        const float2 x = __ldg(reinterpret_cast<const float2*>(p + q));
+        v[q] = x.x, v[q + 1] = x.y;
       }
       fid = __ldg(cfid + comp_of<SPATIAL>(a, tw, (int32_t)e.x));
     }
-    accumulate_samples_hot<AW>(acc, s_hot[w], ok, fid, [&](int j) { return v[j]; });
+    accumulate_samples_hot<AM>(acc, s_hot[w], ok, fid, [&](int j) { return v[j]; });
     __syncwarp();  // the cached sums one reduction at a time
   };
   int n = 0;
@@ -1843,11 +1839,10 @@ __global__ void __launch_bounds__(256) k_feat_points_rec(const __grid_constant__
 template <bool SPATIAL>
 static void launch_feat_points(const SegArgs& a, const FeatAcc& acc, const int32_t* cfid,
                                const RecView& rv, dim3 grid, cudaStream_t s) {
-  switch (rv.aw) {
-    case 1: k_feat_points_rec<SPATIAL, 1><<<grid, 256, 0, s>>>(a, acc, cfid, rv); break;
-    case 2: k_feat_points_rec<SPATIAL, 2><<<grid, 256, 0, s>>>(a, acc, cfid, rv); break;
+  switch (rv.rw) {
     case 4: k_feat_points_rec<SPATIAL, 4><<<grid, 256, 0, s>>>(a, acc, cfid, rv); break;
-    default: k_feat_points_rec<SPATIAL, 8><<<grid, 256, 0, s>>>(a, acc, cfid, rv); break;
+    case 8: k_feat_points_rec<SPATIAL, 8><<<grid, 256, 0, s>>>(a, acc, cfid, rv); break;
+    default: k_feat_points_rec<SPATIAL, 12><<<grid, 256, 0, s>>>(a, acc, cfid, rv); break;
   }
 }
 

@@ -345,7 +345,7 @@ void msf_destroy(msf_ctx* c) {
   for (DevBuf* b : {&c->feat.rootbits, &c->feat.wordrank, &c->feat.blocksums, &c->feat.acc,
                     &c->feat.out})
     b->release();
-  for (DevBuf* b : {&c->bin.hist, &c->bin.offs, &c->bin.cursor, &c->bin.rec_vn, &c->bin.rec_a,
+  for (DevBuf* b : {&c->bin.hist, &c->bin.offs, &c->bin.cursor, &c->bin.rec_vn, &c->bin.rec,
                     &c->bin.absmax, &c->bin.outside, &c->bin.scan_tmp, &c->bin.total,
                     &c->bin.ovf})
     b->release();

@@ -163,13 +163,14 @@ struct BatchScratch {
 };
 
 struct BinScratch {
-  DevBuf hist, offs, cursor, rec_vn, rec_a, absmax, outside, scan_tmp, total, ovf;
+  DevBuf hist, offs, cursor, rec_vn, rec, absmax, outside, scan_tmp, total, ovf;
   // The records of the last binning stay for the trajectory joins and the feature statistics:
   // the samples grouped by (field step, bucket of 2^rec_logR voxels) in the slot ranges
   // offs[t][bucket] (offs [T][nb + 1]; offs[t][nb] ends field step t's records), each its voxel
-  // and its point's voxel at the next point step (rec_vn) and rec_aw attribute words (rec_a).
+  // and its point's voxel at the next point step (rec_vn), and rec_words words that start with
+  // its attributes (rec).
   bool rec_valid = false;
-  int rec_logR = 0, rec_nb = 0, rec_aw = 0;
+  int rec_logR = 0, rec_nb = 0, rec_words = 0;
 };
 
 // Scratch of the clustering (k_cluster.cu): centres, their sums and cells, label buffers for
