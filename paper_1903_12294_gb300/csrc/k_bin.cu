@@ -27,6 +27,7 @@
 //                  the trajectory joins
 #include <cuda_runtime.h>
 #include <math.h>
+#include <stddef.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -774,7 +775,8 @@ static void allow_smem(K kernel, size_t bytes, std::atomic<size_t>& set) {
   }
 }
 
-// phase 0: keys of point steps [j0, j0 + nj); 1: their records; 2: every (bucket, field step)
+// phase 0: keys of point steps [j0, j0 + nj); 1: their records; 2: every (bucket, field step);
+// 3: the nj of them that phase 2 listed
 template <int A>
 static void launch_bin(msf_ctx* ctx, BinArgs b, bool keep, int phase, bool smem, cudaStream_t s,
                        int j0, int nj) {
@@ -788,7 +790,7 @@ static void launch_bin(msf_ctx* ctx, BinArgs b, bool keep, int phase, bool smem,
   } else if (phase == 1) {
     ScopedKernel k(ctx, "k_bin_place", s);
     k_bin_place<A><<<gp, kPlaceNT, 0, s>>>(b);
-  } else {
+  } else if (phase == 2) {
     {
       ScopedKernel k(ctx, "k_bin_reduce", s);
       const size_t sm = reduce_smem(A, b.logR);
@@ -803,12 +805,12 @@ static void launch_bin(msf_ctx* ctx, BinArgs b, bool keep, int phase, bool smem,
         k_bin_reduce<A, false><<<gr, kBinNT, sm, s>>>(b);
       }
     }
+  } else {
     {
-      // the buckets k_bin_reduce listed (more records than it stages); blocks beyond their
-      // number leave at once
+      // the buckets k_bin_reduce listed (more records than it stages)
       ScopedKernel k(ctx, "k_bin_reduce_wide", s);
       const size_t sm = reduce_wide_smem(A, b.logR);
-      const unsigned g = (unsigned)std::min<int64_t>((int64_t)b.nb * b.T, (int64_t)ctx->sm_count * 2);
+      const unsigned g = (unsigned)std::min<int64_t>(nj, (int64_t)ctx->sm_count * 2);
       if (keep) {
         static std::atomic<size_t> set{0};
         allow_smem(k_bin_reduce_wide<A, true>, sm, set);
@@ -836,6 +838,13 @@ static void launch_bin_a(msf_ctx* ctx, const BinArgs& b, bool keep, int phase, b
     default: launch_bin<8>(ctx, b, keep, phase, smem, s, j0, nj); break;
   }
 }
+
+// The result words of a binning, behind its histogram: cleared with it and copied back at once.
+struct BinWords {
+  unsigned absmax[MSF_MAX_ATTR];
+  uint32_t err, novf;             // bounded waits that gave up, buckets left to the wide pass
+  unsigned long long outside[1];  // [Tp]
+};
 
 int bin_run(msf_ctx* ctx, unsigned flags) {
   Dataset& d = ctx->ds;
@@ -871,14 +880,14 @@ int bin_run(msf_ctx* ctx, unsigned flags) {
   if (NR >= ((int64_t)1 << 32) || TB >= ((int64_t)1 << 31) ||
       (d.P + kPlaceChunk - 1) / kPlaceChunk > 0x7FFFFFFF)
     return MSF_ERR_TOO_LARGE;
-  MSF_TRY(S.hist.ensure(sizeof(uint32_t) * TB));
+  const size_t hist_bytes = (sizeof(uint32_t) * (size_t)TB + 7) & ~size_t(7);
+  const size_t word_bytes = offsetof(BinWords, outside) + sizeof(unsigned long long) * d.Tp;
+  MSF_TRY(S.hist.ensure(hist_bytes + word_bytes));
+  MSF_TRY(ctx_result(ctx, word_bytes));
   MSF_TRY(S.offs.ensure(sizeof(uint32_t) * (TB + d.T)));
   MSF_TRY(S.cursor.ensure(sizeof(uint32_t) * kCurStride * TB));
   MSF_TRY(S.rec_vn.ensure(sizeof(uint2) * std::max<int64_t>(NR, 1)));
   MSF_TRY(S.rec.ensure(sizeof(uint32_t) * RW * std::max<int64_t>(NR, 1)));
-  MSF_TRY(S.absmax.ensure(sizeof(unsigned) * MSF_MAX_ATTR));
-  MSF_TRY(S.outside.ensure(sizeof(unsigned long long) * d.Tp));
-  MSF_TRY(S.total.ensure(sizeof(uint32_t) * 4));  // [2] error word, [3] wide items
   MSF_TRY(S.ovf.ensure(sizeof(uint32_t) * (size_t)d.T * (size_t)b.nb));
   MSF_TRY(d.key.ensure(sizeof(int32_t) * ((int64_t)d.Tp * d.P + 4)));  // slack: bulk copies
   MSF_TRY(d.count.ensure(sizeof(int32_t) * d.T * d.V));
@@ -894,11 +903,12 @@ int bin_run(msf_ctx* ctx, unsigned flags) {
   b.rec = S.rec.as<uint32_t>();
   b.wait_cycles = ctx->wait_cycles;
   b.pf_ahead = ctx->sm_count * (d.A <= 4 ? 3 : 2);  // resident reduce blocks
-  b.err = S.total.as<uint32_t>() + 2;
-  b.novf = S.total.as<uint32_t>() + 3;
+  BinWords* dw = reinterpret_cast<BinWords*>(S.hist.as<char>() + hist_bytes);
+  b.err = &dw->err;
+  b.novf = &dw->novf;
   b.ovf = S.ovf.as<uint32_t>();
-  b.absmax = S.absmax.as<unsigned>();
-  b.outside = S.outside.as<unsigned long long>();
+  b.absmax = dw->absmax;
+  b.outside = dw->outside;
   b.count = d.count.as<int32_t>();
   b.mean = d.mean.as<float>();
   b.sumq = keep ? d.sumq.as<long long>() : nullptr;
@@ -911,14 +921,10 @@ int bin_run(msf_ctx* ctx, unsigned flags) {
   const bool piped = ctx->points_pending && d.P > 0;
   if (piped) ct = ctx->chunk_t;
   ctx->points_pending = false;
-  MSF_CUDA_TRY(cudaMemsetAsync(b.hist, 0, sizeof(uint32_t) * TB, s));
+  MSF_CUDA_TRY(cudaMemsetAsync(b.hist, 0, hist_bytes + word_bytes, s));
   if (d.scale_fixed)  // the whole dataset's maxima: a slab's can only be smaller
     MSF_CUDA_TRY(cudaMemcpyAsync(b.absmax, d.scale_absmax, sizeof(unsigned) * MSF_MAX_ATTR,
                                  cudaMemcpyHostToDevice, s));
-  else
-    MSF_CUDA_TRY(cudaMemsetAsync(b.absmax, 0, sizeof(unsigned) * MSF_MAX_ATTR, s));
-  MSF_CUDA_TRY(cudaMemsetAsync(b.outside, 0, sizeof(unsigned long long) * d.Tp, s));
-  MSF_CUDA_TRY(cudaMemsetAsync(b.err, 0, 2 * sizeof(uint32_t), s));  // error word, wide items
   if (d.P > 0) {
     const int G = (int)ct.size() - 1;
     auto keys = [&](int g) -> int {
@@ -942,20 +948,22 @@ int bin_run(msf_ctx* ctx, unsigned flags) {
   }
   launch_bin_a(ctx, b, keep, 2, smem, s);
   MSF_CUDA_TRY(cudaGetLastError());
-  std::vector<unsigned long long> out(d.Tp);
-  unsigned hmax[MSF_MAX_ATTR] = {};
-  MSF_CUDA_TRY(cudaMemcpyAsync(out.data(), S.outside.p, sizeof(unsigned long long) * d.Tp,
-                               cudaMemcpyDeviceToHost, s));
-  MSF_CUDA_TRY(cudaMemcpyAsync(hmax, S.absmax.p, sizeof(hmax), cudaMemcpyDeviceToHost, s));
-  uint32_t herr = 0;
-  MSF_CUDA_TRY(cudaMemcpyAsync(&herr, b.err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+  const BinWords* hw = static_cast<const BinWords*>(ctx->res);
+  MSF_CUDA_TRY(cudaMemcpyAsync(ctx->res, dw, word_bytes, cudaMemcpyDeviceToHost, s));
   S.rec_valid = false;
   MSF_CUDA_TRY(cudaStreamSynchronize(s));
+  if (hw->novf && !hw->err) {  // crowded buckets (rare): the wide pass, now that they are known
+    launch_bin_a(ctx, b, keep, 3, smem, s, 0, (int)hw->novf);
+    MSF_CUDA_TRY(cudaGetLastError());
+    MSF_CUDA_TRY(cudaMemcpyAsync(ctx->res, dw, word_bytes, cudaMemcpyDeviceToHost, s));
+    MSF_CUDA_TRY(cudaStreamSynchronize(s));
+  }
   ctx->timer.flush();
-  if (herr) {
+  if (hw->err) {
     d.binned = false;
     return MSF_ERR_TIMEOUT;
   }
+  const unsigned* hmax = hw->absmax;
   S.rec_valid = d.P > 0;
   S.rec_logR = b.logR;
   S.rec_nb = b.nb;
@@ -967,7 +975,7 @@ int bin_run(msf_ctx* ctx, unsigned flags) {
     d.kscale[a] = scale_exponent_bits(hmax[a], (long long)b.scale_n);
   }
   int64_t o = 0;
-  for (auto v : out) o += (int64_t)v;
+  for (int j = 0; j < d.Tp; ++j) o += (int64_t)hw->outside[j];
   d.out_of_domain = o;
   d.in_domain = d.P * (int64_t)d.Tp - o;
   d.binned = true;

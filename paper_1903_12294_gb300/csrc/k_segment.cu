@@ -496,10 +496,7 @@ __device__ __forceinline__ void tile_body(const SegArgs& a, const int tile, cons
 
   // ---- phase 5: compact outputs ----------------------------------------------------------
   if (ncomp_tile > g.cmax || nrun_tile > a.maxr) {  // cannot happen by construction
-    if (tid == 0) {
-      atomicOr(&a.counters[1], 1ull);
-      a.tileinfo[tile] = make_int2(0, 0);
-    }
+    if (tid == 0) a.tileinfo[tile] = make_int2(0, -1);  // (k_flatten reports it)
     return;
   }
   const uint32_t rbase = (uint32_t)tile * (uint32_t)a.maxr;
@@ -531,6 +528,8 @@ __global__ void __launch_bounds__(256, 6) k_tile(const __grid_constant__ SegArgs
   __shared__ int s_warp[8];
   extern __shared__ uint32_t s_dyn[];
   const TileSmem sm{s_mask, s_rb, s_warp, s_dyn, reinterpret_cast<uint16_t*>(s_dyn + MAXR), MAXR};
+  // the counters of the query (added to from k_flatten on) start at zero
+  if (a.tile0 == 0 && blockIdx.x == 0 && threadIdx.x < 2) a.counters[threadIdx.x] = 0ull;
   tile_body<NP, SPATIAL, VEC>(a, a.tile0 + (int)blockIdx.x, sm);
 }
 
@@ -874,6 +873,7 @@ __device__ __forceinline__ void flatten_body(const SegArgs& a, const int tile, i
   if (threadIdx.x == 0) s_n = 0;
   __syncthreads();
   const int nc = min(__ldcg(&a.tileinfo[tile].y), a.g.cmax);
+  if (nc < 0 && threadIdx.x == 0) atomicOr(&a.counters[1], 1ull);
   const uint32_t cbase = (uint32_t)tile * (uint32_t)a.g.cmax;
   int roots = 0;
   for (int k = threadIdx.x; k < nc; k += blockDim.x) {
@@ -1228,7 +1228,7 @@ int segment_run(msf_ctx* ctx, const msf_criteria* crit, int32_t* labels, int64_t
   a.labels = labels;
   cudaStream_t s = ctx->stream;
   const int sched = segment_schedule(ctx, crit);
-  MSF_CUDA_TRY(cudaMemsetAsync(a.counters, 0, sizeof(unsigned long long) * 4, s));
+  MSF_TRY(ctx_result(ctx, sizeof(unsigned long long) * 2));
   // Without a schedule set or tuned the criterion is evaluated inside the tile pass: its loads
   // overlap the labelling, which is bound by instruction issue, and the masks' round trip through
   // L2 goes. The streaming pass was the faster one on no size measured (one query, streamed
@@ -1336,8 +1336,9 @@ int segment_run(msf_ctx* ctx, const msf_criteria* crit, int32_t* labels, int64_t
     }
   }
   MSF_CUDA_TRY(cudaGetLastError());
-  unsigned long long h[2];
-  MSF_CUDA_TRY(cudaMemcpyAsync(h, a.counters, sizeof(h), cudaMemcpyDeviceToHost, s));
+  const auto* h = static_cast<const unsigned long long*>(ctx->res);
+  MSF_CUDA_TRY(cudaMemcpyAsync(ctx->res, a.counters, sizeof(unsigned long long) * 2,
+                               cudaMemcpyDeviceToHost, s));
   MSF_CUDA_TRY(cudaStreamSynchronize(s));
   ctx->timer.flush();
   if (h[1]) return MSF_ERR_INTERNAL;
@@ -2013,9 +2014,8 @@ int segment_field_fixed(const Geometry& g, int npred, const DevPred& pred, uint3
   a.tileinfo = S.tileinfo;
   a.counters = S.counters;
   a.labels = labels;
-  // The scratch keeps the previous call's contents: only the counters must start at zero
-  // (every other entry the kernels read is written earlier in this same call).
-  MSF_CUDA_TRY(cudaMemsetAsync(a.counters, 0, sizeof(unsigned long long) * 8, s));
+  // The scratch keeps the previous call's contents: only the counters must start at zero, which
+  // the tile pass sees to (every other entry the kernels read is written earlier in this call).
   launch_tile_any(a, spatial, g.ntiles, s);
   MSF_CUDA_TRY(cudaGetLastError());
   if (edges & (MSF_EDGE_SPATIAL | MSF_EDGE_TEMPORAL)) {

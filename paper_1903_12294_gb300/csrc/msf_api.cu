@@ -142,6 +142,17 @@ int ctx_field_ready(msf_ctx* ctx) {
   return MSF_OK;
 }
 
+int ctx_result(msf_ctx* ctx, size_t bytes) {
+  if (bytes <= ctx->res_bytes) return MSF_OK;
+  if (ctx->res) cudaFreeHost(ctx->res);
+  ctx->res = nullptr;
+  ctx->res_bytes = 0;
+  const size_t n = std::max<size_t>(bytes, 4096);
+  MSF_CUDA_TRY(cudaMallocHost(&ctx->res, n));
+  ctx->res_bytes = n;
+  return MSF_OK;
+}
+
 int ctx_join(msf_ctx* ctx) {
   MSF_CUDA_TRY(cudaEventRecord(ctx->ev_join, ctx->aux));
   MSF_CUDA_TRY(cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0));
@@ -346,8 +357,7 @@ void msf_destroy(msf_ctx* c) {
                     &c->feat.out})
     b->release();
   for (DevBuf* b : {&c->bin.hist, &c->bin.offs, &c->bin.cursor, &c->bin.rec_vn, &c->bin.rec,
-                    &c->bin.absmax, &c->bin.outside, &c->bin.scan_tmp, &c->bin.total,
-                    &c->bin.ovf})
+                    &c->bin.scan_tmp, &c->bin.ovf})
     b->release();
   c->bin.rec_valid = false;
   c->last.cfid.release();
@@ -357,6 +367,7 @@ void msf_destroy(msf_ctx* c) {
                     &c->clu.pcell_cursor, &c->clu.psample, &c->clu.ptime, &c->clu.pindex})
     b->release();
   c->host_staging.release();
+  if (c->res) cudaFreeHost(c->res);
   c->post.release();
   c->batch.release();
   c->timer.release();

@@ -163,7 +163,8 @@ struct BatchScratch {
 };
 
 struct BinScratch {
-  DevBuf hist, offs, cursor, rec_vn, rec, absmax, outside, scan_tmp, total, ovf;
+  // hist ends in the binning's result words (one clear, one copy back): see BinWords
+  DevBuf hist, offs, cursor, rec_vn, rec, scan_tmp, ovf;
   // The records of the last binning stay for the trajectory joins and the feature statistics:
   // the samples grouped by (field step, bucket of 2^rec_logR voxels) in the slot ranges
   // offs[t][bucket] (offs [T][nb + 1]; offs[t][nb] ends field step t's records), each its voxel
@@ -237,6 +238,10 @@ struct msf_ctx {
   msf::ClusterScratch clu;
   msf::PostScratch post;
   msf::DevBuf host_staging;  // device-side staging for host label buffers
+  // Page-locked words the calls' results come back to (grow-only): a copy into pageable memory
+  // is staged by the driver and waits for the device each time, one into these is not.
+  void* res = nullptr;
+  size_t res_bytes = 0;
   msf::SegState last;        // retained segmentation of the last msf_segment call
   uint64_t epoch = 1;        // bumped whenever the dataset or its binning changes
   int tile_by = 0, tile_bz = 0, tile_bt = 0;
@@ -292,6 +297,7 @@ int ctx_aux(msf_ctx* ctx);  // creates the auxiliary stream and its events on fi
 int ctx_fork(msf_ctx* ctx);
 int ctx_join(msf_ctx* ctx);
 int ctx_field_ready(msf_ctx* ctx);  // the context stream waits for a field copy in flight
+int ctx_result(msf_ctx* ctx, size_t bytes);  // ctx->res holds at least `bytes`
 
 // An auxiliary stream with its fork and join events, for a main stream given at each use.
 struct StreamPair {
