@@ -407,6 +407,11 @@ __device__ __forceinline__ void tile_body(const SegArgs& a, const int tile, cons
   const int nr = __popc(st);
   int nrun_tile;
   const int rb = block_exscan(nr, s_warp, &nrun_tile);
+  if (nrun_tile == 0) {  // no member in the tile: the rows' empty masks are all it leaves
+    if (row != kNoRow) a.seg[gs] = make_uint2(0u, (uint32_t)tile * (uint32_t)a.maxr);
+    if (tid == 0) a.tileinfo[tile] = make_int2(0, 0);
+    return;
+  }
   s_rb[s] = rb;
   for (int j = 0; j < nr; ++j) s_par[rb + j] = rb + j;
   __syncthreads();
@@ -632,6 +637,7 @@ __device__ __forceinline__ void hook_tile(const SegArgs& a, int tile, unsigned l
 template <bool SPATIAL>
 __global__ void __launch_bounds__(256, 4) k_hook(const __grid_constant__ SegArgs a) {
   __shared__ unsigned long long s_set[kHookSet];
+  if (__ldg(&a.tileinfo[blockIdx.x].x) == 0) return;  // no member in the tile
   for (int i = threadIdx.x; i < kHookSet; i += 256) s_set[i] = ~0ull;
   __syncthreads();
   hook_tile<SPATIAL>(a, blockIdx.x, s_set);
@@ -752,11 +758,12 @@ static uint32_t rec_chunk(int64_t per_step, int steps, int sm_count) {
 }
 
 // records [b0, b1) of block x of field step t; false when the block has none
-__device__ __forceinline__ bool rec_block(const RecView& rv, int t, uint32_t& b0, uint32_t& b1) {
+__device__ __forceinline__ bool rec_block(const RecView& rv, int t, uint32_t x, uint32_t& b0,
+                                          uint32_t& b1) {
   const int64_t h = (int64_t)t * (rv.nb + 1);
   const uint32_t rb = __ldg(rv.offs + h);
   const uint32_t re = __ldg(rv.offs + h + rv.nb);
-  b0 = rb + blockIdx.x * rv.chunk;
+  b0 = rb + x * rv.chunk;
   if (b0 >= re) return false;
   b1 = min(re, b0 + rv.chunk);
   return true;
@@ -861,8 +868,33 @@ __global__ void __launch_bounds__(256) k_links_rec(const __grid_constant__ SegAr
   __shared__ uint2 s_buf[8][kRecBuf];
   const int tw = ta + (int)blockIdx.y;
   uint32_t b0, b1;
-  if (!rec_block(rv, a.g.t0 + tw, b0, b1)) return;
+  if (!rec_block(rv, a.g.t0 + tw, blockIdx.x, b0, b1)) return;
   links_rec_range<SPATIAL>(a, rv, tw, b0, b1, s_buf[threadIdx.x >> 5]);
+}
+
+// The cross-tile and the trajectory joins of a small window in one launch: blocks [0, nhook) take
+// a tile each, the others record block x = i % nx of window step i / nx. Where all of them are
+// resident at once, two launches on two streams cost their events and nothing overlaps better
+// (the step of a 32^3 x 8 window 259 us, so and with the feature passes joined likewise 244 to
+// 253 us).
+template <bool SPATIAL>
+__global__ void __launch_bounds__(256, 4) k_joins(const __grid_constant__ SegArgs a,
+                                                  const __grid_constant__ RecView rv, int nhook,
+                                                  int nx) {
+  __shared__ __align__(16) unsigned long long s_mem[kHookSet];
+  static_assert(sizeof(uint2) * 8 * kRecBuf <= sizeof(s_mem), "the record buffers fit");
+  if ((int)blockIdx.x < nhook) {
+    if (__ldg(&a.tileinfo[blockIdx.x].x) == 0) return;  // no member in the tile
+    for (int i = threadIdx.x; i < kHookSet; i += 256) s_mem[i] = ~0ull;
+    __syncthreads();
+    hook_tile<SPATIAL>(a, blockIdx.x, s_mem);
+    return;
+  }
+  const int i = (int)blockIdx.x - nhook, tw = i / nx;
+  uint32_t b0, b1;
+  if (!rec_block(rv, a.g.t0 + tw, (uint32_t)(i - tw * nx), b0, b1)) return;
+  links_rec_range<SPATIAL>(a, rv, tw, b0, b1,
+                           reinterpret_cast<uint2*>(s_mem) + kRecBuf * (threadIdx.x >> 5));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1302,7 +1334,24 @@ int segment_run(msf_ctx* ctx, const msf_criteria* crit, int32_t* labels, int64_t
     if (spatial) k_links<true><<<grid, 256, 0, ls>>>(al);
     else k_links<false><<<grid, 256, 0, ls>>>(al);
   };
-  if (split_tiles > 0) {
+  // a small window's joins in one launch (every block resident at once)
+  const bool hooks = (crit->edges & (MSF_EDGE_SPATIAL | MSF_EDGE_TEMPORAL)) != 0;
+  bool joined = false;
+  if (traj && !serial && hooks && rec_links && split_tiles == 0 && g.tw > 1) {
+    RecView rv = rec_view(ctx);
+    rv.chunk = rec_chunk(a.P, g.tw - 1, ctx->sm_count);
+    const int64_t nx = std::max<int64_t>(1, (a.P + rv.chunk - 1) / rv.chunk);
+    const int64_t blocks = g.ntiles + nx * (g.tw - 1);
+    joined = blocks <= 4 * (int64_t)ctx->sm_count;
+    if (joined) {
+      ScopedKernel k(ctx, "k_joins");
+      if (spatial) k_joins<true><<<(unsigned)blocks, 256, 0, s>>>(a, rv, g.ntiles, (int)nx);
+      else k_joins<false><<<(unsigned)blocks, 256, 0, s>>>(a, rv, g.ntiles, (int)nx);
+    }
+  }
+  if (joined) {
+    // nothing left to launch
+  } else if (split_tiles > 0) {
     MSF_TRY(ctx_fork(ctx));            // after the first tile rows
     links(ctx->aux, 0, ready_chunks);
     tiles(split_tiles, g.ntiles - split_tiles);
@@ -1312,13 +1361,13 @@ int segment_run(msf_ctx* ctx, const msf_criteria* crit, int32_t* labels, int64_t
     MSF_TRY(ctx_fork(ctx));
     links(ctx->aux, 0, nchunk);
   }
-  if ((crit->edges & (MSF_EDGE_SPATIAL | MSF_EDGE_TEMPORAL)) != 0) {
+  if (hooks && !joined) {
     ScopedKernel k(ctx, "k_hook");
     if (spatial) k_hook<true><<<g.ntiles, 256, 0, s>>>(a);
     else k_hook<false><<<g.ntiles, 256, 0, s>>>(a);
   }
   if (traj && serial) links(s, 0, nchunk);
-  if (traj && !serial) MSF_TRY(ctx_join(ctx));
+  if (traj && !serial && !joined) MSF_TRY(ctx_join(ctx));
   {
     ScopedKernel k(ctx, "k_flatten");
     k_flatten<<<g.ntiles, 256, 0, s>>>(a);
@@ -1630,10 +1679,10 @@ __device__ __forceinline__ void vox_warp(const FeatAcc& acc, const Geometry& g,
 }
 
 template <bool SPATIAL>
-__global__ void __launch_bounds__(256) k_feat_vox(const __grid_constant__ SegArgs a, FeatAcc acc,
-                                                  const int32_t* __restrict__ cfid,
-                                                  const float* __restrict__ field,
-                                                  const int32_t* __restrict__ count) {
+__device__ __forceinline__ void feat_vox_tile(const SegArgs& a, const FeatAcc& acc,
+                                              const int32_t* __restrict__ cfid,
+                                              const float* __restrict__ field,
+                                              const int32_t* __restrict__ count, const int tile) {
   constexpr int MAXR = kSegPerTile * (SPATIAL ? 16 : 32);
   constexpr int kBig = kSegPerTile * 32 / kCompWarp;  // slots above kCompWarp voxels
   extern __shared__ uint32_t s_dynv[];
@@ -1644,7 +1693,6 @@ __global__ void __launch_bounds__(256) k_feat_vox(const __grid_constant__ SegArg
   __shared__ int s_nbig, s_big[kBig];
   const Geometry& g = a.g;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int tile = blockIdx.x;
   const int2 info = __ldg(a.tileinfo + tile);
   const int ncomp = min(info.y, MAXR);
   if (info.x == 0 || ncomp == 0) return;
@@ -1760,6 +1808,14 @@ __global__ void __launch_bounds__(256) k_feat_vox(const __grid_constant__ SegArg
   }
 }
 
+template <bool SPATIAL>
+__global__ void __launch_bounds__(256) k_feat_vox(const __grid_constant__ SegArgs a, FeatAcc acc,
+                                                  const int32_t* __restrict__ cfid,
+                                                  const float* __restrict__ field,
+                                                  const int32_t* __restrict__ count) {
+  feat_vox_tile<SPATIAL>(a, acc, cfid, field, count, blockIdx.x);
+}
+
 template <bool SP>
 constexpr size_t feat_vox_smem() {
   return ((size_t)kSegPerTile * (SP ? 16 : 32) + kVoxHash) * sizeof(uint32_t) +
@@ -1776,17 +1832,15 @@ constexpr size_t feat_vox_smem() {
 // [x * chunk, (x + 1) * chunk) of window field step y.
 // RW: words of a record (4, 8 or 12, the first 2, 6 or 8 attributes).
 template <bool SPATIAL, int RW>
-__global__ void __launch_bounds__(256) k_feat_points_rec(const __grid_constant__ SegArgs a,
-                                                         FeatAcc acc,
-                                                         const int32_t* __restrict__ cfid,
-                                                         const __grid_constant__ RecView rv) {
+__device__ __forceinline__ void feat_points_block(const SegArgs& a, const FeatAcc& acc,
+                                                  const int32_t* __restrict__ cfid,
+                                                  const RecView& rv, const int tw, uint32_t x) {
   constexpr int AM = RW == 4 ? 2 : RW == 8 ? 6 : 8;
   __shared__ uint2 s_buf[8][kRecBuf];   // per warp: (voxel, record) of its members
   __shared__ HotCache s_hot[8][kHotWays];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int tw = blockIdx.y;
   uint32_t b0, b1;
-  if (!rec_block(rv, a.g.t0 + tw, b0, b1)) return;  // block-uniform
+  if (!rec_block(rv, a.g.t0 + tw, x, b0, b1)) return;  // block-uniform
   hot_clear(s_hot[w]);
   const uint32_t step0 = step_seg0(a.g, tw);
   auto take = [&](bool ok, uint2 e) {  // 32 members (fewer at the end)
@@ -1835,6 +1889,51 @@ __global__ void __launch_bounds__(256) k_feat_points_rec(const __grid_constant__
   take(lane < n, lane < n ? s_buf[w][lane] : make_uint2(0u, b0));
   __syncthreads();
   hot_merge(acc, s_hot);
+}
+
+template <bool SPATIAL, int RW>
+__global__ void __launch_bounds__(256) k_feat_points_rec(const __grid_constant__ SegArgs a,
+                                                         FeatAcc acc,
+                                                         const int32_t* __restrict__ cfid,
+                                                         const __grid_constant__ RecView rv) {
+  feat_points_block<SPATIAL, RW>(a, acc, cfid, rv, blockIdx.y, blockIdx.x);
+}
+
+// Both of a small window in one launch (as k_joins): blocks [0, ntiles) take a tile each, the
+// others record block i % nx of window step i / nx.
+template <bool SPATIAL, int RW>
+__global__ void __launch_bounds__(256) k_feat_both(const __grid_constant__ SegArgs a, FeatAcc acc,
+                                                   const int32_t* __restrict__ cfid,
+                                                   const float* __restrict__ field,
+                                                   const int32_t* __restrict__ count,
+                                                   const __grid_constant__ RecView rv, int nx) {
+  if ((int)blockIdx.x < a.g.ntiles) {
+    feat_vox_tile<SPATIAL>(a, acc, cfid, field, count, blockIdx.x);
+  } else {
+    const int i = (int)blockIdx.x - a.g.ntiles, tw = i / nx;
+    feat_points_block<SPATIAL, RW>(a, acc, cfid, rv, tw, (uint32_t)(i - tw * nx));
+  }
+}
+
+template <bool SPATIAL, int RW>
+static void launch_feat_both_rw(const SegArgs& a, const FeatAcc& acc, const int32_t* cfid,
+                                const float* field, const int32_t* count, const RecView& rv,
+                                int nx, unsigned blocks, cudaStream_t s) {
+  static std::atomic<uint64_t> attr_set{0};
+  ensure_smem_attr(k_feat_both<SPATIAL, RW>, feat_vox_smem<SPATIAL>(), attr_set);
+  k_feat_both<SPATIAL, RW><<<blocks, 256, feat_vox_smem<SPATIAL>(), s>>>(a, acc, cfid, field, count,
+                                                                         rv, nx);
+}
+
+template <bool SPATIAL>
+static void launch_feat_both(const SegArgs& a, const FeatAcc& acc, const int32_t* cfid,
+                             const float* field, const int32_t* count, const RecView& rv, int nx,
+                             unsigned blocks, cudaStream_t s) {
+  switch (rv.rw) {
+    case 4: launch_feat_both_rw<SPATIAL, 4>(a, acc, cfid, field, count, rv, nx, blocks, s); break;
+    case 8: launch_feat_both_rw<SPATIAL, 8>(a, acc, cfid, field, count, rv, nx, blocks, s); break;
+    default: launch_feat_both_rw<SPATIAL, 12>(a, acc, cfid, field, count, rv, nx, blocks, s); break;
+  }
 }
 
 template <bool SPATIAL>
@@ -1895,15 +1994,25 @@ int seg_feature_stats(msf_ctx* ctx, const RankArrays& rk, const FeatAcc& acc, in
   // voxel pass on the auxiliary stream
   const bool points = a.P > 0 && d.A > 0 && a.nj > 0;
   if (points && !recs) return MSF_ERR_INTERNAL;  // not reached: see above
+  RecView rv = rec_view(ctx);
+  int rmax = 1;  // most point steps in one field step of the window
+  for (int t = g.t0; t < g.t0 + g.tw; ++t) rmax = std::max(rmax, d.h_pj0[t + 1] - d.h_pj0[t]);
+  rv.chunk = rec_chunk(a.P * rmax, g.tw, ctx->sm_count);
+  const int64_t nx = std::max<int64_t>(1, (a.P * rmax + rv.chunk - 1) / rv.chunk);
+  const int64_t both = g.ntiles + nx * g.tw;
+  if (points && both <= 4 * (int64_t)ctx->sm_count) {
+    ScopedKernel k(ctx, "k_feat_both");
+    const float* f = d.field.as<float>();
+    const int32_t* cnt = d.count.as<int32_t>();
+    if (spatial) launch_feat_both<true>(a, acc, cfid, f, cnt, rv, (int)nx, (unsigned)both, s);
+    else launch_feat_both<false>(a, acc, cfid, f, cnt, rv, (int)nx, (unsigned)both, s);
+    MSF_CUDA_TRY(cudaGetLastError());
+    return MSF_OK;
+  }
   if (points) {
     MSF_TRY(ctx_fork(ctx));
     ScopedKernel k(ctx, "k_feat_points", ctx->aux);
-    RecView rv = rec_view(ctx);
-    int rmax = 1;  // most point steps in one field step of the window
-    for (int t = g.t0; t < g.t0 + g.tw; ++t) rmax = std::max(rmax, d.h_pj0[t + 1] - d.h_pj0[t]);
-    rv.chunk = rec_chunk(a.P * rmax, g.tw, ctx->sm_count);
-    const int64_t nx = (a.P * rmax + rv.chunk - 1) / rv.chunk;
-    dim3 grid((unsigned)std::max<int64_t>(nx, 1), (unsigned)g.tw);
+    dim3 grid((unsigned)nx, (unsigned)g.tw);
     if (spatial) launch_feat_points<true>(a, acc, cfid, rv, grid, ctx->aux);
     else launch_feat_points<false>(a, acc, cfid, rv, grid, ctx->aux);
   }
@@ -2144,9 +2253,11 @@ __global__ void __launch_bounds__(256, 4) k_hook_batch(const __grid_constant__ B
   __shared__ unsigned long long s_set[kHookSet];
   __shared__ __align__(16) SegArgs s_args;
   load_args(&s_args, b.qargs + blockIdx.y);
-  for (int i = threadIdx.x; i < kHookSet; i += 256) s_set[i] = ~0ull;
   __syncthreads();
   if ((int)blockIdx.x >= s_args.g.ntiles) return;  // block-uniform
+  if (__ldg(&s_args.tileinfo[blockIdx.x].x) == 0) return;  // no member in the tile
+  for (int i = threadIdx.x; i < kHookSet; i += 256) s_set[i] = ~0ull;
+  __syncthreads();
   hook_tile<SPATIAL>(s_args, blockIdx.x, s_set);
 }
 
@@ -2179,7 +2290,7 @@ __global__ void __launch_bounds__(256, 4) k_links_batch_rec(const __grid_constan
     const int tw = c0 + st;
     if (tw >= s_args.g.tw - 1) break;  // block-uniform
     uint32_t b0, b1;
-    if (!rec_block(rv, s_args.g.t0 + tw, b0, b1)) continue;  // block-uniform
+    if (!rec_block(rv, s_args.g.t0 + tw, blockIdx.x, b0, b1)) continue;  // block-uniform
     links_rec_range<SPATIAL>(s_args, rv, tw, b0, b1, s_buf[threadIdx.x >> 5]);
   }
 }
