@@ -542,59 +542,6 @@ __global__ void __launch_bounds__(256, 6) k_tile(const __grid_constant__ SegArgs
 // k_hook: joins across tile boundaries
 // ---------------------------------------------------------------------------------------------
 
-// Cross-tile joins of one segment (tw, z, y, xs) with mask m != 0: its first run against the
-// last runs of the nine rows to the left (another tile), the backward rows in y/z that lie in
-// another tile, and the row one step earlier when the segment opens a time chunk. Every join of
-// two components goes through join(c0, c1).
-template <bool SPATIAL, bool CG, class J>
-__device__ __forceinline__ void hook_seg(const SegArgs& a, int tw, int z, int y, int xs,
-                                         uint32_t m, uint32_t rb, J&& join) {
-  const Geometry& g = a.g;
-  const uint32_t st = run_starts(m, SPATIAL);
-
-  auto join_rows = [&](int64_t gs2, bool spatial_rows) {
-    const uint2 e2 = ld_seg<CG>(a.seg + gs2);
-    const uint32_t m2 = e2.x;
-    if (!m2) return;
-    const uint32_t st2 = run_starts(m2, SPATIAL);
-    const uint32_t rb2 = e2.y;
-    row_contacts(m, m2, spatial_rows, SPATIAL, [&](int x1, int x2) {
-      const uint32_t c1 = ld_seg<CG>(a.runcomp + rb + run_index(st, x1));
-      const uint32_t c2 = ld_seg<CG>(a.runcomp + rb2 + run_index(st2, x2));
-      if (c1 != c2) join(c1, c2);
-    });
-  };
-
-  if (SPATIAL) {
-    // x-neighbour segments (always another tile): bit 0 here against bit 31 of the segment
-    // to the left, for all 9 (dy, dz)
-    if ((m & 1u) && xs > 0) {
-      const uint32_t c0 = ld_seg<CG>(a.runcomp + rb);
-      uint32_t last = kNoComp;
-      for (int k = 0; k < 9; ++k) {
-        const int z2 = z + k / 3 - 1, y2 = y + k % 3 - 1;
-        if (z2 < 0 || z2 >= g.nz || y2 < 0 || y2 >= g.ny) continue;
-        const uint2 e2 = ld_seg<CG>(a.seg + seg_index(g, tw, z2, y2, xs - 1));
-        if (!(e2.x >> 31)) continue;
-        const uint32_t c2 = ld_seg<CG>(a.runcomp + e2.y + __popc(run_starts(e2.x, SPATIAL)) - 1);
-        if (c2 != c0 && c2 != last) join(c0, c2);
-        last = c2;
-      }
-    }
-    // backward rows in y/z that lie in another tile
-    const int dys[4] = {-1, -1, 0, 1}, dzs[4] = {0, -1, -1, -1};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int y2 = y + dys[k], z2 = z + dzs[k];
-      if (y2 < 0 || y2 >= g.ny || z2 < 0) continue;
-      if ((y2 >> g.lby) == (y >> g.lby) && (z2 >> g.lbz) == (z >> g.lbz)) continue;
-      join_rows(seg_index(g, tw, z2, y2, xs), true);
-    }
-  }
-  if ((a.edges & MSF_EDGE_TEMPORAL) && tw > 0 && ((tw + g.toff) & ((1 << g.lbt) - 1)) == 0)
-    join_rows(seg_index(g, tw - 1, z, y, xs), false);
-}
-
 // The component pairs one tile joins across its faces repeat heavily (a feature crossing a face
 // touches it in many rows). Each tile keeps the pairs it has joined in a shared-memory set and
 // joins a pair only the first time it meets it.
@@ -615,32 +562,100 @@ __device__ __forceinline__ bool pair_first_seen(unsigned long long* set, uint32_
   return true;  // crowded: join without remembering
 }
 
-// One tile's cross-face joins, one thread per segment (s_set cleared by the caller).
+struct HookSmem {
+  unsigned long long set[kHookSet];
+  uint32_t mask[kSegPerTile], rb[kSegPerTile];
+  int warp[8];
+  uint16_t task[kSegPerTile * 14];  // row | direction << 8
+};
+
+// One tile's cross-face joins. A row with members meets up to 14 rows of other tiles: the nine to
+// its left (its first run against their last ones), the backward rows in y/z that lie in another
+// tile, and the row one step earlier when it opens a time chunk. A few rows of a tile have
+// members, and the pass waits on L2: the (row, direction) pairs are listed first and the block's
+// threads take one each, so that the lookups of a row run beside each other (one thread walking
+// its row's directions, 256^3 x 24 with three predicates, 0.81 ms, now 0.60 ms).
 template <bool SPATIAL, bool CG = false>
-__device__ __forceinline__ void hook_tile(const SegArgs& a, int tile, unsigned long long* s_set) {
+__device__ __forceinline__ void hook_tile(const SegArgs& a, int tile, HookSmem& S) {
   const Geometry& g = a.g;
+  const int tid = threadIdx.x;
+  for (int i = tid; i < kHookSet; i += 256) S.set[i] = ~0ull;
   const TileCoord tc = tile_coord(g, tile);
-  const int sg = threadIdx.x;
-  const int ly = sg & ((1 << g.lby) - 1), lz = (sg >> g.lby) & ((1 << g.lbz) - 1);
-  const int lt = sg >> (g.lby + g.lbz);
-  const int y = (tc.ty << g.lby) + ly, z = (tc.tz << g.lbz) + lz;
-  const int tw = (tc.tt << g.lbt) + lt - g.toff;
-  if (y >= g.ny || z >= g.nz || tw < 0 || tw >= g.tw) return;
-  const uint2 e = ld_seg<CG>(a.seg + seg_index(g, tw, z, y, tc.xs));
-  if (!e.x) return;
-  hook_seg<SPATIAL, CG>(a, tw, z, y, tc.xs, e.x, e.y, [&](uint32_t c0, uint32_t c1) {
-    if (pair_first_seen(s_set, c0, c1)) gunion(a.cparent, c0, c1);
-  });
+  auto coords = [&](int r, int& tw, int& z, int& y) {
+    y = (tc.ty << g.lby) + (r & ((1 << g.lby) - 1));
+    z = (tc.tz << g.lbz) + ((r >> g.lby) & ((1 << g.lbz) - 1));
+    tw = (tc.tt << g.lbt) + (r >> (g.lby + g.lbz)) - g.toff;
+  };
+  uint32_t dirs = 0u;
+  {
+    int tw, z, y;
+    coords(tid, tw, z, y);
+    uint2 e = make_uint2(0u, 0u);
+    if (y < g.ny && z < g.nz && tw >= 0 && tw < g.tw)
+      e = ld_seg<CG>(a.seg + seg_index(g, tw, z, y, tc.xs));
+    S.mask[tid] = e.x;
+    S.rb[tid] = e.y;
+    if (e.x) {
+      if (SPATIAL) {
+        const uint32_t ys = (y > 0 ? 1u : 0u) | 2u | (y + 1 < g.ny ? 4u : 0u);
+        if ((e.x & 1u) && tc.xs > 0)
+          dirs = (z > 0 ? ys : 0u) | ys << 3 | (z + 1 < g.nz ? ys << 6 : 0u);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {  // dy -1, -1, 0, 1; dz 0, -1, -1, -1
+          const int y2 = y + (k == 3) - (k < 2), z2 = z - (k > 0);
+          if (y2 >= 0 && y2 < g.ny && z2 >= 0 &&
+              ((y2 >> g.lby) != (y >> g.lby) || (z2 >> g.lbz) != (z >> g.lbz)))
+            dirs |= 1u << (9 + k);
+        }
+      }
+      if ((a.edges & MSF_EDGE_TEMPORAL) && tw > 0 && ((tw + g.toff) & ((1 << g.lbt) - 1)) == 0)
+        dirs |= 1u << 13;
+    }
+  }
+  int total;
+  int pos = block_exscan(__popc(dirs), S.warp, &total);
+  for (; dirs; dirs &= dirs - 1) S.task[pos++] = (uint16_t)(tid | (__ffs(dirs) - 1) << 8);
+  __syncthreads();
+  auto join = [&](uint32_t c0, uint32_t c1) {
+    if (c0 != c1 && pair_first_seen(S.set, c0, c1)) gunion(a.cparent, c0, c1);
+  };
+  for (int i = tid; i < total; i += 256) {
+    const int r = S.task[i] & 255, k = S.task[i] >> 8;
+    int tw, z, y;
+    coords(r, tw, z, y);
+    int xs = tc.xs;
+    if (k < 9) {
+      z += k / 3 - 1;
+      y += k % 3 - 1;
+      --xs;
+    } else if (k < 13) {
+      y += (k == 12) - (k < 11);
+      z -= k > 9;
+    } else {
+      --tw;
+    }
+    const uint2 e2 = ld_seg<CG>(a.seg + seg_index(g, tw, z, y, xs));
+    const uint32_t m = S.mask[r], rb = S.rb[r], m2 = e2.x;
+    if (k < 9) {
+      if (m2 >> 31)
+        join(ld_seg<CG>(a.runcomp + rb),
+             ld_seg<CG>(a.runcomp + e2.y + __popc(run_starts(m2, SPATIAL)) - 1));
+    } else if (m2) {
+      const uint32_t st = run_starts(m, SPATIAL), st2 = run_starts(m2, SPATIAL);
+      row_contacts(m, m2, k < 13, SPATIAL, [&](int x1, int x2) {
+        join(ld_seg<CG>(a.runcomp + rb + run_index(st, x1)),
+             ld_seg<CG>(a.runcomp + e2.y + run_index(st2, x2)));
+      });
+    }
+  }
 }
 
 // one CTA per tile
 template <bool SPATIAL>
 __global__ void __launch_bounds__(256, 4) k_hook(const __grid_constant__ SegArgs a) {
-  __shared__ unsigned long long s_set[kHookSet];
+  __shared__ __align__(16) HookSmem s_hook;
   if (__ldg(&a.tileinfo[blockIdx.x].x) == 0) return;  // no member in the tile
-  for (int i = threadIdx.x; i < kHookSet; i += 256) s_set[i] = ~0ull;
-  __syncthreads();
-  hook_tile<SPATIAL>(a, blockIdx.x, s_set);
+  hook_tile<SPATIAL>(a, blockIdx.x, s_hook);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -881,20 +896,18 @@ template <bool SPATIAL>
 __global__ void __launch_bounds__(256, 4) k_joins(const __grid_constant__ SegArgs a,
                                                   const __grid_constant__ RecView rv, int nhook,
                                                   int nx) {
-  __shared__ __align__(16) unsigned long long s_mem[kHookSet];
-  static_assert(sizeof(uint2) * 8 * kRecBuf <= sizeof(s_mem), "the record buffers fit");
+  __shared__ __align__(16) HookSmem s_hook;
+  static_assert(sizeof(uint2) * 8 * kRecBuf <= sizeof(s_hook), "the record buffers fit");
   if ((int)blockIdx.x < nhook) {
     if (__ldg(&a.tileinfo[blockIdx.x].x) == 0) return;  // no member in the tile
-    for (int i = threadIdx.x; i < kHookSet; i += 256) s_mem[i] = ~0ull;
-    __syncthreads();
-    hook_tile<SPATIAL>(a, blockIdx.x, s_mem);
+    hook_tile<SPATIAL>(a, blockIdx.x, s_hook);
     return;
   }
   const int i = (int)blockIdx.x - nhook, tw = i / nx;
   uint32_t b0, b1;
   if (!rec_block(rv, a.g.t0 + tw, (uint32_t)(i - tw * nx), b0, b1)) return;
   links_rec_range<SPATIAL>(a, rv, tw, b0, b1,
-                           reinterpret_cast<uint2*>(s_mem) + kRecBuf * (threadIdx.x >> 5));
+                           reinterpret_cast<uint2*>(&s_hook) + kRecBuf * (threadIdx.x >> 5));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -2250,15 +2263,13 @@ __global__ void __launch_bounds__(256) k_mask_batch(const __grid_constant__ Batc
 // (tile, query) = (blockIdx.x, blockIdx.y): the tile's cross-face joins with its pair set
 template <bool SPATIAL>
 __global__ void __launch_bounds__(256, 4) k_hook_batch(const __grid_constant__ BatchPlan b) {
-  __shared__ unsigned long long s_set[kHookSet];
+  __shared__ __align__(16) HookSmem s_hook;
   __shared__ __align__(16) SegArgs s_args;
   load_args(&s_args, b.qargs + blockIdx.y);
   __syncthreads();
   if ((int)blockIdx.x >= s_args.g.ntiles) return;  // block-uniform
   if (__ldg(&s_args.tileinfo[blockIdx.x].x) == 0) return;  // no member in the tile
-  for (int i = threadIdx.x; i < kHookSet; i += 256) s_set[i] = ~0ull;
-  __syncthreads();
-  hook_tile<SPATIAL>(s_args, blockIdx.x, s_set);
+  hook_tile<SPATIAL>(s_args, blockIdx.x, s_hook);
 }
 
 // (point block, chunk item) = (blockIdx.x, row0 + blockIdx.y); chunk items in absolute point
@@ -2427,10 +2438,7 @@ __global__ void __launch_bounds__(256, 4) k_batch_fused(const __grid_constant__ 
       const int64_t p = (int64_t)pb * kFusedPoints + threadIdx.x;
       if (p < s_args.P) links_chunk<SPATIAL, true>(s_args, p, c * kLinkSteps);
     } else if (type == kFHook) {
-      unsigned long long* s_set = reinterpret_cast<unsigned long long*>(s_dyn);
-      for (int i = threadIdx.x; i < kHookSet; i += 256) s_set[i] = ~0ull;
-      __syncthreads();
-      hook_tile<SPATIAL, true>(s_args, (int)idx, s_set);
+      hook_tile<SPATIAL, true>(s_args, (int)idx, *reinterpret_cast<HookSmem*>(s_dyn));
     } else if (type == kFFlat) {
       flatten_body(s_args, (int)idx, &s_n);
     } else {
@@ -2447,7 +2455,7 @@ __global__ void __launch_bounds__(256, 4) k_batch_fused(const __grid_constant__ 
 template <bool SP>
 static constexpr size_t fused_dyn_smem() {
   const size_t tile = tile_dyn_smem<SP>();
-  const size_t hook = sizeof(unsigned long long) * kHookSet;
+  const size_t hook = sizeof(HookSmem);
   const size_t fin = sizeof(int32_t) * kSegPerTile * (SP ? 16 : 32);
   return std::max(tile, std::max(hook, fin));
 }
