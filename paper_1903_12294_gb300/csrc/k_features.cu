@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(256) k_pts(const __grid_constant__ FeatArgs a)
     }
   }
   const float* attr = a.attr + j * a.A * a.P + p;
-  accumulate_samples_hot<MSF_MAX_ATTR>(a.acc, s_hot[threadIdx.x >> 5], fid >= 0, fid,
+  accumulate_samples_hot(a.acc, s_hot[threadIdx.x >> 5], fid >= 0, fid,
                                        [&](int i) { return __ldg(attr + i * a.P); });
   __syncthreads();
   hot_merge(a.acc, s_hot);

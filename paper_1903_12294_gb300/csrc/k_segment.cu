@@ -1839,9 +1839,14 @@ constexpr size_t feat_vox_smem() {
 // samples of the window's field steps, grouped by (field step, bucket of consecutive voxels),
 // each with its voxel and its attributes side by side. Members are packed as for the joins; 32
 // of them lie in one bucket or a few (a few rows of the grid), so their component lookups hit
-// cached rows, and they mostly share one feature (the butterfly path of reduce_samples). The
-// samples are those of every point step falling in the window's field steps that binning placed
-// inside the grid: the same as the per-point pass takes. Block (x, y) takes records
+// cached rows, and they mostly share one feature. A warp therefore has a feature of its own, the
+// last one that most of a round's samples belonged to: lanes whose sample belongs to it add to
+// sums of their own (an exact square and one fp64 addition per attribute), reduced when the
+// feature changes and committed once per block; only the other lanes go through reduce_samples,
+// whose groups take turns (8M particles x 24 steps, one feature with nine tenths of the members:
+// all groups through it 4.4 ms, now 3.4 ms). The samples are those of every point step falling in
+// the window's field steps that binning placed inside the grid: the same as the per-point pass
+// takes. Block (x, y) takes records
 // [x * chunk, (x + 1) * chunk) of window field step y.
 // RW: words of a record (4, 8 or 12, the first 2, 6 or 8 attributes).
 template <bool SPATIAL, int RW>
@@ -1850,17 +1855,43 @@ __device__ __forceinline__ void feat_points_block(const SegArgs& a, const FeatAc
                                                   const RecView& rv, const int tw, uint32_t x) {
   constexpr int AM = RW == 4 ? 2 : RW == 8 ? 6 : 8;
   __shared__ uint2 s_buf[8][kRecBuf];   // per warp: (voxel, record) of its members
-  __shared__ HotCache s_hot[8][kHotWays];
+  __shared__ HotCache s_hot[8][1];  // per warp: its feature and sums, for the block's commit
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   uint32_t b0, b1;
   if (!rec_block(rv, a.g.t0 + tw, x, b0, b1)) return;  // block-uniform
-  hot_clear(s_hot[w]);
+  if (lane == 0) s_hot[w][0].fid = -1;
   const uint32_t step0 = step_seg0(a.g, tw);
+  int32_t own = -1;  // the warp's feature and the lane's sums for it
+  long long q1[AM];
+  double q2[AM];
+#pragma unroll
+  for (int j = 0; j < AM; ++j) {
+    q1[j] = 0;
+    q2[j] = 0.0;
+  }
+  auto give = [&] {  // the warp's sums for its feature into its cache; empty afterwards
+    HotCache& c = s_hot[w][0];
+#pragma unroll
+    for (int j = 0; j < AM; ++j) {
+      if (j >= acc.A) break;
+      const unsigned long long t = limb_sum(0xFFFFFFFFu, (unsigned long long)q1[j]);
+#pragma unroll
+      for (int o = 16; o; o >>= 1) q2[j] += __shfl_xor_sync(0xFFFFFFFFu, q2[j], o);
+      if (lane == 0) {
+        c.sq[j] = t;
+        c.s2[j] = q2[j];
+      }
+      q1[j] = 0;
+      q2[j] = 0.0;
+    }
+    if (lane == 0) c.fid = own;
+    __syncwarp();
+  };
   auto take = [&](bool ok, uint2 e) {  // 32 members (fewer at the end)
-    int64_t fid = -1;
+    int32_t fid = -1;
+    const float* p = rv.rec + (size_t)e.y * RW;
     float v[AM] = {};
     if (ok) {
-      const float* p = rv.rec + (size_t)e.y * RW;
 #pragma unroll
       for (int q = 0; q < AM; q += 2) {
         const float2 x = __ldg(reinterpret_cast<const float2*>(p + q));
@@ -1868,8 +1899,42 @@ __device__ __forceinline__ void feat_points_block(const SegArgs& a, const FeatAc
       }
       fid = __ldg(cfid + comp_of<SPATIAL>(a, tw, (int32_t)e.x));
     }
-    accumulate_samples_hot<AM>(acc, s_hot[w], ok, fid, [&](int j) { return v[j]; });
-    __syncwarp();  // the cached sums one reduction at a time
+    const unsigned act = __ballot_sync(0xFFFFFFFFu, ok);
+    if (!act) return;
+    unsigned mine = __ballot_sync(0xFFFFFFFFu, ok && fid == own);
+    if (__popc(mine) < 8) {  // does another feature have most of the round?
+      const int32_t f = __shfl_sync(0xFFFFFFFFu, fid, __fns(act, 0, (__popc(act) + 1) / 2));
+      const unsigned m = __ballot_sync(0xFFFFFFFFu, ok && fid == f);
+      if (__popc(m) >= 24) {
+        if (own >= 0) {
+          give();
+          if (lane == 0) hot_commit(acc, s_hot[w][0]);
+          __syncwarp();
+        }
+        own = f;
+        mine = m;
+      }
+    }
+    if (ok && fid == own) {
+#pragma unroll
+      for (int j = 0; j < AM; ++j) {
+        if (j >= acc.A) break;
+        const double x = f2d(isfinite(v[j]) ? v[j] : 0.f);
+        q1[j] += quantise(v[j], acc.kscale[j]);
+        q2[j] = __fma_rn(x, x, q2[j]);
+      }
+    }
+    if (act & ~mine)
+      reduce_samples(
+          acc, ok && fid != own, fid, [&](int j) { return __ldg(p + j); },
+          [&](int64_t f, int j, unsigned long long qs, float h, float l, double wd, bool dbl, bool) {
+            const int64_t i = ((int64_t)(blockIdx.x & (acc.K - 1)) * acc.F + f) * acc.A + j;
+            atomicAdd(acc.sq + i, qs);
+            if (dbl) atomicAdd(acc.sa2 + i, wd);
+            else add_pair(acc.sa2 + i, h, l);
+          },
+          mine == 0u);
+    __syncwarp();
   };
   int n = 0;
   for (uint32_t base = b0 + 32u * kRecPer * w; base < b1; base += 256u * kRecPer) {
@@ -1900,6 +1965,7 @@ __device__ __forceinline__ void feat_points_block(const SegArgs& a, const FeatAc
     __syncwarp();
   }
   take(lane < n, lane < n ? s_buf[w][lane] : make_uint2(0u, b0));
+  if (own >= 0) give();
   __syncthreads();
   hot_merge(acc, s_hot);
 }

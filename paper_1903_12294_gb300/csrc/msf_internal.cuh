@@ -831,10 +831,12 @@ __device__ __forceinline__ unsigned long long limb_sum(unsigned m, unsigned long
 // squares), and one lane per feature hands the sums to sink(f, j, qs, h, l, w, dbl, one): the sum
 // of squares is h + l (a double-float pair, each exact in fp32), or w in fp64 when dbl is set
 // (non-finite or extreme values, rare); one is set when all the warp's samples belong to f (the
-// call then has a single leader). AMAX: most attributes. All 32 lanes must call this.
-template <int AMAX, class Val, class Sink>
+// call then has a single leader). alone: the samples are all the warp's (else the call never
+// takes the whole-warp path). All 32 lanes must call this. The attributes are a loop: unrolled,
+// the code of both paths no longer fits the instruction cache, and the warps wait for it.
+template <class Val, class Sink>
 __device__ __forceinline__ void reduce_samples(const FeatAcc& acc, bool ok, int64_t fid, Val&& val,
-                                               Sink&& sink) {
+                                               Sink&& sink, bool alone = true) {
   const unsigned act = __ballot_sync(0xFFFFFFFFu, ok);
   if (!act) return;
   const int lane = threadIdx.x & 31;
@@ -842,10 +844,9 @@ __device__ __forceinline__ void reduce_samples(const FeatAcc& acc, bool ok, int6
   // The whole warp then reduces by butterfly (lanes without a sample add zeros).
   const int first = __ffs(act) - 1;
   const int64_t f0 = __shfl_sync(0xFFFFFFFFu, fid, first);
-  if (__all_sync(0xFFFFFFFFu, !ok || fid == f0)) {
-#pragma unroll
-    for (int j = 0; j < AMAX; ++j) {
-      if (j >= acc.A) break;
+  if (alone && __all_sync(0xFFFFFFFFu, !ok || fid == f0)) {
+#pragma unroll 1
+    for (int j = 0; j < acc.A; ++j) {
       const float v = ok ? val(j) : 0.f;
       const unsigned long long u = ok ? (unsigned long long)quantise(v, acc.kscale[j]) : 0ull;
       // exact 64-bit sum (mod 2^64) from three lane reductions of 21/21/22-bit parts
@@ -888,9 +889,8 @@ __device__ __forceinline__ void reduce_samples(const FeatAcc& acc, bool ok, int6
   // 2^-52 of the largest drop out, well inside the sums' fp64-level tolerance.
   const unsigned grp = __match_any_sync(act, fid);
   const int leader = __ffs(grp) - 1;
-#pragma unroll
-  for (int j = 0; j < AMAX; ++j) {
-    if (j >= acc.A) break;
+#pragma unroll 1
+  for (int j = 0; j < acc.A; ++j) {
     const float v = val(j);
     const unsigned long long u = (unsigned long long)quantise(v, acc.kscale[j]);
     const unsigned long long qs = limb_sum(grp, u);
@@ -970,10 +970,10 @@ __device__ __forceinline__ void hot_commit(const FeatAcc& acc, HotCache& c) {
 // reduce_samples committing through the warp's caches. A call whose samples all belong to one
 // other feature commits the cached feature of its way and caches that one instead: samples walked
 // in voxel order come in runs of one feature, and the run at hand is the one worth caching.
-template <int AMAX, class Val>
+template <class Val>
 __device__ __forceinline__ void accumulate_samples_hot(const FeatAcc& acc, HotCache (&cs)[kHotWays],
                                                        bool ok, int64_t fid, Val&& val) {
-  reduce_samples<AMAX>(acc, ok, fid, val,
+  reduce_samples(acc, ok, fid, val,
                  [&](int64_t f, int j, unsigned long long qs, float h, float l, double w,
                      bool dbl, bool one) {
                    HotCache& c = cs[(((uint32_t)f * 0x9E3779B1u) >> 16) & (kHotWays - 1)];
@@ -1000,8 +1000,9 @@ __device__ __forceinline__ void accumulate_samples_hot(const FeatAcc& acc, HotCa
 
 // The caches of a block's 8 warps into the accumulators, a feature's sums over the warps committed
 // once. All threads, after a barrier.
-__device__ __forceinline__ void hot_merge(const FeatAcc& acc, HotCache (&h)[8][kHotWays]) {
-  for (int i = threadIdx.x; i < kHotWays * 8 * acc.A; i += blockDim.x) {
+template <int WAYS>
+__device__ __forceinline__ void hot_merge(const FeatAcc& acc, HotCache (&h)[8][WAYS]) {
+  for (int i = threadIdx.x; i < WAYS * 8 * acc.A; i += blockDim.x) {
     const int j = i % acc.A, w = i / acc.A % 8, e = i / (8 * acc.A);
     const long long f = h[w][e].fid;
     bool first = f >= 0;
