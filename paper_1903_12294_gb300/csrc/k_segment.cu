@@ -1842,9 +1842,10 @@ constexpr size_t feat_vox_smem() {
 // cached rows, and they mostly share one feature. A warp therefore has a feature of its own, the
 // last one that most of a round's samples belonged to: lanes whose sample belongs to it add to
 // sums of their own (an exact square and one fp64 addition per attribute), reduced when the
-// feature changes and committed once per block; only the other lanes go through reduce_samples,
-// whose groups take turns (8M particles x 24 steps, one feature with nine tenths of the members:
-// all groups through it 4.4 ms, now 3.4 ms). The samples are those of every point step falling in
+// feature changes and committed once per block. The other members wait in a list until there are
+// 32 of them for reduce_samples, whose instructions a few of them cost as many as 32 do (8M
+// particles x 24 steps, one feature with nine tenths of the members: all members through it
+// 4.4 ms, every round's others at once 3.4 ms, now 2.9 ms). The samples are those of every point step falling in
 // the window's field steps that binning placed inside the grid: the same as the per-point pass
 // takes. Block (x, y) takes records
 // [x * chunk, (x + 1) * chunk) of window field step y.
@@ -1855,6 +1856,7 @@ __device__ __forceinline__ void feat_points_block(const SegArgs& a, const FeatAc
                                                   const RecView& rv, const int tw, uint32_t x) {
   constexpr int AM = RW == 4 ? 2 : RW == 8 ? 6 : 8;
   __shared__ uint2 s_buf[8][kRecBuf];   // per warp: (voxel, record) of its members
+  __shared__ uint2 s_left[8][64];       // per warp: (feature, record) of those not of its own
   __shared__ HotCache s_hot[8][1];  // per warp: its feature and sums, for the block's commit
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   uint32_t b0, b1;
@@ -1887,11 +1889,13 @@ __device__ __forceinline__ void feat_points_block(const SegArgs& a, const FeatAc
     if (lane == 0) c.fid = own;
     __syncwarp();
   };
+  const unsigned below = (1u << lane) - 1u;
+  int nl = 0;  // members in s_left
   auto take = [&](bool ok, uint2 e) {  // 32 members (fewer at the end)
     int32_t fid = -1;
-    const float* p = rv.rec + (size_t)e.y * RW;
     float v[AM] = {};
     if (ok) {
+      const float* p = rv.rec + (size_t)e.y * RW;
 #pragma unroll
       for (int q = 0; q < AM; q += 2) {
         const float2 x = __ldg(reinterpret_cast<const float2*>(p + q));
@@ -1900,9 +1904,8 @@ __device__ __forceinline__ void feat_points_block(const SegArgs& a, const FeatAc
       fid = __ldg(cfid + comp_of<SPATIAL>(a, tw, (int32_t)e.x));
     }
     const unsigned act = __ballot_sync(0xFFFFFFFFu, ok);
-    if (!act) return;
     unsigned mine = __ballot_sync(0xFFFFFFFFu, ok && fid == own);
-    if (__popc(mine) < 8) {  // does another feature have most of the round?
+    if (act && __popc(mine) < 8) {  // does another feature have most of the round?
       const int32_t f = __shfl_sync(0xFFFFFFFFu, fid, __fns(act, 0, (__popc(act) + 1) / 2));
       const unsigned m = __ballot_sync(0xFFFFFFFFu, ok && fid == f);
       if (__popc(m) >= 24) {
@@ -1924,47 +1927,64 @@ __device__ __forceinline__ void feat_points_block(const SegArgs& a, const FeatAc
         q2[j] = __fma_rn(x, x, q2[j]);
       }
     }
-    if (act & ~mine)
-      reduce_samples(
-          acc, ok && fid != own, fid, [&](int j) { return __ldg(p + j); },
-          [&](int64_t f, int j, unsigned long long qs, float h, float l, double wd, bool dbl, bool) {
-            const int64_t i = ((int64_t)(blockIdx.x & (acc.K - 1)) * acc.F + f) * acc.A + j;
-            atomicAdd(acc.sq + i, qs);
-            if (dbl) atomicAdd(acc.sa2 + i, wd);
-            else add_pair(acc.sa2 + i, h, l);
-          },
-          mine == 0u);
+    const unsigned left = act & ~mine;
+    if (ok && fid != own) s_left[w][nl + __popc(left & below)] = make_uint2((uint32_t)fid, e.y);
+    nl += __popc(left);
+    __syncwarp();
+  };
+  auto take_left = [&] {  // the first 32 of s_left
+    const bool ok = lane < nl;
+    const uint2 e = ok ? s_left[w][lane] : make_uint2(0u, 0u);
+    const uint2 rest = 32 + lane < nl ? s_left[w][32 + lane] : make_uint2(0u, 0u);
+    __syncwarp();
+    if (32 + lane < nl) s_left[w][lane] = rest;
+    nl = max(nl - 32, 0);
+    const float* p = rv.rec + (size_t)e.y * RW;
+    reduce_samples(
+        acc, ok, (int64_t)(int32_t)e.x, [&](int j) { return __ldg(p + j); },
+        [&](int64_t f, int j, unsigned long long qs, float h, float l, double wd, bool dbl, bool) {
+          const int64_t i = ((int64_t)(blockIdx.x & (acc.K - 1)) * acc.F + f) * acc.A + j;
+          atomicAdd(acc.sq + i, qs);
+          if (dbl) atomicAdd(acc.sa2 + i, wd);
+          else add_pair(acc.sa2 + i, h, l);
+        });
     __syncwarp();
   };
   int n = 0;
-  for (uint32_t base = b0 + 32u * kRecPer * w; base < b1; base += 256u * kRecPer) {
-    uint32_t v[kRecPer];
-    bool ok[kRecPer];
+  for (uint32_t base = b0 + 32u * kRecPer * w;; base += 256u * kRecPer) {
+    const bool more = base < b1;  // else the remainders
+    if (more) {
+      uint32_t v[kRecPer];
+      bool ok[kRecPer];
 #pragma unroll
-    for (int u = 0; u < kRecPer; ++u) {
-      const uint32_t r = base + 32u * u + lane;
-      v[u] = r < b1 ? __ldcs(&rv.rec_vn[r].x) : 0xFFFFFFFFu;
+      for (int u = 0; u < kRecPer; ++u) {
+        const uint32_t r = base + 32u * u + lane;
+        v[u] = r < b1 ? __ldcs(&rv.rec_vn[r].x) : 0xFFFFFFFFu;
+      }
+#pragma unroll
+      for (int u = 0; u < kRecPer; ++u) ok[u] = v[u] != 0xFFFFFFFFu && is_member(a, step0, v[u]);
+#pragma unroll
+      for (int u = 0; u < kRecPer; ++u) {
+        const unsigned b = __ballot_sync(0xFFFFFFFFu, ok[u]);
+        if (ok[u]) s_buf[w][n + __popc(b & below)] = make_uint2(v[u], base + 32u * u + lane);
+        n += __popc(b);
+      }
+      __syncwarp();
     }
-#pragma unroll
-    for (int u = 0; u < kRecPer; ++u) ok[u] = v[u] != 0xFFFFFFFFu && is_member(a, step0, v[u]);
-#pragma unroll
-    for (int u = 0; u < kRecPer; ++u) {
-      const unsigned b = __ballot_sync(0xFFFFFFFFu, ok[u]);
-      if (ok[u])
-        s_buf[w][n + __popc(b & ((1u << lane) - 1u))] = make_uint2(v[u], base + 32u * u + lane);
-      n += __popc(b);
-    }
-    __syncwarp();
     // oldest first: the buffer's members in record order keep runs of one feature together
     int i0 = 0;
-    for (; i0 + 32 <= n; i0 += 32) take(true, s_buf[w][i0 + lane]);
+    for (; more ? i0 + 32 <= n : i0 < n || nl; i0 += 32) {
+      const bool ok = i0 + lane < n;
+      take(ok, ok ? s_buf[w][i0 + lane] : make_uint2(0u, b0));
+      if (nl >= 32 || (!more && i0 + 32 >= n && nl)) take_left();
+    }
+    if (!more) break;
     n -= i0;
     const uint2 rest = lane < n ? s_buf[w][i0 + lane] : make_uint2(0u, 0u);
     __syncwarp();
     if (i0 && lane < n) s_buf[w][lane] = rest;  // the remainder to the front
     __syncwarp();
   }
-  take(lane < n, lane < n ? s_buf[w][lane] : make_uint2(0u, b0));
   if (own >= 0) give();
   __syncthreads();
   hot_merge(acc, s_hot);

@@ -831,12 +831,11 @@ __device__ __forceinline__ unsigned long long limb_sum(unsigned m, unsigned long
 // squares), and one lane per feature hands the sums to sink(f, j, qs, h, l, w, dbl, one): the sum
 // of squares is h + l (a double-float pair, each exact in fp32), or w in fp64 when dbl is set
 // (non-finite or extreme values, rare); one is set when all the warp's samples belong to f (the
-// call then has a single leader). alone: the samples are all the warp's (else the call never
-// takes the whole-warp path). All 32 lanes must call this. The attributes are a loop: unrolled,
-// the code of both paths no longer fits the instruction cache, and the warps wait for it.
+// call then has a single leader). All 32 lanes must call this. The attributes are a loop:
+// unrolled, the code of both paths no longer fits the instruction cache, and the warps wait for it.
 template <class Val, class Sink>
 __device__ __forceinline__ void reduce_samples(const FeatAcc& acc, bool ok, int64_t fid, Val&& val,
-                                               Sink&& sink, bool alone = true) {
+                                               Sink&& sink) {
   const unsigned act = __ballot_sync(0xFFFFFFFFu, ok);
   if (!act) return;
   const int lane = threadIdx.x & 31;
@@ -844,7 +843,7 @@ __device__ __forceinline__ void reduce_samples(const FeatAcc& acc, bool ok, int6
   // The whole warp then reduces by butterfly (lanes without a sample add zeros).
   const int first = __ffs(act) - 1;
   const int64_t f0 = __shfl_sync(0xFFFFFFFFu, fid, first);
-  if (alone && __all_sync(0xFFFFFFFFu, !ok || fid == f0)) {
+  if (__all_sync(0xFFFFFFFFu, !ok || fid == f0)) {
 #pragma unroll 1
     for (int j = 0; j < acc.A; ++j) {
       const float v = ok ? val(j) : 0.f;
