@@ -39,6 +39,14 @@ namespace msf {
 int scan_exclusive_u32(msf_ctx* ctx, const uint32_t* in, uint32_t* out, int64_t n, DevBuf& tmp,
                        uint32_t* total);
 
+// How the approximate scan forms a distance: sqrt(k2 * (dx^2 + dy^2 + dz^2) + kt * dt^2) + |dv|,
+// the distance divided by the value's weight (values == false, a zero weight: |dv| is left out and
+// nothing divided). ok == false: the weights are outside what its error bound covers.
+struct ScanScale {
+  float k2, kt, slack;
+  bool ok, values;
+};
+
 struct SlicArgs {
   int nx, ny, nz, T, A;
   int64_t V, P;
@@ -73,7 +81,8 @@ struct SlicArgs {
   float* ptime;                 // [slots] its time
   uint32_t* pindex;             // [slots] its index t * P + p in the window (t: point step)
   int sub[4], nsub;             // subcells of a cell along x, y, z, t, and their number
-  bool plain;                   // weights and sizes the pruned scan and the packed sums allow
+  bool plain;                   // sizes and scales the packed sums allow
+  ScanScale scan_f, scan_p;     // the approximate scan of the field and of the point samples
 };
 
 // Time of window point step t: with r point steps in field step f, the i-th (0-based) sits at
@@ -343,13 +352,16 @@ __global__ void __launch_bounds__(256, 4) k_slic_assign_field(const __grid_const
 // first by more than 4e-6 of it, the first is the answer; otherwise, and with weights or values
 // that the error bound does not cover, the lane scans the list again with the deciding
 // operations. 54 to 81 candidates in the deciding operations, an IEEE square root each, bounded
-// the passes by instruction issue.
+// the passes by instruction issue, and the scan still does: it divides the distance by the value's
+// weight (no multiplication after the root), lets the root flush denormals (an absolute error
+// that the slack of the comparison covers) and takes two steps or two centres per packed fp32
+// instruction.
 //
 // Sums: a sample adds to its centre's place in shared memory, and the block commits each place
 // once (adding up in the warp took a loop over the members of every group with 64-bit shuffles).
 //
 // 128^3 x 32 field and 1M x 32 point samples, 16,384 centres, ten assignments: field 68.2 -> 34.0
-// ms, points 60.2 -> 18.2 ms.
+// ms, points 60.2 -> 18.2 ms; in packed operations 18.1 -> 16.9 and 18.2 -> 16.2 ms.
 constexpr int kCand = 384;   // centres in a block's list; more: the per-sample lookup
 constexpr int kWCand = 96;   // centres in a warp's list; more: the warp scans the block's list
 
@@ -359,11 +371,12 @@ struct CandList {
   int id[kCand];
 };
 
-struct WarpList {
-  float4 pos[kWCand];  // x, y, z, t
+struct __align__(16) WarpList {    // two centres side by side
+  float xy[kWCand / 2][4], zt[kWCand / 2][4];  // x, x, y, y; z, z, t, t
   float val[kWCand];
   uint16_t q[kWCand];  // place in the block's list
 };
+static_assert(kWCand % 2 == 0, "the list is padded to pairs");
 
 // distance between u and the nearest point of [lo, hi], in the rounding of the region test
 __device__ __forceinline__ float box_dist(float u, float lo, float hi) {
@@ -371,9 +384,9 @@ __device__ __forceinline__ float box_dist(float u, float lo, float hi) {
 }
 
 // centre q of the block's list, when it reaches the box, into the warp's list; returns the
-// number listed (-1: too many). All lanes.
+// number listed (-1: too many; an odd list is padded with a centre out of reach). All lanes.
 __device__ __forceinline__ int warp_list(const SlicArgs& a, const CandList& c, int nc, WarpList& w,
-                                         const float (&lo)[4], const float (&hi)[4]) {
+                                         const float (&lo)[4], const float (&hi)[4], bool values) {
   const int lane = threadIdx.x & 31;
   int n = 0;
   for (int b = 0; b < nc; b += 32) {
@@ -390,10 +403,16 @@ __device__ __forceinline__ int warp_list(const SlicArgs& a, const CandList& c, i
     n += __popc(m);
     if (n > kWCand) return -1;  // warp-uniform
     if (in) {
-      w.pos[at] = p;
-      w.val[at] = c.val[q];
+      const int h = at >> 1, o = at & 1;
+      w.xy[h][o] = p.x, w.xy[h][2 + o] = p.y;
+      w.zt[h][o] = p.z, w.zt[h][2 + o] = p.w;
+      w.val[at] = values ? c.val[q] : __fmul_rn(0.f, c.val[q]);  // (a NaN stays one)
       w.q[at] = (uint16_t)q;
     }
+  }
+  if ((n & 1) && lane == 0) {
+    w.xy[n >> 1][1] = w.xy[n >> 1][3] = w.zt[n >> 1][1] = w.zt[n >> 1][3] = INFINITY;
+    w.val[n] = 0.f;
   }
   __syncwarp();
   return n;
@@ -424,37 +443,81 @@ __device__ __noinline__ int exact_best(const SlicArgs& a, const CandList& c, con
 
 __device__ __forceinline__ float sqrt_approx(float x) {
   float r;
-  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
 
+// two fp32 values in one 64-bit register pair: packed operations, each rounded as the single one
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// the two smallest so far (m1, m2) and the place of the smallest, with candidate i at distance e
+__device__ __forceinline__ void best_two(float e, int i, float& m1, float& m2, int& best) {
+  m2 = fminf(m2, fmaxf(m1, e));
+  best = e < m1 ? i : best;
+  m1 = fminf(m1, e);
+}
+
+// does the smallest approximate distance decide?
+__device__ __forceinline__ bool decided(const ScanScale& k, float m1, float m2) {
+  return m1 < 1e18f && m2 > fmaf(m1, 4e-6f, m1) + k.slack;
+}
+
 // the same by the approximate scan of the warp's list where that decides
-__device__ __forceinline__ int list_best(const SlicArgs& a, const CandList& c, const WarpList& w,
-                                         int n, int nc, float xs, float ys, float zs, float ts,
-                                         float wv, float vs) {
+__device__ __forceinline__ int list_best(const SlicArgs& a, const ScanScale& k, const CandList& c,
+                                         const WarpList& w, int n, int nc, float xs, float ys,
+                                         float zs, float ts, float wv, float vs) {
   if (n < 0) return exact_best(a, c, nullptr, nc, xs, ys, zs, ts, wv, vs);
-  if (!a.plain) return exact_best(a, c, w.q, n, xs, ys, zs, ts, wv, vs);
-  const float C0 = a.C[0], C1 = a.C[1], C2 = a.C[2], C3 = a.C[3], cf2 = a.c_f * a.c_f;
+  if (!k.ok) return exact_best(a, c, w.q, n, xs, ys, zs, ts, wv, vs);
+  const float C0 = a.C[0], C1 = a.C[1], C2 = a.C[2], C3 = a.C[3];
+  const f32x2 nx = pack2(-xs, -xs), ny = pack2(-ys, -ys), nz = pack2(-zs, -zs);
+  const f32x2 nt = pack2(-ts, -ts), nv = k.values ? pack2(-vs, -vs) : 0ull;
+  const f32x2 k2 = pack2(k.k2, k.k2), kt = pack2(k.kt, k.kt);
   float m1 = INFINITY, m2 = INFINITY;
   int best = -1;
-#pragma unroll 4
-  for (int i = 0; i < n; ++i) {
-    const float4 p = w.pos[i];
-    const float dx = __fsub_rn(p.x, xs), dy = __fsub_rn(p.y, ys), dz = __fsub_rn(p.z, zs);
-    const float dt = __fsub_rn(p.w, ts);
-    const bool in = fabsf(dx) <= C0 && fabsf(dy) <= C1 && fabsf(dz) <= C2 && fabsf(dt) <= C3;
-    const float s2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, cf2 * (dt * dt))));
-    const float d = fmaf(a.w_d, sqrt_approx(s2), wv * fabsf(vs - w.val[i]));
-    const float e = in ? d : INFINITY;
-    m2 = fminf(m2, fmaxf(m1, e));
-    best = e < m1 ? i : best;
-    m1 = fminf(m1, e);
+#pragma unroll 2
+  for (int i = 0; i < n; i += 2) {
+    const ulonglong2 xy = *reinterpret_cast<const ulonglong2*>(w.xy[i >> 1]);
+    const ulonglong2 zt = *reinterpret_cast<const ulonglong2*>(w.zt[i >> 1]);
+    const f32x2 v = *reinterpret_cast<const f32x2*>(w.val + i);
+    const f32x2 dx = add2(xy.x, nx), dy = add2(xy.y, ny), dz = add2(zt.x, nz), dt = add2(zt.y, nt);
+    const f32x2 s3 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
+    const float2 s = unpack2(fma2(mul2(dt, kt), dt, mul2(s3, k2)));
+    const float2 d = unpack2(add2(v, nv));
+    const float2 ux = unpack2(dx), uy = unpack2(dy), uz = unpack2(dz), ut = unpack2(dt);
+    const bool in0 = fabsf(ux.x) <= C0 && fabsf(uy.x) <= C1 && fabsf(uz.x) <= C2 && fabsf(ut.x) <= C3;
+    const bool in1 = fabsf(ux.y) <= C0 && fabsf(uy.y) <= C1 && fabsf(uz.y) <= C2 && fabsf(ut.y) <= C3;
+    const float e0 = in0 ? sqrt_approx(s.x) + fabsf(d.x) : INFINITY;
+    const float e1 = in1 ? sqrt_approx(s.y) + fabsf(d.y) : INFINITY;
+    best_two(e0, i, m1, m2, best);
+    best_two(e1, i + 1, m1, m2, best);
   }
-  if (best < 0 && m1 == INFINITY && m2 == INFINITY) {
-    // no centre in reach, or distances beyond fp32: the deciding scan tells
-    return exact_best(a, c, w.q, n, xs, ys, zs, ts, wv, vs);
-  }
-  if (m1 < 1e30f && m2 > fmaf(m1, 4e-6f, m1) + 1e-30f) return w.q[best];
+  // (no centre in reach, or distances too large: the deciding scan tells)
+  if (best >= 0 && decided(k, m1, m2)) return w.q[best];
   return exact_best(a, c, w.q, n, xs, ys, zs, ts, wv, vs);
 }
 
@@ -538,9 +601,9 @@ __device__ __forceinline__ void add64(uint32_t* p, unsigned long long v) {
 // the steps' sum (1024 samples: no counter exceeds 16 bits).
 constexpr int kFieldSteps = 4;
 
-struct FieldList {
-  float4 pv[kWCand];           // x, y, z, value
-  float dt[kWCand][kFieldSteps];  // c_f^2 (t - step)^2, or infinity
+struct __align__(16) FieldList {
+  float4 pv[kWCand];           // x, y, z, -value
+  float dt[kWCand][kFieldSteps];  // kt (t - step)^2, or infinity
   uint16_t q[kWCand];
 };
 
@@ -558,8 +621,8 @@ __global__ void __launch_bounds__(256, 4) k_slic_assign_field_tiled(const __grid
   const int64_t ntiles = (int64_t)ntx * nty * ntz * ntt;
   const int wx = (w % (TX / 8)) * 8, wy = (w / (TX / 8)) % (TY / 4) * 4;
   const int wz = w / ((TX / 8) * (TY / 4));
-  const float C0 = a.C[0], C1 = a.C[1], C2 = a.C[2], C3 = a.C[3], cf2 = a.c_f * a.c_f;
-  const float wd = fmaxf(a.w_d, 1e-37f);  // times infinity is infinity, with w_d = 0 too
+  const float C0 = a.C[0], C1 = a.C[1], C2 = a.C[2], C3 = a.C[3];
+  const ScanScale& k = a.scan_f;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     int64_t r = tile;
     const int bx = (int)(r % ntx); r /= ntx;
@@ -612,11 +675,12 @@ __global__ void __launch_bounds__(256, 4) k_slic_assign_field_tiled(const __grid
         break;
       }
       if (in) {
-        L.pv[at] = make_float4(p.x, p.y, p.z, s_c.val[q]);
+        const float v = s_c.val[q];
+        L.pv[at] = make_float4(p.x, p.y, p.z, k.values ? -v : __fmul_rn(0.f, v));  // (NaN stays)
 #pragma unroll
         for (int s = 0; s < S; ++s) {
           const float dt = __fsub_rn(p.w, step_time(s));
-          L.dt[at][s] = fabsf(dt) <= C3 ? cf2 * (dt * dt) : INFINITY;
+          L.dt[at][s] = fabsf(dt) <= C3 ? k.kt * (dt * dt) : INFINITY;
         }
         L.q[at] = (uint16_t)q;
       }
@@ -634,19 +698,23 @@ __global__ void __launch_bounds__(256, 4) k_slic_assign_field_tiled(const __grid
         m1[s] = m2[s] = INFINITY;
         best[s] = -1;
       }
-      if (n >= 0 && a.plain) {
+      if (n >= 0 && k.ok) {
+        f32x2 ff[S / 2];
+#pragma unroll
+        for (int s = 0; s < S; s += 2) ff[s / 2] = k.values ? pack2(f[s], f[s + 1]) : 0ull;
 #pragma unroll 2
         for (int i = 0; i < n; ++i) {
           const float4 p = L.pv[i];
           const float dx = __fsub_rn(p.x, xs), dy = __fsub_rn(p.y, ys), dz = __fsub_rn(p.z, zs);
           const bool in = fabsf(dx) <= C0 && fabsf(dy) <= C1 && fabsf(dz) <= C2;
-          const float s3 = in ? fmaf(dx, dx, fmaf(dy, dy, dz * dz)) : INFINITY;
+          const float s3 = in ? k.k2 * fmaf(dx, dx, fmaf(dy, dy, dz * dz)) : INFINITY;
+          const f32x2 ss = pack2(s3, s3), vv = pack2(p.w, p.w);
 #pragma unroll
-          for (int s = 0; s < S; ++s) {
-            const float e = fmaf(wd, sqrt_approx(s3 + L.dt[i][s]), a.w_f * fabsf(f[s] - p.w));
-            m2[s] = fminf(m2[s], fmaxf(m1[s], e));
-            best[s] = e < m1[s] ? i : best[s];
-            m1[s] = fminf(m1[s], e);
+          for (int s = 0; s < S; s += 2) {
+            const float2 s4 = unpack2(add2(ss, *reinterpret_cast<const f32x2*>(&L.dt[i][s])));
+            const float2 d = unpack2(add2(ff[s / 2], vv));
+            best_two(sqrt_approx(s4.x) + fabsf(d.x), i, m1[s], m2[s], best[s]);
+            best_two(sqrt_approx(s4.y) + fabsf(d.y), i, m1[s + 1], m2[s + 1], best[s + 1]);
           }
         }
       }
@@ -659,7 +727,7 @@ __global__ void __launch_bounds__(256, 4) k_slic_assign_field_tiled(const __grid
           q = -1;
           c = best_centre(a, xs, ys, zs, ts, a.w_f, f[s], 5);
         } else {
-          if (best[s] >= 0 && m1[s] < 1e30f && m2[s] > fmaf(m1[s], 4e-6f, m1[s]) + 1e-30f)
+          if (best[s] >= 0 && decided(k, m1[s], m2[s]))
             q = L.q[best[s]];
           else
             q = exact_best(a, s_c, n >= 0 ? L.q : nullptr, n >= 0 ? n : nc, xs, ys, zs, ts, a.w_f,
@@ -843,13 +911,13 @@ __global__ void __launch_bounds__(256, 4) k_slic_assign_points_cells(const __gri
           blo[q] = __uint_as_float(__reduce_min_sync(0xFFFFFFFFu, __float_as_uint(u[q])));
           bhi[q] = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(u[q])));
         }
-        n = warp_list(a, s_c, nc, s_w[w], blo, bhi);
+        n = warp_list(a, s_c, nc, s_w[w], blo, bhi, a.scan_p.values);
       }
       if (take) {
         const uint32_t li = a.pindex[slot];
         int q = -1, best;
         if (nc >= 0) {
-          q = list_best(a, s_c, s_w[w], n, nc, sm.x, sm.y, sm.z, ts, a.w_p, sm.w);
+          q = list_best(a, a.scan_p, s_c, s_w[w], n, nc, sm.x, sm.y, sm.z, ts, a.w_p, sm.w);
           best = q >= 0 ? s_c.id[q] : -1;
         } else {
           best = best_centre(a, sm.x, sm.y, sm.z, ts, a.w_p, sm.w, VS);
@@ -1043,10 +1111,26 @@ int cluster_run(msf_ctx* ctx, const msf_cluster_params* prm, int32_t* flabel, in
   const unsigned gp = (unsigned)std::max<int64_t>(1, std::min<int64_t>((nps + 255) / 256,
                                                                        (int64_t)ctx->sm_count * 32));
   const unsigned gt = (unsigned)ctx->sm_count * 8;  // tiled field pass: persistent blocks
-  // The approximate scan's error bound wants weights that add up and values far from overflow;
-  // the packed coordinate sums want voxel centres and their scale to be exact in fp32.
-  a.plain = a.w_p >= 0.f && a.w_f >= 0.f && a.w_d >= 0.f && a.kpos >= 1 &&
-            std::max(std::max(d.nx, d.T), std::max(d.ny, d.nz)) <= (1 << 22);
+  // The approximate scan's error bound wants weights that add up and are not far apart, and
+  // distances far from overflow (1e18 and less decide: a squared term that overflows belongs to a
+  // larger one). Absolute errors: a root below 2^-63 may be taken as zero, and the deciding
+  // operations may lose products to underflow. The packed coordinate sums want voxel centres and
+  // their scale to be exact in fp32.
+  const bool small = std::max(std::max(d.nx, d.T), std::max(d.ny, d.nz)) <= (1 << 22);
+  a.plain = a.kpos >= 1 && small;
+  auto scan_scale = [&](float wv) {
+    const double k = wv > 0.f ? (double)a.w_d / wv : (double)a.w_d;
+    ScanScale r;
+    r.k2 = (float)(k * k);
+    r.kt = (float)(k * k * ((double)a.c_f * a.c_f));
+    r.slack = 1e-18f + (wv > 0.f ? 1e-30f / wv : 0.f);
+    r.values = wv > 0.f;
+    r.ok = small && a.w_d >= 0.f && (wv == 0.f || (wv >= 1e-9f && wv <= 1e9f)) &&
+           (k == 0.0 || (k >= 1e-9 && k <= 1e9)) && (double)r.kt <= 1e30;
+    return r;
+  };
+  a.scan_f = scan_scale(a.w_f);
+  a.scan_p = scan_scale(a.w_p);
   k_slic_seed<<<kb, 256, 0, s>>>(a);
   {
     ScopedKernel k(ctx, "k_slic_assign_field");
