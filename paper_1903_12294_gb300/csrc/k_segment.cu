@@ -1860,7 +1860,7 @@ constexpr size_t feat_vox_smem() {
 // feature changes and committed once per block. The other members wait in a list until there are
 // 32 of them for reduce_samples, whose instructions a few of them cost as many as 32 do (8M
 // particles x 24 steps, one feature with nine tenths of the members: all members through it
-// 4.4 ms, every round's others at once 3.4 ms, now 2.9 ms). The samples are those of every point step falling in
+// 4.4 ms, every round's others at once 3.4 ms, a full round of them 2.9 ms, their groups chained 2.2 ms). The samples are those of every point step falling in
 // the window's field steps that binning placed inside the grid: the same as the per-point pass
 // takes. Block (x, y) takes records
 // [x * chunk, (x + 1) * chunk) of window field step y.
@@ -2006,7 +2006,7 @@ __device__ __forceinline__ void feat_points_block(const SegArgs& a, const FeatAc
 }
 
 template <bool SPATIAL, int RW>
-__global__ void __launch_bounds__(256) k_feat_points_rec(const __grid_constant__ SegArgs a,
+__global__ void __launch_bounds__(256, RW == 12 ? 3 : 4) k_feat_points_rec(const __grid_constant__ SegArgs a,
                                                          FeatAcc acc,
                                                          const int32_t* __restrict__ cfid,
                                                          const __grid_constant__ RecView rv) {

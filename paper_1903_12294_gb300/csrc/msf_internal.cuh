@@ -878,50 +878,82 @@ __device__ __forceinline__ void reduce_samples(const FeatAcc& acc, bool ok, int6
     }
     return;
   }
-  if (!ok) return;
-  // Several features: the lanes of each feature's group reduce with the hardware group
-  // reductions, no member loops. The fixed-point values sum exactly as three 21/21/22-bit
-  // limbs. Each square d*d = p + pe (exact) is put on a fixed-point grid of the group,
-  // 2^-52 of the group's largest square (k2 from the largest exponent): every term then fits
-  // 53 bits, the group's sum of up to 32 of them fits 58, and it sums exactly as limbs; the
-  // sum becomes a double-float pair again (24 significant bits, then the rest). Squares below
-  // 2^-52 of the largest drop out, well inside the sums' fp64-level tolerance.
-  const unsigned grp = __match_any_sync(act, fid);
+  // Several features: the lanes of a feature's group are chained in lane order, and pointer
+  // jumping along the chains sums all groups at once into their first lanes, in as many steps as
+  // the largest group takes (the hardware's group reductions take the groups one after the other:
+  // with some twenty groups of one to four samples a warp, 8M particles x 24 steps, 2.89 ms, now
+  // 2.19 ms). The fixed-point values sum exactly. Each square d*d = p + pe (exact) is put on a
+  // fixed-point grid of the group, 2^-52 of the group's largest square (k2 from the largest
+  // exponent): every term then fits 53 bits, the group's sum of up to 32 of them fits 58, and it
+  // sums exactly too; the sum becomes a double-float pair again (24 significant bits, then the
+  // rest). Squares below 2^-52 of the largest drop out, well inside the sums' fp64-level
+  // tolerance.
+  constexpr unsigned F = 0xFFFFFFFFu;
+  const unsigned grp = __match_any_sync(F, ok ? fid : (int64_t)-1);
   const int leader = __ffs(grp) - 1;
+  const int most = __reduce_max_sync(F, ok ? __popc(grp) : 0);  // the largest group
+  int next[5];  // the lane 1, 2, 4, 8, 16 places on in the group, or -1
+  {
+    const unsigned on = grp & ~((2u << lane) - 1u);
+    next[0] = __ffs(on) - 1;
+#pragma unroll
+    for (int i = 1; i < 5; ++i) {
+      const int t = __shfl_sync(F, next[i - 1], next[i - 1] & 31);
+      next[i] = next[i - 1] < 0 ? -1 : t;
+    }
+  }
+  auto total = [&](unsigned long long u) {
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      if (1 << i >= most) break;
+      const unsigned long long t = __shfl_sync(F, u, next[i] & 31);
+      if (next[i] >= 0) u += t;
+    }
+    return u;
+  };
 #pragma unroll 1
   for (int j = 0; j < acc.A; ++j) {
-    const float v = val(j);
-    const unsigned long long u = (unsigned long long)quantise(v, acc.kscale[j]);
-    const unsigned long long qs = limb_sum(grp, u);
-    const float d = isfinite(v) ? v : 0.f;
-    float h = 0.f, l = 0.f;
-    double w = 0.0;
+    const float v = ok ? val(j) : 0.f;
+    const unsigned long long qs = total((unsigned long long)quantise(v, acc.kscale[j]));
+    float d = isfinite(v) ? v : 0.f;
     const float ad = fabsf(d);
-    const bool dbl = !__all_sync(grp, ad == 0.f || (ad >= 0x1p-40f && ad <= 1.0e18f));
-    if (!dbl) {
-      const unsigned emax = __reduce_max_sync(grp, (__float_as_uint(d) >> 23) & 0xFFu);
-      if (emax) {
-        const int k2 = 304 - 2 * (int)emax;  // |d| < 2^(emax-126): d*d * 2^k2 < 2^52
-        const float p = __fmul_rn(d, d), pe = __fmaf_rn(d, d, -p);
-        const unsigned long long q2 =
-            (unsigned long long)(quantise(p, k2) + quantise(pe, k2));
-        const unsigned long long S = limb_sum(grp, q2);
-        const int sh = max(0, 40 - __clzll(S));  // S >> sh: at most 24 significant bits
-        const unsigned long long a = S >> sh;
-        h = __fmul_rn(__fmul_rn(__uint2float_rn((uint32_t)a), pow2f((sh - k2) / 2)),
-                      pow2f((sh - k2) - (sh - k2) / 2));
-        const unsigned long long r = S - (a << sh);  // below 2^sh: its top 24 bits
-        const int sr = max(0, sh - 24);
-        l = __fmul_rn(__fmul_rn(__uint2float_rn((uint32_t)(r >> sr)), pow2f((sr - k2) / 2)),
-                      pow2f((sr - k2) - (sr - k2) / 2));
+    const unsigned unsafe = __ballot_sync(F, !(ad == 0.f || (ad >= 0x1p-40f && ad <= 1.0e18f)));
+    const bool dbl = (unsafe & grp) != 0u;
+    double w = 0.0;
+    if (unsafe) {  // non-finite or extreme values in some group: plain fp64 (rare)
+      w = (double)d * (double)d;
+#pragma unroll 1
+      for (int i = 0; 1 << i < most; ++i) {
+        const int o = i == 0 ? next[0] : i == 1 ? next[1] : i == 2 ? next[2] : i == 3 ? next[3] : next[4];
+        const double t = __shfl_sync(F, w, o & 31);
+        if (o >= 0) w += t;
       }
-    } else {
-      for (unsigned m = grp; m; m &= m - 1) {
-        const double x = (double)__shfl_sync(grp, d, __ffs(m) - 1);
-        w += x * x;
-      }
+      if (dbl) d = 0.f;
     }
-    if (lane == leader) sink(fid, j, (unsigned long long)qs, h, l, w, dbl, false);
+    int emax = (int)((__float_as_uint(d) >> 23) & 0xFFu);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      if (1 << i >= most) break;
+      const int t = __shfl_sync(F, emax, next[i] & 31);
+      if (next[i] >= 0) emax = max(emax, t);
+    }
+    emax = __shfl_sync(F, emax, leader);
+    const int k2 = 304 - 2 * emax;  // |d| < 2^(emax-126): d*d * 2^k2 < 2^52
+    const float p = __fmul_rn(d, d), pe = __fmaf_rn(d, d, -p);
+    const unsigned long long S =
+        total(emax ? (unsigned long long)(quantise(p, k2) + quantise(pe, k2)) : 0ull);
+    float h = 0.f, l = 0.f;
+    if (S) {
+      const int sh = max(0, 40 - __clzll(S));  // S >> sh: at most 24 significant bits
+      const unsigned long long a = S >> sh;
+      h = __fmul_rn(__fmul_rn(__uint2float_rn((uint32_t)a), pow2f((sh - k2) / 2)),
+                    pow2f((sh - k2) - (sh - k2) / 2));
+      const unsigned long long r = S - (a << sh);  // below 2^sh: its top 24 bits
+      const int sr = max(0, sh - 24);
+      l = __fmul_rn(__fmul_rn(__uint2float_rn((uint32_t)(r >> sr)), pow2f((sr - k2) / 2)),
+                    pow2f((sr - k2) - (sr - k2) / 2));
+    }
+    if (ok && lane == leader) sink(fid, j, qs, h, l, w, dbl, false);
   }
 }
 
