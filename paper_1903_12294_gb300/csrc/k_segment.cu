@@ -90,37 +90,6 @@ __device__ __forceinline__ bool cmp_pred(const DevPred& p, uint32_t raw) {
   return (x >= p.lo) & (x <= p.hi);
 }
 
-// Shared-memory union-find over run slots (values only decrease). Path halving: each visited
-// slot is pointed at its grandparent with atomicMin, which only lowers a parent to another
-// ancestor in the same set, so it composes with concurrent linking.
-__device__ __forceinline__ uint32_t sfind(uint32_t* par, uint32_t a) {
-  volatile uint32_t* vp = par;
-  while (true) {
-    const uint32_t p = vp[a];
-    if (p == a) return a;
-    const uint32_t gp = vp[p];
-    if (gp == p) return p;
-    atomicMin(par + a, gp);
-    a = gp;
-  }
-}
-
-__device__ __forceinline__ void sunion(uint32_t* par, uint32_t a, uint32_t b) {
-  while (true) {
-    a = sfind(par, a);
-    b = sfind(par, b);
-    if (a == b) return;
-    if (a > b) {
-      uint32_t t = a;
-      a = b;
-      b = t;
-    }
-    uint32_t old = atomicMin(&par[b], a);
-    if (old == b) return;
-    b = old;
-  }
-}
-
 // Global union-find over component ids; reads bypass L1 so they see other SMs' links. Path
 // halving: each visited node is pointed at its grandparent with atomicMin, which can only lower
 // a parent to another ancestor in the same set, so it composes with concurrent linking.
@@ -1860,9 +1829,9 @@ constexpr size_t feat_vox_smem() {
 // feature changes and committed once per block. The other members wait in a list until there are
 // 32 of them for reduce_samples, whose instructions a few of them cost as many as 32 do (8M
 // particles x 24 steps, one feature with nine tenths of the members: all members through it
-// 4.4 ms, every round's others at once 3.4 ms, a full round of them 2.9 ms, their groups chained 2.2 ms). The samples are those of every point step falling in
-// the window's field steps that binning placed inside the grid: the same as the per-point pass
-// takes. Block (x, y) takes records
+// 4.4 ms, every round's others at once 3.4 ms, a full round of them 2.9 ms, their groups chained
+// 2.2 ms). The samples are those of every point step falling in the window's field steps that
+// binning placed inside the grid: the same as the per-point pass takes. Block (x, y) takes records
 // [x * chunk, (x + 1) * chunk) of window field step y.
 // RW: words of a record (4, 8 or 12, the first 2, 6 or 8 attributes).
 template <bool SPATIAL, int RW>

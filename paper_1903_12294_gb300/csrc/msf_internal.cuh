@@ -382,6 +382,37 @@ __device__ __forceinline__ int32_t voxel_of(float px, float py, float pz, int nx
   return ((int)fz * ny + (int)fy) * nx + (int)fx;
 }
 
+// Shared-memory union-find over a block's slots (values only decrease). Path halving: each visited
+// slot is pointed at its grandparent with atomicMin, which only lowers a parent to another
+// ancestor in the same set, so it composes with concurrent linking.
+__device__ __forceinline__ uint32_t sfind(uint32_t* par, uint32_t a) {
+  volatile uint32_t* vp = par;
+  while (true) {
+    const uint32_t p = vp[a];
+    if (p == a) return a;
+    const uint32_t gp = vp[p];
+    if (gp == p) return p;
+    atomicMin(par + a, gp);
+    a = gp;
+  }
+}
+
+__device__ __forceinline__ void sunion(uint32_t* par, uint32_t a, uint32_t b) {
+  while (true) {
+    a = sfind(par, a);
+    b = sfind(par, b);
+    if (a == b) return;
+    if (a > b) {
+      uint32_t t = a;
+      a = b;
+      b = t;
+    }
+    uint32_t old = atomicMin(&par[b], a);
+    if (old == b) return;
+    b = old;
+  }
+}
+
 // q = round_half_even(v * 2^k) with integer operations only: v = +-man * 2^(exp - 150), so
 // v * 2^k = +-man * 2^sh. Equal to llrint(ldexp((double)v, k)) for every finite fp32 v whose
 // result fits the exponent rule (|q| < 2^62); non-finite v gives 0.
