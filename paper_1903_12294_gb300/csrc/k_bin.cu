@@ -129,12 +129,6 @@ __device__ __forceinline__ float i64_to_f32_rn(long long s) {
   return __uint_as_float(bits | (s < 0 ? 0x80000000u : 0u));
 }
 
-// Per-voxel mean from the exact fixed-point sum: ((float)sum / (float)count) * 2^-k, every step
-// an IEEE fp32 operation rounded to nearest-even (the scaling split into two exact factors).
-__device__ __forceinline__ float voxel_mean(long long s, int c, float f1, float f2) {
-  return __fmul_rn(__fmul_rn(__fdiv_rn(i64_to_f32_rn(s), __int2float_rn(c)), f1), f2);
-}
-
 // Exact fp32 quotient x / c (IEEE round to nearest): a power-of-two count is an exact scaling,
 // anything else takes the IEEE division. Both give the correctly rounded quotient.
 __device__ __forceinline__ float div_count(float x, int c) {

@@ -77,7 +77,6 @@ struct Dataset {
 // ---------------------------------------------------------------------------------------------
 constexpr int kSegPerTile = 256;                 // BY * BZ * BT
 constexpr long long kWaitCycles = 2000000000ll;  // bounded device waits: about one second
-constexpr int kMaxRunsPerTile = kSegPerTile * 16; // at most 16 runs in a 32-bit row mask
 
 // Unsigned 32-bit division by a runtime constant: q = (t + ((n - t) >> s1)) >> s2 with
 // t = umulhi(m, n) (the round-up method of Granlund and Montgomery), exact for all n < 2^32.
@@ -671,14 +670,6 @@ __device__ __forceinline__ void commit_row(const FeatAcc& acc, int64_t fid, cons
   atomicAdd(scp + 1, (unsigned long long)r.n * (unsigned long long)r.z);
   atomicAdd(scp + 2, (unsigned long long)r.n * (unsigned long long)r.y);
   atomicAdd(scp + 3, (unsigned long long)r.sum_x);
-}
-
-// Voxels of one 32-voxel row straight into the accumulators.
-__device__ __forceinline__ void accumulate_row(const FeatAcc& acc, unsigned act, int64_t fid,
-                                               int lane, int x0, int tw, int z, int y, float f,
-                                               int c) {
-  reduce_row(act, fid, lane, x0, tw, z, y, f, c,
-             [&](int64_t g, const RowSums& r) { commit_row(acc, g, r); });
 }
 
 // ---------------------------------------------------------------------------------------------
