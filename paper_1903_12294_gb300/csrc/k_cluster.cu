@@ -596,7 +596,7 @@ __device__ __forceinline__ void add64(uint32_t* p, unsigned long long v) {
 // region test and of the distance is the same for them, and so is the list; a listed centre
 // carries the squared time term of every step, infinite where its region does not reach the step
 // (the time test of the step, in the deciding operations, made once per centre). One step at a
-// time the passes took 34.0 ms (ten assignments of 67M samples), now 18.0 ms. A sample's place
+// time the passes took 34.0 ms (ten assignments of 67M samples), so 18.1 ms. A sample's place
 // adds its tile coordinates as packed counters: count and x in one word, y and z in another, and
 // the steps' sum (1024 samples: no counter exceeds 16 bits).
 constexpr int kFieldSteps = 4;

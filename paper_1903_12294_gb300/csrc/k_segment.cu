@@ -108,8 +108,8 @@ __device__ __forceinline__ uint32_t gfind(uint32_t* par, uint32_t a) {
 }
 
 // The two finds walk in step, their loads in flight together, and stop as soon as they meet: the
-// unions wait on L2 (one after the other, the joins of 8M particles x 24 steps took 1.22 ms, now
-// 1.14 ms, the cross-tile ones 0.88, now 0.81).
+// unions wait on L2 (8M particles x 24 steps, one after the other: joins 1.22 ms, cross-tile ones
+// 0.88 ms; in step 1.14 and 0.81 ms).
 __device__ __forceinline__ void gunion(uint32_t* par, uint32_t a, uint32_t b) {
   while (true) {
     while (true) {
@@ -1455,7 +1455,7 @@ __global__ void __launch_bounds__(256) k_comp_fid(const __grid_constant__ SegArg
 // The same for a small window in one launch: block 0 sets the label bits in shared memory, counts
 // them and ranks every component; the other blocks empty the accumulators. A small step is a
 // chain of launches of a few microseconds each, and clearing the bits, marking, three scans,
-// clearing and ranking were seven of them (32^3 x 8: 351 us the step, now 304 us).
+// clearing and ranking were seven of them (32^3 x 8: 351 us the step, so 304 us).
 __global__ void __launch_bounds__(1024) k_feat_ranks(const __grid_constant__ SegArgs a,
                                                      FeatAcc acc, int32_t* cfid, int32_t* flabel,
                                                      int nwords) {

@@ -449,7 +449,8 @@ __device__ __forceinline__ long long quantise(float v, int k) {
 // into copy blockIdx.x % K, so that the atomics of a large feature spread over K addresses;
 // k_records sums the copies. Sums of field values and squares are formed per warp group in
 // double-float (fp32 pairs with exact TwoSum/TwoProd steps) and committed as two fp64 atomics;
-// no fp64 arithmetic runs on the SM (the part's fp64 pipe is narrow).
+// the part's fp64 pipe is narrow, so fp64 arithmetic on the SM is left to sums that one lane
+// keeps for many samples (the caches of the point samples' squares).
 // ---------------------------------------------------------------------------------------------
 struct FeatAcc {
   unsigned long long* n_vox;
