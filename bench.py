@@ -50,7 +50,8 @@ TRAFFIC = {
     # ncu DRAM bytes (read + write) of one launch, from a single-kernel capture of the unchanged
     # kernel (profiles/); combustion: the 4-timestep capture (--timesteps 4) scaled by 6 to the
     # 24-step launch (a launch's records and voxels grow in proportion to its field steps)
-    (3, "k_feat_points"): (600_658_176 + 10_216_960) * 6,
+    (3, "k_bin_reduce"): (1_074_027_000 + 1_551_283_000) * 6,
+    (3, "k_feat_points"): (679_826_000 + 8_584_000) * 6,
 }
 
 
@@ -308,7 +309,7 @@ def run_gpu(args):
 
     # dominant kernel and its roofline (per-launch CUDA-event durations from the profiled pass)
     npa = len({(s, a if s == 2 else 0) for s, a, *_ in wl.preds})
-    fused = bool(msf.msf_get_tuning(ctx.h, crit)[3] & msf.MSF_SCHED_FUSED_CRITERION)
+    fused = "k_mask" not in ktimes  # the criterion is evaluated inside the tile pass
     abytes = algorithmic_bytes(wl, npa, fused_criterion=fused)
     peak, peak_kind = peaks()
     copy_gbs = d2d_copy_gbs(dev) if rank == 0 else None
