@@ -1821,32 +1821,48 @@ constexpr size_t feat_vox_smem() {
 
 // Point statistics from the binned records (while they hold the loaded dataset's binning): the
 // samples of the window's field steps, grouped by (field step, bucket of consecutive voxels),
-// each with its voxel and its attributes side by side. Members are packed as for the joins; 32
-// of them lie in one bucket or a few (a few rows of the grid), so their component lookups hit
-// cached rows, and they mostly share one feature. A warp therefore has a feature of its own, the
-// last one that most of a round's samples belonged to: lanes whose sample belongs to it add to
-// sums of their own (an exact square and one fp64 addition per attribute), reduced when the
-// feature changes and committed once per block. The other members wait in a list until there are
-// 32 of them for reduce_samples, whose instructions a few of them cost as many as 32 do (8M
-// particles x 24 steps, one feature with nine tenths of the members: all members through it
-// 4.4 ms, every round's others at once 3.4 ms, a full round of them 2.9 ms, their groups chained
-// 2.2 ms). The samples are those of every point step falling in the window's field steps that
-// binning placed inside the grid: the same as the per-point pass takes. Block (x, y) takes records
+// each with its voxel and its attributes side by side. A warp walks windows of 256 records; the
+// members of a window, in the order of the lanes that hold them, make packs of 32 (the last one
+// what is left). The samples that a feature has in one pack are summed together, and a sum of
+// squares is rounded to a double-float there: the packs are part of the result, so whatever is
+// gathered from several packs to fill a warp stays apart by pack.
+//   - 32 members of whole packs at a time look up their components (they lie in one bucket or a
+//     few, a few rows of the grid, so the lookups hit cached rows).
+//   - They mostly share one feature, so a warp has a feature of its own, the last one that most of
+//     a round's samples belonged to: lanes whose sample belongs to it add to sums of their own (an
+//     exact square and one fp64 addition per attribute), reduced when the feature changes and
+//     committed once per block.
+//   - The other members wait in a list until there are 32 of them for reduce_samples, whose
+//     instructions a few of them cost as many as 32 do.
+// 8M particles x 24 steps, one feature with nine tenths of the members: a pack at a time, all through
+// reduce_samples, 5.5 ms, so 2.45 ms. (2.18 ms with the members of several packs summed together, but
+// then nearly equal samples of small features that had been summed apart were rounded together.)
+// The samples are those of every point step falling in the window's field steps that binning
+// placed inside the grid: the same as the per-point pass takes. Block (x, y) takes records
 // [x * chunk, (x + 1) * chunk) of window field step y.
 // RW: words of a record (4, 8 or 12, the first 2, 6 or 8 attributes).
+constexpr int kPackPer = 8;                        // records per lane and window
+constexpr int kPackBuf = 32 + 32 * kPackPer;       // a part of packs kept back, a window's packs
+static_assert(kRecChunkMax <= 32768, "a record's place in its block takes 15 bits");
+
 template <bool SPATIAL, int RW>
 __device__ __forceinline__ void feat_points_block(const SegArgs& a, const FeatAcc& acc,
                                                   const int32_t* __restrict__ cfid,
                                                   const RecView& rv, const int tw, uint32_t x) {
   constexpr int AM = RW == 4 ? 2 : RW == 8 ? 6 : 8;
-  __shared__ uint2 s_buf[8][kRecBuf];   // per warp: (voxel, record) of its members
-  __shared__ uint2 s_left[8][64];       // per warp: (feature, record) of those not of its own
+  constexpr unsigned F = 0xFFFFFFFFu;
+  // per warp: (voxel, place) of its members and (feature, place) of those not of its own feature;
+  // place: the record within the block, bits 0..14 (bits 8..14 its window), the pack within the
+  // window, bits 16..18, and in the second list bit 31: the pack has samples of one feature only
+  __shared__ uint2 s_buf[8][kPackBuf];
+  __shared__ uint2 s_left[8][32];
   __shared__ HotCache s_hot[8][1];  // per warp: its feature and sums, for the block's commit
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   uint32_t b0, b1;
   if (!rec_block(rv, a.g.t0 + tw, x, b0, b1)) return;  // block-uniform
   if (lane == 0) s_hot[w][0].fid = -1;
   const uint32_t step0 = step_seg0(a.g, tw);
+  const float* rec0 = rv.rec + (size_t)b0 * RW;
   int32_t own = -1;  // the warp's feature and the lane's sums for it
   long long q1[AM];
   double q2[AM];
@@ -1860,9 +1876,9 @@ __device__ __forceinline__ void feat_points_block(const SegArgs& a, const FeatAc
 #pragma unroll
     for (int j = 0; j < AM; ++j) {
       if (j >= acc.A) break;
-      const unsigned long long t = limb_sum(0xFFFFFFFFu, (unsigned long long)q1[j]);
+      const unsigned long long t = limb_sum(F, (unsigned long long)q1[j]);
 #pragma unroll
-      for (int o = 16; o; o >>= 1) q2[j] += __shfl_xor_sync(0xFFFFFFFFu, q2[j], o);
+      for (int o = 16; o; o >>= 1) q2[j] += __shfl_xor_sync(F, q2[j], o);
       if (lane == 0) {
         c.sq[j] = t;
         c.s2[j] = q2[j];
@@ -1875,11 +1891,12 @@ __device__ __forceinline__ void feat_points_block(const SegArgs& a, const FeatAc
   };
   const unsigned below = (1u << lane) - 1u;
   int nl = 0;  // members in s_left
-  auto take = [&](bool ok, uint2 e) {  // 32 members (fewer at the end)
+  // members of whole packs, 32 at most; last: none, and the list is emptied
+  auto take = [&](bool ok, uint2 e, bool last) {
     int32_t fid = -1;
     float v[AM] = {};
     if (ok) {
-      const float* p = rv.rec + (size_t)e.y * RW;
+      const float* p = rec0 + (e.y & 0x7FFFu) * RW;
 #pragma unroll
       for (int q = 0; q < AM; q += 2) {
         const float2 x = __ldg(reinterpret_cast<const float2*>(p + q));
@@ -1887,12 +1904,12 @@ __device__ __forceinline__ void feat_points_block(const SegArgs& a, const FeatAc
       }
       fid = __ldg(cfid + comp_of<SPATIAL>(a, tw, (int32_t)e.x));
     }
-    const unsigned act = __ballot_sync(0xFFFFFFFFu, ok);
-    unsigned mine = __ballot_sync(0xFFFFFFFFu, ok && fid == own);
+    const unsigned act = __ballot_sync(F, ok);
+    unsigned mine = __ballot_sync(F, ok && fid == own);
     if (act && __popc(mine) < 8) {  // does another feature have most of the round?
-      const int32_t f = __shfl_sync(0xFFFFFFFFu, fid, __fns(act, 0, (__popc(act) + 1) / 2));
-      const unsigned m = __ballot_sync(0xFFFFFFFFu, ok && fid == f);
-      if (__popc(m) >= 24) {
+      const int32_t f = __shfl_sync(F, fid, __fns(act, 0, (__popc(act) + 1) / 2));
+      const unsigned m = __ballot_sync(F, ok && fid == f);
+      if (__popc(m) >= 16 && 4 * __popc(m) >= 3 * __popc(act)) {
         if (own >= 0) {
           give();
           if (lane == 0) hot_commit(acc, s_hot[w][0]);
@@ -1912,62 +1929,83 @@ __device__ __forceinline__ void feat_points_block(const SegArgs& a, const FeatAc
       }
     }
     const unsigned left = act & ~mine;
-    if (ok && fid != own) s_left[w][nl + __popc(left & below)] = make_uint2((uint32_t)fid, e.y);
-    nl += __popc(left);
-    __syncwarp();
+    if (nl && (last || nl + __popc(left) > 32)) {
+      const bool in = lane < nl;
+      const uint2 r = in ? s_left[w][lane] : make_uint2(0u, 0u);
+      const float* p = rec0 + (r.y & 0x7FFFu) * RW;
+      reduce_samples(
+          acc, in, (int64_t)(((unsigned long long)r.x << 32) | (r.y & ~0xFFu)), r.y >> 31,
+          [&](int j) { return __ldg(p + j); },
+          [&](int64_t key, int j, unsigned long long qs, float h, float l, double wd, bool dbl,
+              bool) {
+            const int64_t i =
+                ((int64_t)(blockIdx.x & (acc.K - 1)) * acc.F + (key >> 32)) * acc.A + j;
+            atomicAdd(acc.sq + i, qs);
+            if (dbl) atomicAdd(acc.sa2 + i, wd);
+            else add_pair(acc.sa2 + i, h, l);
+          });
+      __syncwarp();
+      nl = 0;
+    }
+    if (left) {
+      // is the feature the only one of its pack?
+      const unsigned pack = __match_any_sync(F, ok ? e.y & ~0xFFu : F);
+      const int32_t f0 = __shfl_sync(F, fid, __ffs(pack) - 1);
+      const unsigned mixed = __ballot_sync(F, ok && fid != f0) & pack;
+      if (ok && fid != own)
+        s_left[w][nl + __popc(left & below)] =
+            make_uint2((uint32_t)fid, e.y | (mixed ? 0u : 0x80000000u));
+      nl += __popc(left);
+      __syncwarp();
+    }
   };
-  auto take_left = [&] {  // the first 32 of s_left
-    const bool ok = lane < nl;
-    const uint2 e = ok ? s_left[w][lane] : make_uint2(0u, 0u);
-    const uint2 rest = 32 + lane < nl ? s_left[w][32 + lane] : make_uint2(0u, 0u);
-    __syncwarp();
-    if (32 + lane < nl) s_left[w][lane] = rest;
-    nl = max(nl - 32, 0);
-    const float* p = rv.rec + (size_t)e.y * RW;
-    reduce_samples(
-        acc, ok, (int64_t)(int32_t)e.x, [&](int j) { return __ldg(p + j); },
-        [&](int64_t f, int j, unsigned long long qs, float h, float l, double wd, bool dbl, bool) {
-          const int64_t i = ((int64_t)(blockIdx.x & (acc.K - 1)) * acc.F + f) * acc.A + j;
-          atomicAdd(acc.sq + i, qs);
-          if (dbl) atomicAdd(acc.sa2 + i, wd);
-          else add_pair(acc.sa2 + i, h, l);
-        });
-    __syncwarp();
-  };
-  int n = 0;
-  for (uint32_t base = b0 + 32u * kRecPer * w;; base += 256u * kRecPer) {
-    const bool more = base < b1;  // else the remainders
+  int n = 0;  // members kept back, whole packs
+  for (uint32_t base = b0 + 32u * kPackPer * w;; base += 256u * kPackPer) {
+    const bool more = base < b1;
+    uint32_t v[kPackPer];
+    unsigned okm = 0u;
+    int rank = 0, total = 0;  // of the lane's first member in the window, and the window's members
     if (more) {
-      uint32_t v[kRecPer];
-      bool ok[kRecPer];
 #pragma unroll
-      for (int u = 0; u < kRecPer; ++u) {
+      for (int u = 0; u < kPackPer; ++u) {
         const uint32_t r = base + 32u * u + lane;
         v[u] = r < b1 ? __ldcs(&rv.rec_vn[r].x) : 0xFFFFFFFFu;
       }
 #pragma unroll
-      for (int u = 0; u < kRecPer; ++u) ok[u] = v[u] != 0xFFFFFFFFu && is_member(a, step0, v[u]);
+      for (int u = 0; u < kPackPer; ++u)
+        okm |= (v[u] != 0xFFFFFFFFu && is_member(a, step0, v[u]) ? 1u : 0u) << u;
 #pragma unroll
-      for (int u = 0; u < kRecPer; ++u) {
-        const unsigned b = __ballot_sync(0xFFFFFFFFu, ok[u]);
-        if (ok[u]) s_buf[w][n + __popc(b & below)] = make_uint2(v[u], base + 32u * u + lane);
-        n += __popc(b);
+      for (int u = 0; u < kPackPer; ++u) {
+        const unsigned b = __ballot_sync(F, (okm >> u) & 1u);
+        rank += __popc(b & below);
+        total += __popc(b);
       }
-      __syncwarp();
     }
-    // oldest first: the buffer's members in record order keep runs of one feature together
-    int i0 = 0;
-    for (; more ? i0 + 32 <= n : i0 < n || nl; i0 += 32) {
-      const bool ok = i0 + lane < n;
-      take(ok, ok ? s_buf[w][i0 + lane] : make_uint2(0u, b0));
-      if (nl >= 32 || (!more && i0 + 32 >= n && nl)) take_left();
+    const int full = total & ~31, part = total & 31;
+    auto store = [&](int lo, int hi, int at) {  // the window's members [lo, hi) to s_buf[at, ..)
+      int r = rank;
+#pragma unroll
+      for (int u = 0; u < kPackPer; ++u)
+        if ((okm >> u) & 1u) {
+          if (r >= lo && r < hi)
+            s_buf[w][at + r - lo] =
+                make_uint2(v[u], (base - b0 + 32u * u + lane) | (uint32_t)(r >> 5) << 16);
+          ++r;
+        }
+      __syncwarp();
+    };
+    if (full) store(0, full, 32);
+    const bool flush = n > 0 && (!more || n + part > 32);
+    for (int i = flush ? 0 : 32; i < 32 + full + (more ? 0 : 32); i += 32) {
+      const bool last = i == 32 + full;
+      const bool ok = !last && (i || lane < n);
+      take(ok, ok ? s_buf[w][i + lane] : make_uint2(0u, 0u), last);
     }
     if (!more) break;
-    n -= i0;
-    const uint2 rest = lane < n ? s_buf[w][i0 + lane] : make_uint2(0u, 0u);
+    if (flush) n = 0;
     __syncwarp();
-    if (i0 && lane < n) s_buf[w][lane] = rest;  // the remainder to the front
-    __syncwarp();
+    if (part) store(full, total, n);
+    n += part;
   }
   if (own >= 0) give();
   __syncthreads();

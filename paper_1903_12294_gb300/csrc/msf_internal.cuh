@@ -849,24 +849,28 @@ __device__ __forceinline__ unsigned long long limb_sum(unsigned m, unsigned long
   return (unsigned long long)s0 + ((unsigned long long)s1 << 21) + ((unsigned long long)s2 << 42);
 }
 
-// Point samples of one warp (lane: ok, feature fid, attribute values val(j)): the lanes
-// with the same feature reduce in the warp (exact 64-bit fixed-point sums; double-float sums of
-// squares), and one lane per feature hands the sums to sink(f, j, qs, h, l, w, dbl, one): the sum
-// of squares is h + l (a double-float pair, each exact in fp32), or w in fp64 when dbl is set
-// (non-finite or extreme values, rare); one is set when all the warp's samples belong to f (the
-// call then has a single leader). All 32 lanes must call this. The attributes are a loop:
-// unrolled, the code of both paths no longer fits the instruction cache, and the warps wait for it.
+// Point samples of one warp (lane: ok, key, attribute values val(j)): the lanes with the same key
+// (a feature, or one with more than that in its low word) are a group and reduce in the warp: exact
+// 64-bit fixed-point sums, double-float sums of squares. One lane per group hands the sums to
+// sink(key, j, qs, h, l, w, dbl, one): the sum of squares is h + l (a double-float pair, each exact
+// in fp32), or w in fp64 when dbl is set (non-finite or extreme values, rare); one is set when all
+// the warp's samples are one whole group (the call then has a single leader). whole: the lane's
+// group is all there is of its feature's samples' pack (see feat_points_block), and its squares are
+// summed in pairs, any other's on a fixed-point grid. Either sum keeps 48 bits: with equal or
+// nearly equal samples the deviation formed from it may be off by 2^-23.5, 8e-8, of the mean.
+// All 32 lanes must call this. The attributes are a loop: unrolled, the code of both paths no longer
+// fits the instruction cache, and the warps wait for it.
 template <class Val, class Sink>
-__device__ __forceinline__ void reduce_samples(const FeatAcc& acc, bool ok, int64_t fid, Val&& val,
-                                               Sink&& sink) {
+__device__ __forceinline__ void reduce_samples(const FeatAcc& acc, bool ok, int64_t key, bool whole,
+                                               Val&& val, Sink&& sink) {
   const unsigned act = __ballot_sync(0xFFFFFFFFu, ok);
   if (!act) return;
   const int lane = threadIdx.x & 31;
   // Common case when the samples come in voxel order: every member lane has the same feature.
   // The whole warp then reduces by butterfly (lanes without a sample add zeros).
   const int first = __ffs(act) - 1;
-  const int64_t f0 = __shfl_sync(0xFFFFFFFFu, fid, first);
-  if (__all_sync(0xFFFFFFFFu, !ok || fid == f0)) {
+  const int64_t k0 = __shfl_sync(0xFFFFFFFFu, key, first);
+  if (__all_sync(0xFFFFFFFFu, !ok || (key == k0 && whole))) {
 #pragma unroll 1
     for (int j = 0; j < acc.A; ++j) {
       const float v = ok ? val(j) : 0.f;
@@ -897,24 +901,24 @@ __device__ __forceinline__ void reduce_samples(const FeatAcc& acc, bool ok, int6
 #pragma unroll
         for (int o = 16; o; o >>= 1) w += __shfl_xor_sync(0xFFFFFFFFu, w, o);
       }
-      if (lane == first) sink(f0, j, qs, h, l, w, dbl, true);
+      if (lane == first) sink(k0, j, qs, h, l, w, dbl, true);
     }
     return;
   }
-  // Several features: the lanes of a feature's group are chained in lane order, and pointer
-  // jumping along the chains sums all groups at once into their first lanes, in as many steps as
-  // the largest group takes (the hardware's group reductions take the groups one after the other:
-  // with some twenty groups of one to four samples a warp, 8M particles x 24 steps, 2.89 ms, now
-  // 2.19 ms). The fixed-point values sum exactly. Each square d*d = p + pe (exact) is put on a
-  // fixed-point grid of the group, 2^-52 of the group's largest square (k2 from the largest
-  // exponent): every term then fits 53 bits, the group's sum of up to 32 of them fits 58, and it
-  // sums exactly too; the sum becomes a double-float pair again (24 significant bits, then the
-  // rest). Squares below 2^-52 of the largest drop out, well inside the sums' fp64-level
-  // tolerance.
+  // Several groups: the lanes of a group are chained in lane order, and pointer jumping along the
+  // chains sums all groups at once into their first lanes, in as many steps as the largest group
+  // takes (the hardware's group reductions take the groups one after the other: with some twenty
+  // groups of one to four samples a warp, 8M particles x 24 steps, 2.89 ms, by chains 2.19 ms). The
+  // fixed-point values sum exactly. Each square d*d = p + pe (exact) is put on a fixed-point grid of
+  // the group, 2^-52 of the group's largest square (k2 from the largest exponent): every term then
+  // fits 53 bits, the group's sum of up to 32 of them fits 58, and it sums exactly too; the sum is
+  // cut to a double-float pair again (24 significant bits, then the next 24).
   constexpr unsigned F = 0xFFFFFFFFu;
-  const unsigned grp = __match_any_sync(F, ok ? fid : (int64_t)-1);
+  const unsigned grp = __match_any_sync(F, ok ? key : (int64_t)-1);
   const int leader = __ffs(grp) - 1;
   const int most = __reduce_max_sync(F, ok ? __popc(grp) : 0);  // the largest group
+  const bool pairs = ok && whole && grp != (1u << lane);  // sums its pairs, as the warp above does
+  const bool some_pairs = __any_sync(F, pairs);
   int next[5];  // the lane 1, 2, 4, 8, 16 places on in the group, or -1
   {
     const unsigned on = grp & ~((2u << lane) - 1u);
@@ -940,7 +944,8 @@ __device__ __forceinline__ void reduce_samples(const FeatAcc& acc, bool ok, int6
     const unsigned long long qs = total((unsigned long long)quantise(v, acc.kscale[j]));
     float d = isfinite(v) ? v : 0.f;
     const float ad = fabsf(d);
-    const unsigned unsafe = __ballot_sync(F, !(ad == 0.f || (ad >= 0x1p-40f && ad <= 1.0e18f)));
+    const unsigned unsafe =
+        __ballot_sync(F, !(pairs ? df_safe(d) : ad == 0.f || (ad >= 0x1p-40f && ad <= 1.0e18f)));
     const bool dbl = (unsafe & grp) != 0u;
     double w = 0.0;
     if (unsafe) {  // non-finite or extreme values in some group: plain fp64 (rare)
@@ -976,7 +981,7 @@ __device__ __forceinline__ void reduce_samples(const FeatAcc& acc, bool ok, int6
       l = __fmul_rn(__fmul_rn(__uint2float_rn((uint32_t)(r >> sr)), pow2f((sr - k2) / 2)),
                     pow2f((sr - k2) - (sr - k2) / 2));
     }
-    if (ok && lane == leader) sink(fid, j, qs, h, l, w, dbl, false);
+    if (ok && lane == leader) sink(key, j, qs, h, l, w, dbl, false);
   }
 }
 
@@ -1027,7 +1032,9 @@ __device__ __forceinline__ void hot_commit(const FeatAcc& acc, HotCache& c) {
 template <class Val>
 __device__ __forceinline__ void accumulate_samples_hot(const FeatAcc& acc, HotCache (&cs)[kHotWays],
                                                        bool ok, int64_t fid, Val&& val) {
-  reduce_samples(acc, ok, fid, val,
+  const unsigned act = __ballot_sync(0xFFFFFFFFu, ok);
+  const int64_t f0 = __shfl_sync(0xFFFFFFFFu, fid, act ? __ffs(act) - 1 : 0);
+  reduce_samples(acc, ok, fid, __all_sync(0xFFFFFFFFu, !ok || fid == f0), val,
                  [&](int64_t f, int j, unsigned long long qs, float h, float l, double w,
                      bool dbl, bool one) {
                    HotCache& c = cs[(((uint32_t)f * 0x9E3779B1u) >> 16) & (kHotWays - 1)];
