@@ -16,8 +16,7 @@
 //   scan           offsets = exclusive prefix of hist (every bucket's slot range)
 //   k_bin_place    one CTA per 8192 samples of one point step: each sample, read in order, takes
 //                  its bucket's next slot (one global cursor per bucket) and is stored there as a
-//                  (voxel, attributes) record; also the largest finite |v| per attribute. With few
-//                  buckets (k_bin_place_sorted) a block sorts its samples by bucket first
+//                  (voxel, attributes) record; also the largest finite |v| per attribute
 //
 // Point samples may come on a finer time grid than the field (point step j falls in field step
 // fstep[j]); the records of all point steps of a field step go to that step's buckets.
@@ -335,119 +334,6 @@ __global__ void __launch_bounds__(kPlaceNT) k_bin_place(const __grid_constant__ 
   }
   __syncthreads();
   if ((int)threadIdx.x < A && s_max[threadIdx.x]) atomicMax(b.absmax + threadIdx.x, s_max[threadIdx.x]);
-}
-
-// The same for grids with few buckets, where a block's samples share them: the block counts its
-// samples per bucket in shared memory, takes each bucket's slots with one atomic, puts the records
-// in bucket order in shared memory and stores them as runs of neighbouring slots. One atomic and a
-// 16-byte request of its own per sample bound k_bin_place at 145 G requests/s (1M particles x 32
-// steps, 1024 buckets, A = 2: 455 us, now 392 us; with 16 buckets the atomics of a step queue on
-// 16 addresses). It takes at least two samples per bucket on average, which 64 KB of records bound
-// (sort_samples): beyond that the runs are single records and k_bin_place is the faster one.
-constexpr int kSortNT = 512;
-__host__ __device__ constexpr int sort_samples(int A) {
-  return rec_words(A) == 4 ? 4096 : rec_words(A) == 8 ? 2048 : 1024;
-}
-static bool place_sorted(int A, int nb) { return 2 * nb <= sort_samples(A); }
-static size_t sorted_smem(int A, int nb) {
-  return (size_t)sort_samples(A) * rec_words(A) * 4 + 8 * (size_t)nb;
-}
-
-template <int A>
-__global__ void __launch_bounds__(kSortNT, 3) k_bin_place_sorted(const __grid_constant__ BinArgs b) {
-  constexpr int RW = rec_words(A), VO = rec_pair(A), N = sort_samples(A), PER = N / kSortNT;
-  constexpr int A1 = A > 0 ? A : 1;
-  extern __shared__ __align__(16) uint32_t s_sort[];
-  uint32_t* s_rec = s_sort;               // [N][RW]
-  uint32_t* s_off = s_sort + N * RW;      // [nb] samples per bucket, then their first place
-  uint32_t* s_slot = s_off + b.nb;        // [nb] slot of place 0 (mod 2^32)
-  __shared__ unsigned s_max[A1];
-  __shared__ uint32_t s_warp[kSortNT / 32];
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int j = b.jbase + blockIdx.y;     // the point step
-  uint32_t* crow = b.cursor + (int64_t)__ldg(b.fstep + j) * b.nb * kCurStride;
-  for (int i = tid; i < b.nb; i += kSortNT) s_off[i] = 0u;
-  if (tid < A) s_max[tid] = 0u;
-  __syncthreads();
-  const int32_t* krow = b.key + (int64_t)j * b.P;
-  const bool nxt = j + 1 < b.Tp;  // the next point step's keys follow this step's row
-  const float* arow = b.attr + (int64_t)j * A * b.P;
-  const int64_t p0 = (int64_t)blockIdx.x * N + tid;
-  int32_t k[PER];
-  uint32_t rank[PER];
-#pragma unroll
-  for (int u = 0; u < PER; ++u) k[u] = p0 + u * kSortNT < b.P ? __ldcs(krow + p0 + u * kSortNT) : -1;
-#pragma unroll
-  for (int u = 0; u < PER; ++u)
-    rank[u] = k[u] >= 0 ? atomicAdd(s_off + (k[u] >> b.logR), 1u) : 0u;
-  __syncthreads();
-  // places: an exclusive prefix of the counts, each bucket's slots taken on the way
-  const int per = (b.nb + kSortNT - 1) / kSortNT;
-  const int lo = min(tid * per, b.nb), hi = min(lo + per, b.nb);
-  uint32_t sum = 0;
-  for (int i = lo; i < hi; ++i) sum += s_off[i];
-  uint32_t x = sum;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) s_warp[w] = x;
-  __syncthreads();
-  uint32_t before = 0, total = 0;
-#pragma unroll
-  for (int q = 0; q < kSortNT / 32; ++q) {
-    if (q < w) before += s_warp[q];
-    total += s_warp[q];
-  }
-  uint32_t run = before + x - sum;
-  for (int i = lo; i < hi; ++i) {
-    const uint32_t n = s_off[i];
-    s_off[i] = run;
-    if (n) s_slot[i] = atomicAdd(crow + (int64_t)i * kCurStride, n) - run;
-    run += n;
-  }
-  __syncthreads();
-  // the records to their places (the attributes of samples outside the grid count for the maxima)
-  unsigned lmax[A1];
-#pragma unroll
-  for (int a = 0; a < A1; ++a) lmax[a] = 0u;
-#pragma unroll
-  for (int u = 0; u < PER; ++u) {
-    const int64_t p = p0 + u * kSortNT;
-    if (p >= b.P) continue;
-    uint32_t r[RW];
-#pragma unroll
-    for (int i = 0; i < RW; ++i)
-      r[i] = i < A ? __float_as_uint(__ldcs(arow + (int64_t)(i < A ? i : 0) * b.P + p)) : 0u;
-#pragma unroll
-    for (int a = 0; a < A; ++a) {
-      const float v = __uint_as_float(r[a]);
-      if (isfinite(v)) lmax[a] = max(lmax[a], __float_as_uint(fabsf(v)));
-    }
-    if (k[u] < 0) continue;
-    r[VO] = (uint32_t)k[u];
-    r[VO + 1] = nxt ? (uint32_t)__ldg(krow + b.P + p) : 0xFFFFFFFFu;
-    uint32_t* dst = s_rec + (size_t)(s_off[k[u] >> b.logR] + rank[u]) * RW;
-#pragma unroll
-    for (int i = 0; i < RW; i += 4)
-      *reinterpret_cast<uint4*>(dst + i) = make_uint4(r[i], r[i + 1], r[i + 2], r[i + 3]);
-  }
-#pragma unroll
-  for (int a = 0; a < A; ++a) {
-    const unsigned m = __reduce_max_sync(0xFFFFFFFFu, lmax[a]);
-    if (lane == 0 && m) atomicMax(s_max + a, m);
-  }
-  __syncthreads();
-  if (tid < A && s_max[tid]) atomicMax(b.absmax + tid, s_max[tid]);
-  // one 16-byte unit per thread, neighbouring units by neighbouring threads
-  constexpr int UN = RW / 4;
-  for (int i = tid; i < (int)total * UN; i += kSortNT) {
-    const int q = i / UN, e = i - q * UN;
-    const uint32_t slot = s_slot[s_rec[q * RW + VO] >> b.logR] + (uint32_t)q;
-    *reinterpret_cast<uint4*>(b.rec + (size_t)slot * RW + 4 * e) =
-        *reinterpret_cast<const uint4*>(s_rec + 4 * i);
-  }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -897,15 +783,7 @@ static void launch_bin(msf_ctx* ctx, BinArgs b, bool keep, int phase, bool smem,
     else k_bin_keys<false><<<gs, 256, 0, s>>>(b);
   } else if (phase == 1) {
     ScopedKernel k(ctx, "k_bin_place", s);
-    if (place_sorted(A, b.nb)) {
-      static std::atomic<size_t> set{0};
-      const size_t sm = sorted_smem(A, b.nb);
-      allow_smem(k_bin_place_sorted<A>, sm, set);
-      const dim3 g((unsigned)((b.P + sort_samples(A) - 1) / sort_samples(A)), (unsigned)nj);
-      k_bin_place_sorted<A><<<g, kSortNT, sm, s>>>(b);
-    } else {
-      k_bin_place<A><<<gp, kPlaceNT, 0, s>>>(b);
-    }
+    k_bin_place<A><<<gp, kPlaceNT, 0, s>>>(b);
   } else if (phase == 2) {
     {
       ScopedKernel k(ctx, "k_bin_reduce", s);

@@ -85,3 +85,32 @@ def test_nearly_equal_samples(gpu, n, spread):
     var = ((v - m[:, None]) ** 2).mean(1)
     bound = (2.0 ** -47 + 2.0 ** -50) * m * m
     assert (np.abs(f["std_attr"][:, 0] ** 2 - var) <= bound).all()
+
+
+@pytest.mark.parametrize("nx,P,M,r,T,least", [(32, 20000, 300, 4, 8, 0.12),
+                                              (48, 30000, 300, 2, 8, 0.13)])
+def test_samples_of_one_point_lie_close(gpu, nx, P, M, r, T, least):
+    """All point steps of a field step are placed at the same time, each in the order of its points,
+    so the r samples of a point lie close together in their bucket and often share a pack: in 25 to
+    30 (r = 4) and 21 to 24 per cent (r = 2) of these features of one resting point the rounding of
+    two or more samples together shows. (With every block's samples sorted by bucket before they are
+    stored it is 0.4 and 6 per cent, and the deviations are other ones.)"""
+    rng = np.random.default_rng(nx)
+    field = np.full((T, nx, nx, nx), -1.0, np.float32)
+    even = np.arange(0, nx, 2)
+    z, y, x = (even[c] for c in np.unravel_index(rng.permutation(even.size ** 3)[:M],
+                                                 (even.size,) * 3))
+    field[:, z, y, x] = 1.0
+    who = rng.permutation(P)
+    p = np.empty((3, P))
+    p[:, who[:M]] = np.stack([x, y, z])
+    p[:, who[M:]] = rng.integers(0, nx, (3, P - M))
+    p[0, who[M:]] = p[0, who[M:]] // 2 * 2 + 1      # no member there
+    pos = np.tile((p + 0.5).astype(np.float32), (T * r, 1, 1))
+    attr = ((1 + rng.random(P)) * (1 + 1e-5 * rng.standard_normal((T * r, P)))).astype(np.float32)
+    f = _features(gpu, field, pos, attr[:, None], [j // r for j in range(T * r)])
+    assert len(f) == M * T and (f["n_pts"] == r).all()
+    v = attr[:, who[:M][np.argsort((z * nx + y) * nx + x)]].astype(np.float64)
+    v = v.reshape(T, r, M).transpose(0, 2, 1).reshape(-1, r)
+    exact = np.sqrt(np.maximum((v * v).sum(1) / r - (v.sum(1) / r) ** 2, 0.0))
+    assert (f["std_attr"][:, 0] != exact).mean() >= least
