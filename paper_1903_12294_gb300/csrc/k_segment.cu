@@ -1524,14 +1524,14 @@ __global__ void __launch_bounds__(1024) k_feat_ranks(const __grid_constant__ Seg
 // a block's 32 rows per warp were one long chain, 45 us before, 16 us now).
 constexpr int kCompThread = 8, kCompWarp = 512, kVoxHash = 2048;
 
-// Sums over voxels of one feature: tile-relative coordinates, order-preserving field keys,
-// double-float sums of the field and its squares; odd: a value double-float does not hold.
+// Sums over voxels of one feature: tile-relative coordinates, order-preserving field keys, fp64 sums
+// of the field and its squares (a deviation is formed from them: as double-floats of 48 bits they
+// left three to ten times the error of the rows' sums added up in fp64).
 struct VoxSums {
   int c, sx, sy, sz, st;
   int lo[4], hi[4];  // t, z, y, x
   unsigned kmin, kmax;
-  float s1h, s1l, s2h, s2l;
-  bool odd;
+  double s1, s2;
 };
 
 __device__ __forceinline__ void vox_clear(VoxSums& v) {
@@ -1543,8 +1543,7 @@ __device__ __forceinline__ void vox_clear(VoxSums& v) {
   }
   v.kmin = 0xFFFFFFFFu;
   v.kmax = 0u;
-  v.s1h = v.s1l = v.s2h = v.s2l = 0.f;
-  v.odd = false;
+  v.s1 = v.s2 = 0.0;
 }
 
 // A tile's origin in the window and in the dataset's arrays.
@@ -1585,29 +1584,21 @@ __device__ __forceinline__ void vox_add(VoxSums& v, const Geometry& g, const Til
   const bool isnan_f = f != f;  // NaN takes no part in the extrema
   v.kmin = min(v.kmin, isnan_f ? float_key(INFINITY) : float_key(f));
   v.kmax = max(v.kmax, isnan_f ? float_key(-INFINITY) : float_key(f));
-  const float p = __fmul_rn(f, f), pe = __fmaf_rn(f, f, -p);  // f*f == p + pe exactly
-  df_add(v.s1h, v.s1l, f);
-  df_add(v.s2h, v.s2l, p);
-  df_add(v.s2h, v.s2l, pe);
-  v.odd |= !df_safe(f);
+  const double d = f2d(f);
+  v.s1 += d;
+  v.s2 = __fma_rn(d, d, v.s2);
 }
 
 // n voxels' sums into feature fid. TEST: read the extrema first and leave out the atomics that
 // would change nothing (a large feature gets a commit from every tile it crosses).
 template <bool TEST>
 __device__ __forceinline__ void vox_commit(const FeatAcc& acc, const TileOrigin& o, int64_t fid,
-                                           int n, const VoxSums& v, bool dbl, double s1d,
-                                           double s2d) {
+                                           int n, const VoxSums& v) {
   const int64_t i = (int64_t)(blockIdx.x & (acc.K - 1)) * acc.F + fid;
   atomicAdd(acc.n_vox + i, (unsigned long long)n);
   atomicAdd(acc.n_pts + i, (unsigned long long)v.c);
-  if (dbl) {
-    atomicAdd(acc.sf + i, s1d);
-    atomicAdd(acc.sf2 + i, s2d);
-  } else {
-    add_pair(acc.sf + i, v.s1h, v.s1l);
-    add_pair(acc.sf2 + i, v.s2h, v.s2l);
-  }
+  atomicAdd(acc.sf + i, v.s1);
+  atomicAdd(acc.sf2 + i, v.s2);
   const int org[4] = {o.t0, o.z0, o.y0, o.x0};
   const int sum[4] = {v.st, v.sz, v.sy, v.sx};
   int4 mn = make_int4(0x7FFFFFFF, 0x7FFFFFFF, 0x7FFFFFFF, 0x7FFFFFFF), mx = make_int4(-1, -1, -1, -1);
@@ -1639,7 +1630,6 @@ __device__ __forceinline__ void vox_warp(const FeatAcc& acc, const Geometry& g,
   VoxSums v;
   vox_clear(v);
   for (int i = a + lane; i < b; i += 32) vox_add(v, g, o, list[i], field, count);
-  const bool dbl = __any_sync(F, v.odd);
   v.c = __reduce_add_sync(F, v.c);
   v.sx = __reduce_add_sync(F, v.sx);
   v.sy = __reduce_add_sync(F, v.sy);
@@ -1652,27 +1642,12 @@ __device__ __forceinline__ void vox_warp(const FeatAcc& acc, const Geometry& g,
   }
   v.kmin = __reduce_min_sync(F, v.kmin);
   v.kmax = __reduce_max_sync(F, v.kmax);
-  double s1 = 0.0, s2 = 0.0;
-  if (!dbl) {
 #pragma unroll
-    for (int d = 16; d; d >>= 1) {
-      df_add2(v.s1h, v.s1l, __shfl_xor_sync(F, v.s1h, d), __shfl_xor_sync(F, v.s1l, d));
-      df_add2(v.s2h, v.s2l, __shfl_xor_sync(F, v.s2h, d), __shfl_xor_sync(F, v.s2l, d));
-    }
-  } else {  // non-finite or extreme values: plain fp64 (rare)
-    for (int i = a + lane; i < b; i += 32) {
-      int x, y, z, t;
-      const double f = (double)__ldg(field + tile_voxel(g, o, list[i], x, y, z, t));
-      s1 += f;
-      s2 += f * f;
-    }
-#pragma unroll
-    for (int d = 16; d; d >>= 1) {
-      s1 += __shfl_xor_sync(F, s1, d);
-      s2 += __shfl_xor_sync(F, s2, d);
-    }
+  for (int d = 16; d; d >>= 1) {
+    v.s1 += __shfl_xor_sync(F, v.s1, d);
+    v.s2 += __shfl_xor_sync(F, v.s2, d);
   }
-  if (lane == 0) vox_commit<true>(acc, o, fid, b - a, v, dbl, s1, s2);
+  if (lane == 0) vox_commit<true>(acc, o, fid, b - a, v);
 }
 
 template <bool SPATIAL>
@@ -1784,15 +1759,7 @@ __device__ __forceinline__ void feat_vox_tile(const SegArgs& a, const FeatAcc& a
       VoxSums v;
       vox_clear(v);
       for (int i = st; i < st + n; ++i) vox_add(v, g, o, s_list[i], field, count);
-      double s1 = 0.0, s2 = 0.0;
-      if (v.odd)
-        for (int i = st; i < st + n; ++i) {
-          int x, y, z, t;
-          const double f = (double)__ldg(field + tile_voxel(g, o, s_list[i], x, y, z, t));
-          s1 += f;
-          s2 += f * f;
-        }
-      vox_commit<false>(acc, o, fid, n, v, v.odd, s1, s2);
+      vox_commit<false>(acc, o, fid, n, v);
     }
     __syncwarp();
   }
