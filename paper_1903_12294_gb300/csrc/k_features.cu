@@ -453,7 +453,7 @@ int features_run(msf_ctx* ctx, const msf_criteria* crit, const int32_t* labels,
   a.out = out_kind == MSF_DEVICE ? out
                                  : reinterpret_cast<msf_feature*>(carve(sizeof(msf_feature) * F));
   const unsigned fb = (unsigned)((F * K + kRecNT - 1) / kRecNT);
-  const bool ranked = fast && a.nwords <= kRankWords;
+  const bool ranked = fast && a.nwords <= kRankWords && a.acc.F <= kRankFeatures;
   if (ranked) {
     MSF_TRY(seg_feature_ranks(ctx, a.nwords, a.acc, flabel));
   } else {

@@ -1135,9 +1135,14 @@ int segment_field_fixed(const Geometry& g, int npred, const DevPred& pred, uint3
 // fast feature path (k_segment.cu): marks the feature labels of the retained segmentation in
 // rootbits and counts them; then, after the ranks exist, reduces voxel and point statistics.
 // With both, flabel [F] receives the features' labels. Windows of up to kRankWords words of bits
-// (32 voxel-timesteps each) take seg_feature_ranks instead of the bits, ranks and the empty
-// accumulators' own launches; seg_feature_stats then has its features' ranks (ranked).
-constexpr int64_t kRankWords = 49152;
+// (32 voxel-timesteps each) and kRankFeatures features take seg_feature_ranks instead of the bits,
+// ranks and the empty accumulators' own launches; seg_feature_stats then has its features' ranks
+// (ranked). The ranks are one block's work, so the launches that they save only pay for themselves
+// while there is little of it. All feature statistics of a call, by launches and by one block: 1536
+// words, 28 features 58 and 35 us, 14,810 131 and 122, 24,583 173 and 175; 12,288 words, 192
+// features 60 and 43 us, 9323 101 and 92, 19,645 127 and 130; 24,576 words, 764 features 60 and 62
+// us, 39,104 195 and 262; 49,152 words, 768 features 61 and 86 us, 1.3M 0.48 and 3.2 ms.
+constexpr int64_t kRankWords = 12288, kRankFeatures = 8192;
 int seg_mark_roots(msf_ctx* ctx, uint32_t* rootbits);
 int seg_feature_ranks(msf_ctx* ctx, int64_t nwords, const FeatAcc& acc, int32_t* flabel);
 int seg_feature_stats(msf_ctx* ctx, const RankArrays& rk, const FeatAcc& acc, int32_t* flabel,
