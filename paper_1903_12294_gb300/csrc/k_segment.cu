@@ -546,6 +546,9 @@ __device__ __forceinline__ bool pair_first_seen(unsigned long long* set, uint32_
   return true;  // crowded: join without remembering
 }
 
+// Tiles with at least this many (row, direction) pairs walk them direction by direction.
+constexpr int kHookDense = 1024;
+
 struct HookSmem {
   unsigned long long set[kHookSet];
   uint32_t mask[kSegPerTile], rb[kSegPerTile];
@@ -553,23 +556,53 @@ struct HookSmem {
   uint16_t task[kSegPerTile * 14];  // row | direction << 8
 };
 
+// bytes of it that hook_tile uses
+template <bool SPATIAL>
+constexpr size_t hook_smem() { return SPATIAL ? sizeof(HookSmem) : 16; }
+
 // One tile's cross-face joins. A row with members meets up to 14 rows of other tiles: the nine to
 // its left (its first run against their last ones), the backward rows in y/z that lie in another
 // tile, and the row one step earlier when it opens a time chunk. A few rows of a tile have
 // members, and the pass waits on L2: the (row, direction) pairs are listed first and the block's
 // threads take one each, so that the lookups of a row run beside each other (one thread walking
-// its row's directions, 256^3 x 24 with three predicates, 0.81 ms, now 0.60 ms).
+// its row's directions, 256^3 x 24 with three predicates, 0.81 ms, now 0.60 ms). In a dense tile
+// most rows have most directions, and neighbouring tasks of different kinds hold each other up: there
+// every thread takes its own row, all of them the same direction at a time (128^3 x 16 with 70 %
+// members: by tasks 0.19 ms, so 0.16; the same of 50 % 0.21 and 0.17; 96x64x64x4 with 70 % 69 and 33
+// us, spatial edges).
+// With temporal edges alone a row has one direction, its runs are single voxels and their pairs all
+// differ: every thread takes its own row, without the list and the set, whose shared memory would
+// leave the lines that the threads walk along too little of L1 (128^3 x 16 with 95 % members 0.43 ms,
+// so 0.20; 30 % 44 and 31 us).
 template <bool SPATIAL, bool CG = false>
 __device__ __forceinline__ void hook_tile(const SegArgs& a, int tile, HookSmem& S) {
   const Geometry& g = a.g;
   const int tid = threadIdx.x;
-  for (int i = tid; i < kHookSet; i += 256) S.set[i] = ~0ull;
   const TileCoord tc = tile_coord(g, tile);
   auto coords = [&](int r, int& tw, int& z, int& y) {
     y = (tc.ty << g.lby) + (r & ((1 << g.lby) - 1));
     z = (tc.tz << g.lbz) + ((r >> g.lby) & ((1 << g.lbz) - 1));
     tw = (tc.tt << g.lbt) + (r >> (g.lby + g.lbz)) - g.toff;
   };
+  if constexpr (!SPATIAL) {
+    int tw, z, y;
+    coords(tid, tw, z, y);
+    if (y >= g.ny || z >= g.nz || tw <= 0 || tw >= g.tw || !(a.edges & MSF_EDGE_TEMPORAL) ||
+        ((tw + g.toff) & ((1 << g.lbt) - 1)) != 0)
+      return;
+    const uint2 e = ld_seg<CG>(a.seg + seg_index(g, tw, z, y, tc.xs));
+    if (!e.x) return;
+    const uint2 e2 = ld_seg<CG>(a.seg + seg_index(g, tw - 1, z, y, tc.xs));
+    if (!e2.x) return;
+    const uint32_t st = run_starts(e.x, false), st2 = run_starts(e2.x, false);
+    row_contacts(e.x, e2.x, false, false, [&](int x1, int x2) {
+      const uint32_t c0 = ld_seg<CG>(a.runcomp + e.y + run_index(st, x1));
+      const uint32_t c1 = ld_seg<CG>(a.runcomp + e2.y + run_index(st2, x2));
+      if (c0 != c1) gunion(a.cparent, c0, c1);
+    });
+    return;
+  }
+  for (int i = tid; i < kHookSet; i += 256) S.set[i] = ~0ull;
   uint32_t dirs = 0u;
   {
     int tw, z, y;
@@ -580,17 +613,15 @@ __device__ __forceinline__ void hook_tile(const SegArgs& a, int tile, HookSmem& 
     S.mask[tid] = e.x;
     S.rb[tid] = e.y;
     if (e.x) {
-      if (SPATIAL) {
-        const uint32_t ys = (y > 0 ? 1u : 0u) | 2u | (y + 1 < g.ny ? 4u : 0u);
-        if ((e.x & 1u) && tc.xs > 0)
-          dirs = (z > 0 ? ys : 0u) | ys << 3 | (z + 1 < g.nz ? ys << 6 : 0u);
+      const uint32_t ys = (y > 0 ? 1u : 0u) | 2u | (y + 1 < g.ny ? 4u : 0u);
+      if ((e.x & 1u) && tc.xs > 0)
+        dirs = (z > 0 ? ys : 0u) | ys << 3 | (z + 1 < g.nz ? ys << 6 : 0u);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {  // dy -1, -1, 0, 1; dz 0, -1, -1, -1
-          const int y2 = y + (k == 3) - (k < 2), z2 = z - (k > 0);
-          if (y2 >= 0 && y2 < g.ny && z2 >= 0 &&
-              ((y2 >> g.lby) != (y >> g.lby) || (z2 >> g.lbz) != (z >> g.lbz)))
-            dirs |= 1u << (9 + k);
-        }
+      for (int k = 0; k < 4; ++k) {  // dy -1, -1, 0, 1; dz 0, -1, -1, -1
+        const int y2 = y + (k == 3) - (k < 2), z2 = z - (k > 0);
+        if (y2 >= 0 && y2 < g.ny && z2 >= 0 &&
+            ((y2 >> g.lby) != (y >> g.lby) || (z2 >> g.lbz) != (z >> g.lbz)))
+          dirs |= 1u << (9 + k);
       }
       if ((a.edges & MSF_EDGE_TEMPORAL) && tw > 0 && ((tw + g.toff) & ((1 << g.lbt) - 1)) == 0)
         dirs |= 1u << 13;
@@ -598,13 +629,16 @@ __device__ __forceinline__ void hook_tile(const SegArgs& a, int tile, HookSmem& 
   }
   int total;
   int pos = block_exscan(__popc(dirs), S.warp, &total);
-  for (; dirs; dirs &= dirs - 1) S.task[pos++] = (uint16_t)(tid | (__ffs(dirs) - 1) << 8);
+  const bool dense = total >= kHookDense;
+  if (!dense)
+    for (uint32_t d = dirs; d; d &= d - 1) S.task[pos++] = (uint16_t)(tid | (__ffs(d) - 1) << 8);
   __syncthreads();
   auto join = [&](uint32_t c0, uint32_t c1) {
     if (c0 != c1 && pair_first_seen(S.set, c0, c1)) gunion(a.cparent, c0, c1);
   };
-  for (int i = tid; i < total; i += 256) {
-    const int r = S.task[i] & 255, k = S.task[i] >> 8;
+  for (int i = dense ? 0 : tid; i < (dense ? 14 : total); i += dense ? 1 : 256) {
+    if (dense && !((dirs >> i) & 1u)) continue;
+    const int r = dense ? tid : S.task[i] & 255, k = dense ? i : S.task[i] >> 8;
     int tw, z, y;
     coords(r, tw, z, y);
     int xs = tc.xs;
@@ -637,9 +671,9 @@ __device__ __forceinline__ void hook_tile(const SegArgs& a, int tile, HookSmem& 
 // one CTA per tile
 template <bool SPATIAL>
 __global__ void __launch_bounds__(256, 4) k_hook(const __grid_constant__ SegArgs a) {
-  __shared__ __align__(16) HookSmem s_hook;
+  __shared__ __align__(16) char s_hook[hook_smem<SPATIAL>()];
   if (__ldg(&a.tileinfo[blockIdx.x].x) == 0) return;  // no member in the tile
-  hook_tile<SPATIAL>(a, blockIdx.x, s_hook);
+  hook_tile<SPATIAL>(a, blockIdx.x, *reinterpret_cast<HookSmem*>(s_hook));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -2338,13 +2372,13 @@ __global__ void __launch_bounds__(256) k_mask_batch(const __grid_constant__ Batc
 // (tile, query) = (blockIdx.x, blockIdx.y): the tile's cross-face joins with its pair set
 template <bool SPATIAL>
 __global__ void __launch_bounds__(256, 4) k_hook_batch(const __grid_constant__ BatchPlan b) {
-  __shared__ __align__(16) HookSmem s_hook;
+  __shared__ __align__(16) char s_hook[hook_smem<SPATIAL>()];
   __shared__ __align__(16) SegArgs s_args;
   load_args(&s_args, b.qargs + blockIdx.y);
   __syncthreads();
   if ((int)blockIdx.x >= s_args.g.ntiles) return;  // block-uniform
   if (__ldg(&s_args.tileinfo[blockIdx.x].x) == 0) return;  // no member in the tile
-  hook_tile<SPATIAL>(s_args, blockIdx.x, s_hook);
+  hook_tile<SPATIAL>(s_args, blockIdx.x, *reinterpret_cast<HookSmem*>(s_hook));
 }
 
 // (point block, chunk item) = (blockIdx.x, row0 + blockIdx.y); chunk items in absolute point
@@ -2530,7 +2564,7 @@ __global__ void __launch_bounds__(256, 4) k_batch_fused(const __grid_constant__ 
 template <bool SP>
 static constexpr size_t fused_dyn_smem() {
   const size_t tile = tile_dyn_smem<SP>();
-  const size_t hook = sizeof(HookSmem);
+  const size_t hook = hook_smem<SP>();
   const size_t fin = sizeof(int32_t) * kSegPerTile * (SP ? 16 : 32);
   return std::max(tile, std::max(hook, fin));
 }
