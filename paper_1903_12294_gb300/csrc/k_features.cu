@@ -242,61 +242,91 @@ __device__ __forceinline__ double div_by(double x, double n, double r) {
   return isfinite(q) ? __fma_rn(__fma_rn(-q, n, x), r, q) : q;
 }
 
-// One lane per (feature, copy): the K copies of a feature lie in neighbouring lanes and are summed
-// by exchanges (one thread per feature walked them one after the other, 26 us of a small step).
-// The records go through shared memory so that the block stores them as one run of words (each
-// thread storing its own 312 bytes took 0.27 ms for 584K features, now 0.21 ms).
+// SPLIT: one lane per (feature, copy), the K copies of a feature in neighbouring lanes and summed by
+// exchanges (with few features one thread per feature walks its copies one after the other, 23 us of
+// a small step's 60 features, so 14). Otherwise, and with many features, one thread per feature: a
+// lane per copy reads one word of every sector (one attribute, 4000 features of 16 copies 30 us by
+// features and 21 by copies, 8000 31 and 37, 30,000 31 and 90). The records go through shared memory
+// so that the block stores them as one run of words (each thread storing its own 312 bytes took 0.27
+// ms for 584K features, so 0.21 ms).
+constexpr int64_t kRecSplit = 1 << 16;  // copies of all features up to which a lane takes one each
 constexpr int kRecNT = 128;
 constexpr int kRecWords = (int)(sizeof(msf_feature) / 8);
 static_assert(sizeof(msf_feature) == 8 * kRecWords, "records are whole 8-byte words");
 
+template <bool SPLIT>
 __global__ void __launch_bounds__(kRecNT) k_records(const __grid_constant__ FeatArgs a) {
   __shared__ __align__(16) unsigned long long s_rec[kRecNT * kRecWords];
   constexpr unsigned W = 0xFFFFFFFFu;
   const FeatAcc& c = a.acc;
-  const int per = kRecNT / c.K;  // features per block (K: a power of two, at most 16)
-  const int fl = threadIdx.x / c.K, k = threadIdx.x % c.K;
+  const int L = SPLIT ? c.K : 1;  // lanes per feature (K: a power of two, at most 16)
+  const int per = kRecNT / L;     // features per block
+  const int fl = threadIdx.x / L, k = threadIdx.x % L;
   const int64_t f = (int64_t)blockIdx.x * per + fl;
   const bool in = f < c.F;
-  const int64_t i = in ? (int64_t)k * c.F + f : 0;
-  auto sum = [&](unsigned long long v) {
-    v = in ? v : 0ull;
-    for (int o = c.K >> 1; o; o >>= 1) v += __shfl_xor_sync(W, v, o);
+  unsigned long long nv = 0, np = 0, sc[4] = {0, 0, 0, 0}, sq[MSF_MAX_ATTR] = {};
+  double sf = 0.0, sf2 = 0.0, sa2[MSF_MAX_ATTR] = {};
+  unsigned kmin = 0xFFFFFFFFu, kmax = 0u;
+  int bmin[4] = {0x7FFFFFFF, 0x7FFFFFFF, 0x7FFFFFFF, 0x7FFFFFFF}, bmax[4] = {-1, -1, -1, -1};
+  auto add = [&](int64_t i) {  // copy i / F of the feature
+    nv += c.n_vox[i];
+    np += c.n_pts[i];
+    sf += c.sf[i];
+    sf2 += c.sf2[i];
+    kmin = min(kmin, c.fmin[i]);
+    kmax = max(kmax, c.fmax[i]);
+    const int4 b0 = reinterpret_cast<const int4*>(c.bbmin)[i];
+    const int4 b1 = reinterpret_cast<const int4*>(c.bbmax)[i];
+    const int lo[4] = {b0.x, b0.y, b0.z, b0.w}, hi[4] = {b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      bmin[j] = min(bmin[j], lo[j]);
+      bmax[j] = max(bmax[j], hi[j]);
+      sc[j] += c.sc[i * 4 + j];
+    }
+#pragma unroll
+    for (int j = 0; j < MSF_MAX_ATTR; ++j)
+      if (j < a.A) {
+        sq[j] += c.sq[i * a.A + j];
+        sa2[j] += c.sa2[i * a.A + j];
+      }
+  };
+  if (in) {
+    if (SPLIT) add((int64_t)k * c.F + f);
+    else
+      for (int q = 0; q < c.K; ++q) add((int64_t)q * c.F + f);
+  }
+  auto reduce = [&](auto v, auto&& op) {
+    if (SPLIT)
+      for (int o = L >> 1; o; o >>= 1) v = op(v, __shfl_xor_sync(W, v, o));
     return v;
   };
-  auto sumd = [&](double v) {
-    v = in ? v : 0.0;
-    for (int o = c.K >> 1; o; o >>= 1) v += __shfl_xor_sync(W, v, o);
-    return v;
-  };
-  auto least = [&](auto v) {
-    for (int o = c.K >> 1; o; o >>= 1) v = min(v, __shfl_xor_sync(W, v, o));
-    return v;
-  };
-  auto most = [&](auto v) {
-    for (int o = c.K >> 1; o; o >>= 1) v = max(v, __shfl_xor_sync(W, v, o));
-    return v;
-  };
-  const unsigned long long nv = sum(c.n_vox[i]), np = sum(c.n_pts[i]);
-  const double sf = sumd(c.sf[i]), sf2 = sumd(c.sf2[i]);
-  const unsigned kmin = least(c.fmin[i]), kmax = most(c.fmax[i]);
-  const int4 b0 = reinterpret_cast<const int4*>(c.bbmin)[i];
-  const int4 b1 = reinterpret_cast<const int4*>(c.bbmax)[i];
-  const int bmin[4] = {least(b0.x), least(b0.y), least(b0.z), least(b0.w)};
-  const int bmax[4] = {most(b1.x), most(b1.y), most(b1.z), most(b1.w)};
+  auto sum = [&](auto v) { return reduce(v, [](auto x, auto y) { return x + y; }); };
+  auto least = [&](auto v) { return reduce(v, [](auto x, auto y) { return min(x, y); }); };
+  auto most = [&](auto v) { return reduce(v, [](auto x, auto y) { return max(x, y); }); };
+  nv = sum(nv);
+  np = sum(np);
+  sf = sum(sf);
+  sf2 = sum(sf2);
+  kmin = least(kmin);
+  kmax = most(kmax);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    bmin[j] = least(bmin[j]);
+    bmax[j] = most(bmax[j]);
+    sc[j] = sum(sc[j]);
+  }
   msf_feature& o = *reinterpret_cast<msf_feature*>(s_rec + fl * kRecWords);
   if (k == 0)
     for (int j = 0; j < kRecWords; ++j) s_rec[fl * kRecWords + j] = 0ull;
   const double n = (double)nv, rn = __drcp_rn(n), npd = (double)np;
-  for (int j = 0; j < 4; ++j) {
-    const unsigned long long sc = sum(c.sc[i * 4 + j]);
-    if (k == 0) {
+  if (k == 0) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
       o.bbox_min[j] = bmin[j];
       o.bbox_max[j] = bmax[j];
-      o.centroid[j] = div_by((double)sc, n, rn);
+      o.centroid[j] = div_by((double)sc[j], n, rn);
     }
-  }
-  if (k == 0) {
     o.label = a.flabel ? (in ? a.flabel[f] : 0) : -1;  // -1: set by k_labels
     o.n_attr = a.A;
     o.n_vox = (int64_t)nv;
@@ -309,9 +339,11 @@ __global__ void __launch_bounds__(kRecNT) k_records(const __grid_constant__ Feat
     o.max_field = key_float(kmax);
   }
   const double qnan = __longlong_as_double(0x7ff8000000000000ll);
-  for (int j = 0; j < a.A; ++j) {
-    const long long s = (long long)sum(c.sq[i * a.A + j]);
-    const double sa2 = sumd(c.sa2[i * a.A + j]);
+#pragma unroll
+  for (int j = 0; j < MSF_MAX_ATTR; ++j) {
+    if (j >= a.A) break;
+    const long long s = (long long)sum(sq[j]);
+    const double s2 = sum(sa2[j]);
     if (k) continue;
     o.sumq[j] = s;
     if (np == 0) {
@@ -320,7 +352,7 @@ __global__ void __launch_bounds__(kRecNT) k_records(const __grid_constant__ Feat
     } else {
       const double m = (double)s / (npd * a.scale[j]);
       o.mean_attr[j] = m;
-      const double v = sa2 / npd - m * m;
+      const double v = s2 / npd - m * m;
       o.std_attr[j] = sqrt(v > 0.0 ? v : 0.0);
     }
   }
@@ -452,7 +484,6 @@ int features_run(msf_ctx* ctx, const msf_criteria* crit, const int32_t* labels,
   a.flabel = fast ? flabel : nullptr;
   a.out = out_kind == MSF_DEVICE ? out
                                  : reinterpret_cast<msf_feature*>(carve(sizeof(msf_feature) * F));
-  const unsigned fb = (unsigned)((F * K + kRecNT - 1) / kRecNT);
   const bool ranked = fast && a.nwords <= kRankWords && a.acc.F <= kRankFeatures;
   if (ranked) {
     MSF_TRY(seg_feature_ranks(ctx, a.nwords, a.acc, flabel));
@@ -495,7 +526,10 @@ int features_run(msf_ctx* ctx, const msf_criteria* crit, const int32_t* labels,
   }
   {
     ScopedKernel k(ctx, "k_records");
-    k_records<<<fb, kRecNT, 0, s>>>(a);
+    const bool split = K == 1 || FK <= kRecSplit;
+    const unsigned grid = (unsigned)(((split ? FK : (int64_t)F) + kRecNT - 1) / kRecNT);
+    if (split) k_records<true><<<grid, kRecNT, 0, s>>>(a);
+    else k_records<false><<<grid, kRecNT, 0, s>>>(a);
   }
   if (!fast) {
     ScopedKernel k(ctx, "k_labels");
