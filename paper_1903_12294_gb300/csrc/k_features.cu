@@ -235,11 +235,16 @@ __global__ void __launch_bounds__(256) k_pts(const __grid_constant__ FeatArgs a)
   hot_merge(a.acc, s_hot);
 }
 
-// x / n from r = 1 / n: one correction step with the exact residual, for several quotients by one
-// n (an fp64 division is a chain of operations on this part's narrow pipe).
+// x / n from r = 1 / n (rounded), for several quotients by one n (an fp64 division is a chain of
+// operations on this part's narrow pipe): Markstein's correction step (P. W. Markstein, Computation of
+// elementary functions on the IBM RISC System/6000 processor, IBM J. Res. Dev. 34, 1990). q is within
+// 1.5 units of the quotient, its residual is exact, and the corrected sum differs from x / n by less
+// than 2^-51 units before its one rounding. For a sum x (an integer of at most 53 bits, or a multiple of
+// a power of two) and a count n < 2^31, x / n is no midpoint of two doubles (x would need 54 bits) and
+// at least 2^-32 units away from one, so the rounding is that of the quotient itself.
 __device__ __forceinline__ double div_by(double x, double n, double r) {
   const double q = __dmul_rn(x, r);
-  return isfinite(q) ? __fma_rn(__fma_rn(-q, n, x), r, q) : q;
+  return __fma_rn(__fma_rn(-q, n, x), r, q);
 }
 
 // SPLIT: one lane per (feature, copy), the K copies of a feature in neighbouring lanes and summed by

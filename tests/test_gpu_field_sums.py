@@ -42,3 +42,32 @@ def test_deviation_of_nearly_equal_values(gpu, dx, dy, dz, spread):
     bound = (4 if v.shape[1] == 2 else 16) * 2.0 ** -53 * mean * mean
     np.testing.assert_allclose(f["mean_field"], mean, rtol=16 * 2.0 ** -53)
     assert (np.abs(f["std_field"] ** 2 - var) <= bound).all()
+
+
+def test_centroids_are_ieee_quotients(gpu):
+    """Centroids are the exact integer sums of the coordinates over the voxel count, rounded once:
+    feature sizes from one voxel to some thousands, on rows of up to 4096 voxels."""
+    rng = np.random.default_rng(3)
+    T, ny, nx = 9, 64, 4096
+    f = np.where(rng.random((T, 1, ny, nx)) < 0.45, 1.0, -1.0).astype(np.float32)
+    ctx = gpu.Context(0)
+    try:
+        ctx.load(torch.as_tensor(f).cuda(), torch.full((T, 3, 1), 0.5).cuda(),
+                 torch.ones((T, 1, 1)).cuda())
+        ctx.bin()
+        preds = [(0, 0, 0, 0.0, 0.0)]
+        for edges in (1, 2):
+            lab, n = ctx.segment(0, T, preds, edges)
+            g = ctx.features(0, T, lab, preds, edges)
+            l = lab.cpu().numpy().ravel()
+            at = np.flatnonzero(l >= 0)
+            which = np.searchsorted(g["label"], l[at])
+            count = np.bincount(which, minlength=n)
+            assert np.array_equal(count, g["n_vox"])
+            c = np.stack(np.unravel_index(at, (T, 1, ny, nx)), 1)
+            for j in range(4):
+                s = np.zeros(n, np.int64)
+                np.add.at(s, which, c[:, j])
+                assert np.array_equal(g["centroid"][:, j], s / count), j
+    finally:
+        ctx.close()
