@@ -2,7 +2,7 @@
 // centre properties and per-cluster summaries (§3.4), and trajectory splitting (§3.4).
 //
 // All of them are single passes over resident arrays with integer or fixed-order results:
-//   merging    every pair of centres is tested once (tiles of 256 x 256 in shared memory) and
+//   merging    every pair of centres is tested once (tiles of pairs in shared memory) and
 //              matching pairs are joined in a lock-free union-find whose roots are the smallest
 //              index of their tree (a root is only ever hooked under a smaller one), so the
 //              flattened parents are the groups' smallest indices whatever the order of joins;
@@ -94,53 +94,58 @@ __device__ void uf_union(int* parent, int a, int b) {
 }
 
 constexpr int kMergeTile = 256;
+constexpr int kMergeNarrow = 32768;  // centres up to which a block takes 128 columns
 
 __global__ void k_merge_init(int* parent, int K) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < K; i += gridDim.x * blockDim.x)
     parent[i] = i;
 }
 
-// Block (bj, bi - row0), bj >= bi: rows i of tile bi against columns j > i of tile bj. A pair whose
-// roots were equal when the block started is joined already and needs no value test. Where centres
-// agree widely (the case merging is for) nearly all pairs are such pairs once the first tile's row
-// has been joined with every column, so that row is launched first. The block joins its rows and
-// columns in shared memory and then each with its set's first member in the map, one union per
-// thread or two: a thread that joined every matching pair of its row in the map waited on L2 time
-// and again while its warp stood still (16,384 centres in 986 groups: 0.75 to 0.85 ms, now 0.51 ms).
+// Block (x, y): rows i of tile y (one per thread) against the columns j > i of the TC ones from x * TC.
+// Most pairs of unlike centres fail on the first value compared, so nothing stands before that test.
+// A pair whose roots were equal when the block started is joined already; where centres agree widely
+// (the case merging is for) those are nearly all. The block joins its rows and columns in shared
+// memory and then each with its set's first member in the map, one union per thread or two: a thread
+// that joined every matching pair of its row in the map waited on L2 time and again while its warp
+// stood still.
+// One launch: with the first rows in one of their own, whose joins the rest then knew, centres that
+// hardly agree waited for it (16,384 of them 94 us in one launch, 130 in two, 5000 of them 32 and 61).
+// TC: few columns a block give more blocks and shorter chains, many fewer unions of the same sets in
+// the map (all calls, one launch of 256 columns, then of 128: 16,384 centres without a match 107, 99
+// us, in 1862 groups 282, 266, in 18 468, 270; 40,000 centres in 2310 groups 698, 835 us).
+template <int TC>
 __global__ void __launch_bounds__(kMergeTile) k_merge_pairs(const float* __restrict__ centers,
                                                             int K, float eps, int terms,
-                                                            int* parent, int row0) {
-  const int bi = row0 + blockIdx.y, bj = blockIdx.x;
-  if (bj < bi) return;
-  __shared__ float2 s_v[kMergeTile];
-  __shared__ int s_root[kMergeTile];
-  __shared__ uint32_t s_set[2 * kMergeTile];  // the columns, then the rows of another tile
-  const int j0 = bj * kMergeTile, i0 = bi * kMergeTile, tid = threadIdx.x;
-  const int jn = min(kMergeTile, K - j0), in = min(kMergeTile, K - i0);
-  const uint32_t row = bi == bj ? tid : kMergeTile + tid;
-  s_set[tid] = tid;
-  s_set[kMergeTile + tid] = kMergeTile + tid;
+                                                            int* parent) {
+  const int i0 = (int)blockIdx.y * kMergeTile, j0 = (int)blockIdx.x * TC;
+  if (j0 + TC <= i0) return;
+  __shared__ float s_p[TC], s_f[TC];
+  __shared__ int s_root[TC];
+  __shared__ uint32_t s_set[TC + kMergeTile];  // the columns, then the rows
+  const int tid = threadIdx.x, i = i0 + tid;
+  const int jn = min(TC, K - j0);
+  const uint32_t row = i >= j0 && i < j0 + TC ? (uint32_t)(i - j0) : (uint32_t)(TC + tid);
+  for (int n = tid; n < TC + kMergeTile; n += kMergeTile) s_set[n] = n;
   if (tid < jn) {
-    s_v[tid] = make_float2(centers[6 * (size_t)(j0 + tid) + 4], centers[6 * (size_t)(j0 + tid) + 5]);
+    s_p[tid] = centers[6 * (size_t)(j0 + tid) + 4];
+    s_f[tid] = centers[6 * (size_t)(j0 + tid) + 5];
     s_root[tid] = uf_find(parent, j0 + tid);
   }
   __syncthreads();
-  if (tid < in) {
-    const int i = i0 + tid;
+  if (i < K) {
     const float pi = centers[6 * (size_t)i + 4], fi = centers[6 * (size_t)i + 5];
     const bool use_p = terms & MSF_MERGE_POINT, use_f = terms & MSF_MERGE_FIELD;
-    const int root = bi == bj ? s_root[tid] : uf_find(parent, i);
-    for (int q = bi == bj ? tid + 1 : 0; q < jn; ++q) {
+    const int root = uf_find(parent, i);
+    for (int q = max(0, i + 1 - j0); q < jn; ++q) {
+      if (use_p && !value_match(pi, s_p[q], eps)) continue;
       if (s_root[q] == root) continue;
-      const float2 v = s_v[q];
-      if (use_p && !value_match(pi, v.x, eps)) continue;
-      if (use_f && !value_match(fi, v.y, eps)) continue;
+      if (use_f && !value_match(fi, s_f[q], eps)) continue;
       sunion(s_set, row, q);
     }
   }
   __syncthreads();
-  auto centre = [&](uint32_t n) { return n < kMergeTile ? j0 + (int)n : i0 + (int)n - kMergeTile; };
-  for (uint32_t n = tid; n < 2 * kMergeTile; n += kMergeTile) {
+  auto centre = [&](uint32_t n) { return n < TC ? j0 + (int)n : i0 + (int)n - TC; };
+  for (uint32_t n = tid; n < TC + kMergeTile; n += kMergeTile) {
     const uint32_t first = sfind(s_set, n);
     if (first != n) uf_union(parent, centre(n), centre(first));
   }
@@ -760,9 +765,11 @@ int msf_merge_clusters(msf_ctx* c, const float* centers, int centers_kind, int32
   {
     ScopedKernel k(c, "k_merge_pairs");
     const unsigned nt = (unsigned)((K + kMergeTile - 1) / kMergeTile);
-    k_merge_pairs<<<dim3(nt, 1), kMergeTile, 0, s>>>(dc, K, eps_m, terms, parent, 0);
-    if (nt > 1)
-      k_merge_pairs<<<dim3(nt, nt - 1), kMergeTile, 0, s>>>(dc, K, eps_m, terms, parent, 1);
+    if (K <= kMergeNarrow)
+      k_merge_pairs<128><<<dim3((unsigned)((K + 127) / 128), nt), kMergeTile, 0, s>>>(dc, K, eps_m,
+                                                                                      terms, parent);
+    else
+      k_merge_pairs<256><<<dim3(nt, nt), kMergeTile, 0, s>>>(dc, K, eps_m, terms, parent);
   }
   {
     ScopedKernel k(c, "k_merge_flatten");
