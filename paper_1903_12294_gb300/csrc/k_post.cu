@@ -165,48 +165,31 @@ __global__ void k_merge_flatten(int* parent, int K, uint32_t* n_groups) {
 // ---------------------------------------------------------------------------------------------
 // relabelling through a merge map
 // ---------------------------------------------------------------------------------------------
-// VEC: labels in 16-byte units (an aligned buffer; the last n % 4 labels apart), four in flight
-// per thread: both passes are bound by memory (67M + 34M labels, scalar 0.30 ms, now 0.23).
-template <bool VEC, class F>
-__device__ __forceinline__ void each_label(int64_t n, F&& f) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  const int64_t units = VEC ? n >> 2 : n;
-  const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  for (int64_t i = i0; i < units; i += 4 * stride) f(i, stride, units);
-}
-
-template <bool VEC>
 __global__ void __launch_bounds__(256) k_relabel_check(const int32_t* __restrict__ lab, int64_t n,
                                                        int K, uint32_t* bad) {
   bool b = false;
-  each_label<VEC>(n, [&](int64_t i, int64_t stride, int64_t units) {
-    if constexpr (VEC) {
-      int4 l[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        l[u] = i + u * stride < units ? reinterpret_cast<const int4*>(lab)[i + u * stride]
-                                      : make_int4(-1, -1, -1, -1);
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        b |= max(max(l[u].x, l[u].y), max(l[u].z, l[u].w)) >= K;
-    } else {
-      for (int u = 0; u < 4; ++u)
-        if (i + u * stride < units) b |= lab[i + u * stride] >= K;
-    }
-  });
-  if (VEC && blockIdx.x == 0 && threadIdx.x < (n & 3)) b |= lab[(n & ~3ll) + threadIdx.x] >= K;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x)
+    b |= lab[i] >= K;
   if (__any_sync(kFull, b) && (threadIdx.x & 31) == 0) atomicOr(bad, 1u);
 }
 
+// VEC: labels in 16-byte units (an aligned buffer; the last n % 4 labels apart), four in flight per
+// thread: the pass is bound by memory (50M labels, single ones 103 us, so 62; the check, which only
+// reads, takes 47 us by single labels and 62 by units, and unaligned buffers 112 and 110 by single
+// labels, one and four at a time).
 template <bool VEC>
 __global__ void __launch_bounds__(256) k_relabel_apply(int32_t* __restrict__ lab, int64_t n,
                                                        const int32_t* __restrict__ map,
                                                        const uint32_t* bad) {
   if (*bad) return;  // a label out of range: nothing changes
   auto one = [&](int32_t l) { return l >= 0 ? __ldg(map + l) : l; };
-  each_label<VEC>(n, [&](int64_t i, int64_t stride, int64_t units) {
-    if constexpr (VEC) {
-      int4* lab4 = reinterpret_cast<int4*>(lab);
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if constexpr (VEC) {
+    const int64_t units = n >> 2;
+    int4* lab4 = reinterpret_cast<int4*>(lab);
+    for (int64_t i = i0; i < units; i += 4 * stride) {
       int4 l[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u)
@@ -217,14 +200,16 @@ __global__ void __launch_bounds__(256) k_relabel_apply(int32_t* __restrict__ lab
 #pragma unroll
       for (int u = 0; u < 4; ++u)
         if (i + u * stride < units) lab4[i + u * stride] = l[u];
-    } else {
-      for (int u = 0; u < 4; ++u)
-        if (i + u * stride < units) lab[i + u * stride] = one(lab[i + u * stride]);
     }
-  });
-  if (VEC && blockIdx.x == 0 && threadIdx.x < (n & 3)) {
-    int32_t* p = lab + (n & ~3ll) + threadIdx.x;
-    *p = one(*p);
+    if (blockIdx.x == 0 && threadIdx.x < (n & 3)) {
+      int32_t* p = lab + (n & ~3ll) + threadIdx.x;
+      *p = one(*p);
+    }
+  } else {
+    for (int64_t i = i0; i < n; i += stride) {
+      const int32_t l = lab[i];
+      if (l >= 0) lab[i] = __ldg(map + l);
+    }
   }
 }
 
@@ -820,11 +805,11 @@ int msf_relabel(msf_ctx* c, int32_t* labels, int labels_kind, int64_t n, const i
   uint32_t* bad = S.status.as<uint32_t>();
   MSF_CUDA_TRY(cudaMemsetAsync(bad, 0, sizeof(uint32_t), s));
   const bool vec = ((uintptr_t)dl & 15) == 0;
-  const unsigned g = blocks_for(vec ? (n + 3) / 4 : n, 256, c->sm_count * 8);
+  const unsigned gc = blocks_for(n, 256, c->sm_count * 8);
+  const unsigned g = vec ? blocks_for((n + 3) / 4, 256, c->sm_count * 8) : gc;
   {
     ScopedKernel k(c, "k_relabel_check");
-    if (vec) k_relabel_check<true><<<g, 256, 0, s>>>(dl, n, K, bad);
-    else k_relabel_check<false><<<g, 256, 0, s>>>(dl, n, K, bad);
+    k_relabel_check<<<gc, 256, 0, s>>>(dl, n, K, bad);
   }
   {
     ScopedKernel k(c, "k_relabel_apply");
