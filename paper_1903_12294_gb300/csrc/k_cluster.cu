@@ -598,26 +598,32 @@ __device__ __forceinline__ void add64(uint32_t* p, unsigned long long v) {
 // (the time test of the step, in the deciding operations, made once per centre). One step at a
 // time the passes took 34.0 ms (ten assignments of 67M samples), so 18.1 ms. A sample's place
 // adds its tile coordinates as packed counters: count and x in one word, y and z in another, and
-// the steps' sum (1024 samples: no counter exceeds 16 bits).
+// the steps' sum (1024 samples: no counter exceeds 16 bits). Where four steps together would reach
+// more cells or centres than the lists hold (cells of a step or two), two steps go together or one
+// (field_steps).
 constexpr int kFieldSteps = 4;
 
+template <int S>
 struct __align__(16) FieldList {
-  float4 pv[kWCand];           // x, y, z, -value
-  float dt[kWCand][kFieldSteps];  // kt (t - step)^2, or infinity
+  float4 pv[kWCand];    // x, y, z, -value
+  float dt[kWCand][S];  // kt (t - step)^2, or infinity
   uint16_t q[kWCand];
 };
 
-template <int TX, int TY, int TZ>
-__global__ void __launch_bounds__(256, 4) k_slic_assign_field_tiled(const __grid_constant__ SlicArgs a) {
+// S: steps a thread has room for, 4 or 2; most: how many of them a tile takes (S = 4: all)
+template <int TX, int TY, int TZ, int S>
+__global__ void __launch_bounds__(256, 4) k_slic_assign_field_tiled(const __grid_constant__ SlicArgs a,
+                                                                    int most) {
   static_assert(TX * TY * TZ == 256 && TX % 8 == 0 && TY % 4 == 0, "8 x 4 voxels per warp");
-  constexpr int S = kFieldSteps;
+  static_assert(S == 2 || S == kFieldSteps, "pairs of steps");
+  const int steps = S == 2 ? most : S;
   __shared__ CandList s_c;
-  __shared__ FieldList s_w[8];
+  __shared__ FieldList<S> s_w[8];
   __shared__ uint32_t s_acc[kCand][5];  // count | x, y | z, step, the value sum's halves
   __shared__ int s_warp[8];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int ntx = (a.nx + TX - 1) / TX, nty = (a.ny + TY - 1) / TY, ntz = (a.nz + TZ - 1) / TZ;
-  const int ntt = (a.tw + S - 1) / S;
+  const int ntt = (a.tw + steps - 1) / steps;
   const int64_t ntiles = (int64_t)ntx * nty * ntz * ntt;
   const int wx = (w % (TX / 8)) * 8, wy = (w / (TX / 8)) % (TY / 4) * 4;
   const int wz = w / ((TX / 8) * (TY / 4));
@@ -628,7 +634,7 @@ __global__ void __launch_bounds__(256, 4) k_slic_assign_field_tiled(const __grid
     const int bx = (int)(r % ntx); r /= ntx;
     const int by = (int)(r % nty); r /= nty;
     const int bz = (int)(r % ntz);
-    const int t0 = (int)(r / ntz) * S, nt = min(S, a.tw - t0);
+    const int t0 = (int)(r / ntz) * steps, nt = min(steps, a.tw - t0);
     const int x0 = bx * TX, y0 = by * TY, z0 = bz * TZ;
     auto step_time = [&](int s) { return __fadd_rn((float)(a.t0 + t0 + s), 0.5f); };
     int lo[4], nn[4];
@@ -653,7 +659,7 @@ __global__ void __launch_bounds__(256, 4) k_slic_assign_field_tiled(const __grid
     const float xs = __fadd_rn((float)xv, 0.5f), ys = __fadd_rn((float)yv, 0.5f);
     const float zs = __fadd_rn((float)zv, 0.5f);
     // the warp's list: centres whose region reaches the box of its voxels (and some step)
-    FieldList& L = s_w[w];
+    FieldList<S>& L = s_w[w];
     int n = nc >= 0 ? 0 : -1;
     for (int b = 0; b < nc; b += 32) {
       const int q = b + lane;
@@ -1032,6 +1038,34 @@ static int fixed_scale_host(double max_abs, long long n) {
   return 62 - e - b;
 }
 
+// Steps of a field tile of TX x TY x TZ voxels: as many as leave its cells within a block's list and
+// the centres that a warp's voxels reach (8 x 4 x 1 of them, a centre per cell) within a warp's, with
+// some room for centres that have moved together; four where no number does. 64^3 x 8, six
+// assignments, cells of 4 x 4 x 4 voxels and one step: four steps (each sample looked up by itself) 3.25
+// ms, two 1.27; cells of 8 x 8 x 8 and four steps: four 0.33, two 0.40.
+template <int TX, int TY, int TZ>
+static int field_steps(const SlicArgs& a) {
+  const int tile[3] = {TX - 1, TY - 1, TZ - 1}, warp[3] = {7, 3, 0};
+  for (int s = kFieldSteps; s >= 1; s >>= 1) {
+    double cells = 1.0, reach = 1.0;
+    for (int q = 0; q < 4; ++q) {
+      cells *= std::min<double>(a.k[q], std::floor((q < 3 ? tile[q] : s - 1) / (double)a.C[q]) + 3.0);
+      reach *= std::min<double>(a.k[q], (q < 3 ? warp[q] : s - 1) / (double)a.C[q] + 2.0);
+    }
+    if (cells <= 256.0 && reach <= 0.9 * kWCand) return s;
+  }
+  return kFieldSteps;
+}
+
+template <int TX, int TY, int TZ>
+static void launch_field_tiled(const SlicArgs& a, unsigned grid, cudaStream_t s) {
+  const int steps = field_steps<TX, TY, TZ>(a);
+  if (steps == kFieldSteps)
+    k_slic_assign_field_tiled<TX, TY, TZ, kFieldSteps><<<grid, 256, 0, s>>>(a, steps);
+  else
+    k_slic_assign_field_tiled<TX, TY, TZ, 2><<<grid, 256, 0, s>>>(a, steps);
+}
+
 int cluster_run(msf_ctx* ctx, const msf_cluster_params* prm, int32_t* flabel, int32_t* plabel,
                 float* centers_host, int64_t* counts_host, int* iters) {
   const Dataset& d = ctx->ds;
@@ -1200,8 +1234,8 @@ int cluster_run(msf_ctx* ctx, const msf_cluster_params* prm, int32_t* flabel, in
     }
     {
       ScopedKernel k(ctx, "k_slic_assign_field");
-      if (d.nz > 1) k_slic_assign_field_tiled<8, 8, 4><<<gt, 256, 0, s>>>(a);
-      else k_slic_assign_field_tiled<16, 16, 1><<<gt, 256, 0, s>>>(a);
+      if (d.nz > 1) launch_field_tiled<8, 8, 4>(a, gt, s);
+      else launch_field_tiled<16, 16, 1>(a, gt, s);
     }
     if (nps > 0) {
       ScopedKernel k(ctx, "k_slic_assign_points");
