@@ -752,22 +752,11 @@ static size_t reduce_wide_smem(int A, int logR) {
   return R * (8 * (size_t)A + 4) + std::max(staged, 4 * R * A + 4 * R);
 }
 
-static int bucket_log2(int A, int64_t V) {
-  int l = 11;
-  while (l < 12 && ((V + ((int64_t)1 << l) - 1) >> l) > kHistSmem &&
-         reduce_wide_smem(A, l + 1) <= (size_t)220 * 1024)
-    ++l;
-  return l;
+static int max_bucket_log2(int A) {
+  return reduce_wide_smem(A, 12) <= (size_t)220 * 1024 ? 12 : 11;
 }
-
-template <typename K>
-static void allow_smem(K kernel, size_t bytes, std::atomic<size_t>& set) {
-  // The attribute is per device and set before every launch that needs more than before (also
-  // just under 48 KB: the default limit counts the static shared memory too).
-  if (bytes > set.load()) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    set.store(bytes);
-  }
+static int bucket_log2(int A, int64_t V) {
+  return ((V + 2047) >> 11) > kHistSmem ? max_bucket_log2(A) : 11;
 }
 
 // phase 0: keys of point steps [j0, j0 + nj); 1: their records; 2: every (bucket, field step);
@@ -791,12 +780,12 @@ static void launch_bin(msf_ctx* ctx, BinArgs b, bool keep, int phase, bool smem,
       const size_t sm = reduce_smem(A, b.logR);
       const dim3 gr((unsigned)b.nb, (unsigned)b.T);
       if (keep) {
-        static std::atomic<size_t> set{0};
-        allow_smem(k_bin_reduce<A, true>, sm, set);
+        static std::atomic<uint64_t> set{0};
+        ensure_smem_attr(k_bin_reduce<A, true>, reduce_smem(A, max_bucket_log2(A)), set);
         k_bin_reduce<A, true><<<gr, kBinNT, sm, s>>>(b);
       } else {
-        static std::atomic<size_t> set{0};
-        allow_smem(k_bin_reduce<A, false>, sm, set);
+        static std::atomic<uint64_t> set{0};
+        ensure_smem_attr(k_bin_reduce<A, false>, reduce_smem(A, max_bucket_log2(A)), set);
         k_bin_reduce<A, false><<<gr, kBinNT, sm, s>>>(b);
       }
     }
@@ -807,12 +796,12 @@ static void launch_bin(msf_ctx* ctx, BinArgs b, bool keep, int phase, bool smem,
       const size_t sm = reduce_wide_smem(A, b.logR);
       const unsigned g = (unsigned)std::min<int64_t>(nj, (int64_t)ctx->sm_count * 2);
       if (keep) {
-        static std::atomic<size_t> set{0};
-        allow_smem(k_bin_reduce_wide<A, true>, sm, set);
+        static std::atomic<uint64_t> set{0};
+        ensure_smem_attr(k_bin_reduce_wide<A, true>, reduce_wide_smem(A, max_bucket_log2(A)), set);
         k_bin_reduce_wide<A, true><<<g, kBinNT, sm, s>>>(b);
       } else {
-        static std::atomic<size_t> set{0};
-        allow_smem(k_bin_reduce_wide<A, false>, sm, set);
+        static std::atomic<uint64_t> set{0};
+        ensure_smem_attr(k_bin_reduce_wide<A, false>, reduce_wide_smem(A, max_bucket_log2(A)), set);
         k_bin_reduce_wide<A, false><<<g, kBinNT, sm, s>>>(b);
       }
     }

@@ -1040,20 +1040,6 @@ constexpr size_t tile_dyn_smem() {
   return (size_t)kSegPerTile * (SP ? 16 : 32) * (sizeof(uint32_t) + sizeof(uint16_t));
 }
 
-// Opt a kernel into more than 48 KB of dynamic shared memory, once per device (the attribute
-// belongs to the function on the current device). Safe from several host threads: a repeated
-// set is harmless.
-template <class K>
-static void ensure_smem_attr(K kernel, size_t bytes, std::atomic<uint64_t>& mask) {
-  int dev = 0;
-  cudaGetDevice(&dev);
-  const uint64_t bit = 1ull << (dev & 63);
-  if (!(mask.load(std::memory_order_acquire) & bit)) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    mask.fetch_or(bit, std::memory_order_release);
-  }
-}
-
 // ---------------------------------------------------------------------------------------------
 // k_mask: the criterion alone, as a streaming pass; one 32-bit activity mask per row, written
 // into the row table's mask word (k_tile then starts from the masks, which stay in L2)

@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "msf.h"
+#include "msf_smem.h"
 
 namespace msf {
 
