@@ -211,8 +211,12 @@ int msf_load_timesteps_mr(msf_ctx* ctx, int nx, int ny, int nz, int T, const flo
  * this binning (every in-grid sample with its voxel, the same point's voxel at the next point
  * step and its attributes, grouped by field step and voxel range) stay until the next load or
  * binning: the trajectory joins of msf_segment and the point statistics of the features walk
- * them. Synchronises the stream. Errors: NOT_LOADED, INVALID_ARG (unknown flag), OUT_OF_MEMORY,
- * TOO_LARGE (P * Tp >= 2^32), TIMEOUT (a copy wait gave up), CUDA. */
+ * them. Device memory per point sample: 12 + 4 A bytes of the dataset, 4 of its key, a record of 16
+ * (A <= 2), 32 (A <= 6) or 48 bytes, and 8 more for a second copy of the records' voxels, which is
+ * left out where it does not fit and given back when a later call of the context finds too little
+ * memory (the joins and point statistics then read the records themselves, more slowly; not while a
+ * query server is attached). Synchronises the stream. Errors: NOT_LOADED, INVALID_ARG (unknown
+ * flag), OUT_OF_MEMORY, TOO_LARGE (P * Tp >= 2^32), TIMEOUT (a copy wait gave up), CUDA. */
 int msf_bin_particles(msf_ctx* ctx, unsigned flags, msf_bin_stats* stats);
 
 /* Copy the binning results out (each pointer may be NULL): key [T][P] int32 ([Tp][P] for a

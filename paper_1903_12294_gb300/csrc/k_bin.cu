@@ -63,7 +63,7 @@ struct BinArgs {
                                 // ends the step's records
   uint32_t* cursor;             // [T][nb] next free slot, from offs, one per kCurStride words
   uint2* rec_vn;                // [P*Tp] the sample's voxel, and the same point's voxel at the
-                                // next point step (-1 at the last or outside the grid)
+                                // next point step (-1 at the last or outside the grid); or null
   uint32_t* rec;                // [P*Tp][rec_words(A)] attribute values and the same voxel pair
   unsigned* err;                // bounded waits that gave up
   uint32_t* ovf;                // items (t * nb + bucket) left to the wide reduce
@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(kBinNT, A <= 4 ? 3 : 2) k_bin_reduce(const __g
       place[i] = 0;
       if (q < n) {
         const uint2 vn = staged_record<A>(s_area, q, x[i]);
-        __stcs(b.rec_vn + r0 + q, vn);
+        if (b.rec_vn) __stcs(b.rec_vn + r0 + q, vn);
         v[i] = (int)(vn.x & (uint32_t)(R - 1));
         const int sh = (v[i] & 1) << 4;
         place[i] = (int)((atomicAdd(s_cnt + (v[i] >> 1), 1u << sh) >> sh) & 0xFFFFu);
@@ -648,7 +648,7 @@ __global__ void __launch_bounds__(kBinNT, 1) k_bin_reduce_wide(const __grid_cons
     for (int q = threadIdx.x; q < m; q += kBinNT) {
       float vv[A > 0 ? A : 1];
       const uint2 vn = staged_record<A>(s_st, q, vv);
-      __stcs(b.rec_vn + a0 + q, vn);
+      if (b.rec_vn) __stcs(b.rec_vn + a0 + q, vn);
       const uint32_t v = vn.x & (uint32_t)(R - 1);  // voxel within the bucket
       atomicAdd(s_cnt + v, 1u);
 #pragma unroll
@@ -870,13 +870,14 @@ int bin_run(msf_ctx* ctx, unsigned flags) {
   MSF_TRY(ctx_result(ctx, word_bytes));
   MSF_TRY(S.offs.ensure(sizeof(uint32_t) * (TB + d.T)));
   MSF_TRY(S.cursor.ensure(sizeof(uint32_t) * kCurStride * TB));
-  MSF_TRY(S.rec_vn.ensure(sizeof(uint2) * std::max<int64_t>(NR, 1)));
   MSF_TRY(S.rec.ensure(sizeof(uint32_t) * RW * std::max<int64_t>(NR, 1)));
   MSF_TRY(S.ovf.ensure(sizeof(uint32_t) * (size_t)d.T * (size_t)b.nb));
   MSF_TRY(d.key.ensure(sizeof(int32_t) * ((int64_t)d.Tp * d.P + 4)));  // slack: bulk copies
   MSF_TRY(d.count.ensure(sizeof(int32_t) * d.T * d.V));
   MSF_TRY(d.mean.ensure(sizeof(float) * d.T * d.V * Af));
   if (keep) MSF_TRY(d.sumq.ensure(sizeof(int64_t) * d.T * d.V * Af));
+  // the pairs a second time, where memory allows (after everything that a binning needs)
+  if (S.rec_vn.ensure(sizeof(uint2) * std::max<int64_t>(NR, 1)) != MSF_OK) S.rec_vn.release();
   b.pos = d.pos.as<float>();
   b.attr = d.attr.as<float>();
   b.key = d.key.as<int32_t>();
@@ -952,6 +953,7 @@ int bin_run(msf_ctx* ctx, unsigned flags) {
   S.rec_logR = b.logR;
   S.rec_nb = b.nb;
   S.rec_words = RW;
+  S.rec_pair = rec_pair(d.A);
   for (int a = 0; a < d.A; ++a) {
     float m;
     memcpy(&m, &hmax[a], sizeof(float));

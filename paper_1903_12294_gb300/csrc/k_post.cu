@@ -740,6 +740,7 @@ int msf_merge_clusters(msf_ctx* c, const float* centers, int centers_kind, int32
   if (terms == 0 || (terms & ~(MSF_MERGE_POINT | MSF_MERGE_FIELD))) return MSF_ERR_INVALID_ARG;
   if (K > (1 << 18)) return MSF_ERR_TOO_LARGE;
   MSF_CUDA_TRY(cudaSetDevice(c->device));
+  SpareScope spare(c);
   PostScratch& S = c->post;
   const float* dc;
   MSF_TRY(stage_in(c, centers, centers_kind, 6 * (size_t)K, S.in, &dc));
@@ -791,6 +792,7 @@ int msf_relabel(msf_ctx* c, int32_t* labels, int labels_kind, int64_t n, const i
   // them, so msf_extract_features must read the buffer from now on
   c->last.valid = false;
   MSF_CUDA_TRY(cudaSetDevice(c->device));
+  SpareScope spare(c);
   PostScratch& S = c->post;
   const int32_t* dm;
   MSF_TRY(stage_in(c, map, map_kind, (size_t)K, S.in2, &dm));
@@ -845,6 +847,7 @@ int msf_select_clusters(msf_ctx* c, const float* centers, int centers_kind, int3
   }
   if (K > (1 << 20)) return MSF_ERR_TOO_LARGE;
   MSF_CUDA_TRY(cudaSetDevice(c->device));
+  SpareScope spare(c);
   PostScratch& S = c->post;
   const float* dc;
   MSF_TRY(stage_in(c, centers, centers_kind, 6 * (size_t)K, S.in, &dc));
@@ -914,6 +917,7 @@ int msf_cluster_stats(msf_ctx* c, int32_t t0, int32_t t1, int32_t attr,
   const int64_t tw = t1 - t0, nf = tw * d.V, np = use_p ? tw * d.P : 0;
   if (nf >= ((int64_t)1 << 31) || np >= ((int64_t)1 << 31)) return MSF_ERR_TOO_LARGE;
   MSF_CUDA_TRY(cudaSetDevice(c->device));
+  SpareScope spare(c);
   MSF_TRY(ctx_field_ready(c));
   PostScratch& S = c->post;
   StatArgs a{};
@@ -1020,6 +1024,7 @@ int msf_split_trajectories(msf_ctx* c, int32_t t0, int32_t t1, const int32_t* la
   *n_pieces = 0;
   if (d.P == 0) return MSF_OK;
   MSF_CUDA_TRY(cudaSetDevice(c->device));
+  SpareScope spare(c);
   PostScratch& S = c->post;
   PieceArgs a{};
   MSF_TRY(stage_in(c, labels, labels_kind, (size_t)(tw * (vox ? d.V : d.P)), S.in, &a.lab));

@@ -766,18 +766,26 @@ __global__ void __launch_bounds__(256, 4) k_links(const __grid_constant__ SegArg
 constexpr uint32_t kRecChunkMax = 32768, kRecChunkMin = 1024;
 
 struct RecView {
-  const uint2* rec_vn;    // [records] voxel, the point's voxel at the next point step (or -1)
+  const char* pairs;      // a uint2 every pair_bytes: voxel, the point's voxel at the next point
+                          // step (or -1); side by side, or where they stand in the records
   const float* rec;       // [records][rw] attributes first
   const uint32_t* offs;   // [T][nb + 1] first record of each (field step, bucket); [t][nb]
                           // ends field step t's records
   int nb, rw;
   uint32_t chunk;         // records per block
+  uint32_t pair_bytes;
+  __device__ __forceinline__ const uint2* pair(uint32_t r) const {
+    return reinterpret_cast<const uint2*>(pairs + (size_t)r * pair_bytes);
+  }
 };
 
 static RecView rec_view(const msf_ctx* ctx) {
   const BinScratch& B = ctx->bin;
-  return RecView{B.rec_vn.as<uint2>(), B.rec.as<float>(), B.offs.as<uint32_t>(), B.rec_nb,
-                 B.rec_words, kRecChunkMax};
+  const bool apart = B.rec_vn.p != nullptr;
+  const char* in_records = B.rec.as<char>() + sizeof(uint32_t) * B.rec_pair;
+  return RecView{apart ? B.rec_vn.as<char>() : in_records, B.rec.as<float>(),
+                 B.offs.as<uint32_t>(), B.rec_nb, B.rec_words, kRecChunkMax,
+                 (uint32_t)(apart ? sizeof(uint2) : sizeof(uint32_t) * B.rec_words)};
 }
 
 // Records per block for a pass of `steps` block rows (field steps, or batch items) over at most
@@ -872,7 +880,7 @@ __device__ __forceinline__ void links_rec_range(const SegArgs& a, const RecView&
 #pragma unroll
     for (int u = 0; u < kRecPer; ++u) {
       const uint32_t r = base + 32u * u + lane;
-      e[u] = r < b1 ? __ldcs(rv.rec_vn + r) : make_uint2(0u, 0xFFFFFFFFu);
+      e[u] = r < b1 ? __ldcs(rv.pair(r)) : make_uint2(0u, 0xFFFFFFFFu);
     }
 #pragma unroll
     for (int u = 0; u < kRecPer; ++u)
@@ -1956,7 +1964,7 @@ __device__ __forceinline__ void feat_points_block(const SegArgs& a, const FeatAc
 #pragma unroll
       for (int u = 0; u < kPackPer; ++u) {
         const uint32_t r = base + 32u * u + lane;
-        v[u] = r < b1 ? __ldcs(&rv.rec_vn[r].x) : 0xFFFFFFFFu;
+        v[u] = r < b1 ? __ldcs(&rv.pair(r)->x) : 0xFFFFFFFFu;
       }
 #pragma unroll
       for (int u = 0; u < kPackPer; ++u)

@@ -19,11 +19,30 @@ void set_last_cuda_error(cudaError_t e, const char* what, const char* file, int 
            file, line);
 }
 
+static thread_local msf_ctx* t_spare = nullptr;
+
+SpareScope::SpareScope(msf_ctx* c) : prev(t_spare) { t_spare = c; }
+SpareScope::~SpareScope() { t_spare = prev; }
+
+// Frees the second copy of the voxel pairs; false when there is none or a server reads it.
+static bool give_spare(msf_ctx* c) {
+  if (!c || !c->bin.rec_vn.p || c->servers.load() > 0) return false;
+  cudaStreamSynchronize(c->stream);
+  if (c->aux) cudaStreamSynchronize(c->aux);
+  c->batch.drop_graph();  // its launches hold the address
+  c->bin.rec_vn.release();
+  return true;
+}
+
 int DevBuf::ensure(size_t n) {
   if (n <= bytes && p) return MSF_OK;
   release();
   if (n == 0) n = 16;
   cudaError_t e = cudaMalloc(&p, n);
+  if (e != cudaSuccess && give_spare(t_spare)) {
+    cudaGetLastError();
+    e = cudaMalloc(&p, n);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     p = nullptr;
@@ -357,7 +376,7 @@ void msf_destroy(msf_ctx* c) {
                     &c->feat.out})
     b->release();
   for (DevBuf* b : {&c->bin.hist, &c->bin.offs, &c->bin.cursor, &c->bin.rec_vn, &c->bin.rec,
-                    &c->bin.scan_tmp, &c->bin.ovf})
+                    &c->bin.ovf})
     b->release();
   c->bin.rec_valid = false;
   c->last.cfid.release();
@@ -418,6 +437,7 @@ int msf_load_timesteps_mr(msf_ctx* c, int nx, int ny, int nz, int T, const float
   const int64_t V = (int64_t)nx * ny * nz;
   if (V >= ((int64_t)1 << 31) || P >= ((int64_t)1 << 31)) return MSF_ERR_TOO_LARGE;
   MSF_CUDA_TRY(cudaSetDevice(c->device));
+  SpareScope spare(c);
   Dataset& d = c->ds;
   d.loaded = false;
   d.binned = false;
@@ -525,6 +545,7 @@ int msf_bin_particles(msf_ctx* c, unsigned flags, msf_bin_stats* stats) {
   if (flags & ~(unsigned)MSF_BIN_KEEP_SUMQ) return MSF_ERR_INVALID_ARG;
   if (!c->ds.loaded) return MSF_ERR_NOT_LOADED;
   MSF_CUDA_TRY(cudaSetDevice(c->device));
+  SpareScope spare(c);
   c->epoch++;
   c->last.valid = false;
   MSF_TRY(bin_run(c, flags));
@@ -548,6 +569,7 @@ int msf_get_bins(msf_ctx* c, int32_t* key, int32_t* count, float* mean, int64_t*
   if (!d.binned) return MSF_ERR_NOT_BINNED;
   if (sumq && !d.has_sumq) return MSF_ERR_INVALID_ARG;
   MSF_CUDA_TRY(cudaSetDevice(c->device));
+  SpareScope spare(c);
   const cudaMemcpyKind k = ptr_kind == MSF_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
   cudaStream_t s = c->stream;
   if (key && d.P > 0) MSF_CUDA_TRY(cudaMemcpyAsync(key, d.key.p, sizeof(int32_t) * d.Tp * d.P, k, s));
@@ -568,6 +590,7 @@ int msf_segment(msf_ctx* c, const msf_criteria* crit, int32_t* labels, int label
   const int64_t N = (int64_t)(crit->t1 - crit->t0) * c->ds.V;
   if (N > 0 && !labels) return MSF_ERR_INVALID_ARG;
   MSF_CUDA_TRY(cudaSetDevice(c->device));
+  SpareScope spare(c);
   MSF_TRY(ctx_field_ready(c));
   int32_t* dst = labels;
   if (labels_kind == MSF_HOST && N > 0) {
@@ -595,6 +618,7 @@ int msf_extract_features(msf_ctx* c, const msf_criteria* crit, const int32_t* la
   const int64_t N = (int64_t)(crit->t1 - crit->t0) * c->ds.V;
   if (N > 0 && !labels) return MSF_ERR_INVALID_ARG;
   MSF_CUDA_TRY(cudaSetDevice(c->device));
+  SpareScope spare(c);
   MSF_TRY(ctx_field_ready(c));
   const int32_t* src = labels;
   // Labels this context's last msf_segment wrote for the same query are not read back: the
@@ -620,6 +644,7 @@ int msf_segment_features(msf_ctx* c, const msf_criteria* crit, int32_t* labels, 
   const int64_t N = (int64_t)(crit->t1 - crit->t0) * c->ds.V;
   if (N > 0 && !labels) return MSF_ERR_INVALID_ARG;
   MSF_CUDA_TRY(cudaSetDevice(c->device));
+  SpareScope spare(c);
   MSF_TRY(ctx_field_ready(c));
   int32_t* dst = labels;
   if (labels_kind == MSF_HOST && N > 0) {
@@ -654,6 +679,7 @@ int msf_segment_batch(msf_ctx* c, int nq, const msf_criteria* crits, int32_t* co
   }
   if (nq == 0) return MSF_OK;
   MSF_CUDA_TRY(cudaSetDevice(c->device));
+  SpareScope spare(c);
   MSF_TRY(ctx_field_ready(c));
   return segment_batch_run(c, nq, crits, labels, n_features);
 }
@@ -684,6 +710,7 @@ int msf_cluster(msf_ctx* c, const msf_cluster_params* prm, int32_t* field_labels
   const int64_t nf = tw * d.V, np = nj * d.P;
   if (nf >= ((int64_t)1 << 31) || np >= ((int64_t)1 << 31)) return MSF_ERR_TOO_LARGE;
   MSF_CUDA_TRY(cudaSetDevice(c->device));
+  SpareScope spare(c);
   MSF_TRY(ctx_field_ready(c));
   c->last.valid = false;  // the label buffers may be the retained segmentation's
   int32_t* fl = field_labels;

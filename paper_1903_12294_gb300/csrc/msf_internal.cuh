@@ -39,7 +39,7 @@ void set_last_cuda_error(cudaError_t e, const char* what, const char* file, int 
 struct DevBuf {
   void* p = nullptr;
   size_t bytes = 0;
-  int ensure(size_t n);  // grow to at least n bytes (contents discarded on growth)
+  int ensure(size_t n);  // grow to at least n bytes (contents discarded on growth); see SpareScope
   void release();
   template <class T>
   T* as() const { return static_cast<T*>(p); }
@@ -164,14 +164,15 @@ struct BatchScratch {
 
 struct BinScratch {
   // hist ends in the binning's result words (one clear, one copy back): see BinWords
-  DevBuf hist, offs, cursor, rec_vn, rec, scan_tmp, ovf;
+  DevBuf hist, offs, cursor, rec_vn, rec, ovf;
   // The records of the last binning stay for the trajectory joins and the feature statistics:
   // the samples grouped by (field step, bucket of 2^rec_logR voxels) in the slot ranges
-  // offs[t][bucket] (offs [T][nb + 1]; offs[t][nb] ends field step t's records), each its voxel
-  // and its point's voxel at the next point step (rec_vn), and rec_words words that start with
-  // its attributes (rec).
+  // offs[t][bucket] (offs [T][nb + 1]; offs[t][nb] ends field step t's records), each rec_words
+  // words (rec): its attributes, and from word rec_pair its voxel and its point's voxel at the next
+  // point step. rec_vn holds those pairs a second time, side by side, which the passes that read
+  // nothing else read faster; it is the first memory to go when a call finds too little.
   bool rec_valid = false;
-  int rec_logR = 0, rec_nb = 0, rec_words = 0;
+  int rec_logR = 0, rec_nb = 0, rec_words = 0, rec_pair = 0;
 };
 
 // Scratch of the clustering (k_cluster.cu): centres, their sums and cells, label buffers for
@@ -298,6 +299,17 @@ int ctx_fork(msf_ctx* ctx);
 int ctx_join(msf_ctx* ctx);
 int ctx_field_ready(msf_ctx* ctx);  // the context stream waits for a field copy in flight
 int ctx_result(msf_ctx* ctx, size_t bytes);  // ctx->res holds at least `bytes`
+
+// While one lives, a DevBuf of this thread that finds too little device memory takes what the
+// context can do without (the records' second copy of the voxel pairs, unless a query server reads
+// it) and tries once more. One per entry point that allocates.
+struct SpareScope {
+  explicit SpareScope(msf_ctx* c);
+  ~SpareScope();
+  SpareScope(const SpareScope&) = delete;
+  SpareScope& operator=(const SpareScope&) = delete;
+  msf_ctx* prev;
+};
 
 // An auxiliary stream with its fork and join events, for a main stream given at each use.
 struct StreamPair {

@@ -348,6 +348,7 @@ extern "C" int msf_server_create(msf_ctx* ctx, const msf_server_config* cfg, msf
       c.pool_bytes < 4096)
     return MSF_ERR_INVALID_ARG;
   MSF_CUDA_TRY(cudaSetDevice(ctx->device));
+  SpareScope spare(ctx);
   // the slots' streams read the dataset: everything queued on the context (the field's copy
   // in, binning) completes first
   MSF_TRY(ctx_field_ready(ctx));

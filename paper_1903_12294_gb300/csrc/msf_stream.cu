@@ -203,6 +203,7 @@ extern "C" int msf_segment_streamed(msf_ctx* c, int nx, int ny, int nz, int T, c
     pj0[t] = j;
   }
   MSF_CUDA_TRY(cudaSetDevice(c->device));
+  SpareScope spare(c);
   cudaStream_t s = c->stream;
   StreamBufs B;
   bool uses_points = (crit->edges & MSF_EDGE_TRAJ) != 0;

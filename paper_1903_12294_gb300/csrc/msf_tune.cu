@@ -104,6 +104,7 @@ int msf_autotune(msf_ctx* c, const msf_criteria* crit, int reps, msf_tune_result
   if (g0.tw == 0) return MSF_ERR_INVALID_ARG;
   if (reps < 1) reps = 3;
   MSF_CUDA_TRY(cudaSetDevice(c->device));
+  SpareScope spare(c);
   MSF_TRY(ctx_field_ready(c));
   const Dataset& d = c->ds;
   const int64_t N = (int64_t)g0.tw * d.V;
@@ -254,6 +255,7 @@ int msf_autotune_batch(msf_ctx* c, int nq, const msf_criteria* crits, int32_t* c
   if (twmax == 0) return MSF_ERR_INVALID_ARG;
   if (reps < 1) reps = 3;
   MSF_CUDA_TRY(cudaSetDevice(c->device));
+  SpareScope spare(c);
   MSF_TRY(ctx_field_ready(c));
   const int keep_by = c->batch_by, keep_bz = c->batch_bz, keep_bt = c->batch_bt;
   const int keep_sched = c->batch_sched;
