@@ -1830,8 +1830,9 @@ constexpr size_t feat_vox_smem() {
 //   - The other members wait in a list until there are 32 of them for reduce_samples, whose
 //     instructions a few of them cost as many as 32 do.
 // 8M particles x 24 steps, one feature with nine tenths of the members: a pack at a time, all through
-// reduce_samples, 5.5 ms, so 2.45 ms. (2.18 ms with the members of several packs summed together, but
-// then nearly equal samples of small features that had been summed apart were rounded together.)
+// reduce_samples, 5.5 ms, so 2.69 ms beside the voxel statistics. (2.18 ms with the members of several
+// packs summed together, but then nearly equal samples of small features that had been summed apart
+// were rounded together.)
 // The samples are those of every point step falling in the window's field steps that binning
 // placed inside the grid: the same as the per-point pass takes. Block (x, y) takes records
 // [x * chunk, (x + 1) * chunk) of window field step y.

@@ -994,6 +994,25 @@ __device__ __forceinline__ void reduce_samples(const FeatAcc& acc, bool ok, int6
       l = __fmul_rn(__fmul_rn(__uint2float_rn((uint32_t)(r >> sr)), pow2f((sr - k2) / 2)),
                     pow2f((sr - k2) - (sr - k2) / 2));
     }
+    if (some_pairs) {  // the butterfly's tree, over the places in the chain instead of the lanes
+      float ph = p, pl = pe;
+#pragma unroll 1
+      for (int i = 4; i >= 0; --i) {
+        if (1 << i >= most) continue;
+        const int o = i == 0 ? next[0] : i == 1 ? next[1] : i == 2 ? next[2] : i == 3 ? next[3] : next[4];
+        const float h2 = __shfl_sync(F, ph, o & 31), l2 = __shfl_sync(F, pl, o & 31);
+        if (o >= 0) {
+          float sh, se;
+          two_sum(ph, h2, sh, se);
+          ph = sh;
+          pl = __fadd_rn(__fadd_rn(pl, l2), se);
+        }
+      }
+      if (pairs) {
+        h = ph;
+        l = pl;
+      }
+    }
     if (ok && lane == leader) sink(key, j, qs, h, l, w, dbl, false);
   }
 }
