@@ -13,9 +13,10 @@
 //              a union-find in shared memory over the tile's in-tile neighbour rows. Writes the
 //              compact result: per segment its mask and first run slot, per run its component,
 //              per component its smallest index. Nothing per voxel is written.
-//   k_hook     one CTA per tile, one thread per segment: joins components across the tile's
-//              lower faces (x, y, z and the t-chunk boundary) with a global union-find on the
-//              component table, each distinct component pair once per tile.
+//   k_hook     one CTA per tile: joins components across the tile's lower faces (x, y, z and the
+//              t-chunk boundary) with a global union-find on the component table, each distinct
+//              component pair once per tile. Its threads take a (segment, direction) each, in dense
+//              tiles a segment each.
 //   k_links    trajectory joins: on a binned dataset with one point step per field step, from
 //              the binning's records in bucket order (each record holds its voxel at t and its
 //              point's voxel at t+1); otherwise one thread per (point, chunk of 8 point steps)
@@ -1128,8 +1129,8 @@ __global__ void __launch_bounds__(256) k_mask(const __grid_constant__ SegArgs a)
 
 // Rows of 32 voxels are contiguous when nx is a multiple of 32: the window is one linear run
 // of the predicate arrays, row gs starting at voxel 32 * gs. Each thread takes U 16-byte units
-// 256 apart; eight lanes cover one row. The row mask is put together from four warp ballots
-// (bit k of every lane's four voxels) rather than a lane reduction. FLOAT: no COUNT predicate.
+// 256 apart; eight lanes cover one row, and three exchanges among them put its mask together.
+// FLOAT: no COUNT predicate.
 template <int NP, bool FLOAT>
 __device__ __forceinline__ void mask_lin_block(const SegArgs& a, uint32_t blk) {
   constexpr int U = NP <= 2 ? 4 : 2;
@@ -1290,8 +1291,9 @@ int segment_run(msf_ctx* ctx, const msf_criteria* crit, int32_t* labels, int64_t
   // overlap the labelling, which is bound by instruction issue, and the masks' round trip through
   // L2 goes. The streaming pass was the faster one on no size measured (one query, streamed
   // against inside: 128^3 x 32 373 -> 336 us, 256^3 x 24 3.21 -> 2.82 ms, 1024^2 x 64 364 -> 331
-  // us, 32^3 x 8 with the rest of a step 303 -> 295 us); it stays for callers that set it and for
-  // the tuner.
+  // us, 32^3 x 8 with the rest of a step 303 -> 295 us; and none of 104 queries on rows of 128, 100,
+  // 101 and 33 voxels with no to four predicates and 2 to 100 % members was slower than when the
+  // mask was streamed by default); it stays for callers that set it and for the tuner.
   const bool fused = (sched & MSF_SCHED_FUSED_CRITERION) || segment_automatic(ctx, crit);
   if (!fused) {  // the criterion as a streaming pass, the tile pass then starting from its masks
     ScopedKernel k(ctx, "k_mask");

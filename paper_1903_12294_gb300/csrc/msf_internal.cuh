@@ -823,9 +823,6 @@ struct VoxTable {
   }
 };
 
-// Point samples (one per lane in `ok`): lanes of the same feature reduce their exact
-// fixed-point attribute values and double-float squares; the group's first lane commits.
-// Every lane of the warp must call this.
 // empty accumulators i, i + stride, ..
 __device__ __forceinline__ void acc_init(const FeatAcc& c, int64_t i0, int64_t stride) {
   const int64_t n = c.F * c.K;
