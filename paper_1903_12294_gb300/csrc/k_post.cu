@@ -466,6 +466,17 @@ __device__ __forceinline__ int ctab_slot(int* key, int l) {
   return -1;
 }
 
+// Do all lanes of the warp end a run of the same label here (all of them converged)? Labels that lie
+// along the rows make every sample a run of its own, and neighbouring lanes' the same: they add up in
+// the warp, since 32 of them would queue at the label's place (5000 x 40 x 16, 1000 labels along the
+// rows, the whole call 0.27 ms, so 0.19).
+__device__ __forceinline__ bool warp_of_one(int label) {
+  if (__activemask() != kFull) return false;
+  int same;
+  __match_all_sync(kFull, label, &same);
+  return same && label >= 0;
+}
+
 struct SumTab {
   int key[kCtab];
   unsigned n[kCtab];
@@ -513,6 +524,16 @@ __global__ void __launch_bounds__(256) k_cstat_sum(StatArgs s, StatWalk w) {
   long long rq = 0;
   bool bad = false;  // (labels were checked by pass 1)
   auto flush = [&] {
+    if (warp_of_one(rl)) {
+      rq = (long long)limb_sum(kFull, (unsigned long long)rq);
+      rn = __reduce_add_sync(kFull, rn);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        rlo[j] = __reduce_min_sync(kFull, rlo[j]);
+        rhi[j] = __reduce_max_sync(kFull, rhi[j]);
+      }
+      if (threadIdx.x & 31) rl = -1;
+    }
     if (rl < 0) return;
     const int h = ctab_slot(tab.key, rl);
     if (h < 0) {
@@ -594,6 +615,11 @@ __global__ void __launch_bounds__(256) k_cstat_dev(StatArgs s, StatWalk w) {
   double rd = 0.0, rm = 0.0;
   bool bad = false;
   auto flush = [&] {
+    if (warp_of_one(rl)) {
+#pragma unroll
+      for (int o = 16; o; o >>= 1) rd += __shfl_xor_sync(kFull, rd, o);
+      if (threadIdx.x & 31) rl = -1;
+    }
     if (rl < 0) return;
     const int h = ctab_slot(s_key, rl);
     if (h < 0) atomicAdd(q + rl, rd);
