@@ -210,8 +210,10 @@ __global__ void __launch_bounds__(256) k_vox(const __grid_constant__ FeatArgs a)
   s_tab.flush(a.acc);
 }
 
-// Generic path: every point sample of the window, one thread per (point step, point).
-__global__ void __launch_bounds__(256) k_pts(const __grid_constant__ FeatArgs a) {
+// Generic path: every point sample of the window, one thread per (point step, point). Eight blocks
+// per SM (its keys and labels are gathered; 400K points x 8 steps, 2 % members, five blocks of the 40
+// registers it would take 125 us, eight 104).
+__global__ void __launch_bounds__(256, 8) k_pts(const __grid_constant__ FeatArgs a) {
   __shared__ HotCache s_hot[8][kHotWays];
   hot_clear(s_hot[threadIdx.x >> 5]);
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -251,9 +253,10 @@ __device__ __forceinline__ double div_by(double x, double n, double r) {
 // exchanges (with few features one thread per feature walks its copies one after the other, 23 us of
 // a small step's 60 features, so 14). Otherwise, and with many features, one thread per feature: a
 // lane per copy reads one word of every sector (one attribute, 4000 features of 16 copies 30 us by
-// features and 21 by copies, 8000 31 and 37, 30,000 31 and 90). The records go through shared memory
-// so that the block stores them as one run of words (each thread storing its own 312 bytes took 0.27
-// ms for 584K features, so 0.21 ms).
+// features and 21 by copies, 8000 31 and 37, 30,000 31 and 90). The records of the former go through
+// shared memory so that the block stores them as one run of words (each thread storing its own 312
+// bytes took 0.27 ms for 584K features of one copy, so 0.21 ms); the latter's threads, which walk
+// several copies, are better off with the blocks that the memory would cost them.
 constexpr int64_t kRecSplit = 1 << 16;  // copies of all features up to which a lane takes one each
 constexpr int kRecNT = 128;
 constexpr int kRecWords = (int)(sizeof(msf_feature) / 8);
@@ -261,7 +264,7 @@ static_assert(sizeof(msf_feature) == 8 * kRecWords, "records are whole 8-byte wo
 
 template <bool SPLIT>
 __global__ void __launch_bounds__(kRecNT) k_records(const __grid_constant__ FeatArgs a) {
-  __shared__ __align__(16) unsigned long long s_rec[kRecNT * kRecWords];
+  __shared__ __align__(16) unsigned long long s_rec[SPLIT ? kRecNT * kRecWords : 1];
   constexpr unsigned W = 0xFFFFFFFFu;
   const FeatAcc& c = a.acc;
   const int L = SPLIT ? c.K : 1;  // lanes per feature (K: a power of two, at most 16)
@@ -321,9 +324,9 @@ __global__ void __launch_bounds__(kRecNT) k_records(const __grid_constant__ Feat
     bmax[j] = most(bmax[j]);
     sc[j] = sum(sc[j]);
   }
-  msf_feature& o = *reinterpret_cast<msf_feature*>(s_rec + fl * kRecWords);
-  if (k == 0)
-    for (int j = 0; j < kRecWords; ++j) s_rec[fl * kRecWords + j] = 0ull;
+  msf_feature own;
+  msf_feature& o = SPLIT ? *reinterpret_cast<msf_feature*>(s_rec + fl * kRecWords) : own;
+  if (k == 0) memset(&o, 0, sizeof(o));
   const double n = (double)nv, rn = __drcp_rn(n), npd = (double)np;
   if (k == 0) {
 #pragma unroll
@@ -360,6 +363,10 @@ __global__ void __launch_bounds__(kRecNT) k_records(const __grid_constant__ Feat
       const double v = s2 / npd - m * m;
       o.std_attr[j] = sqrt(v > 0.0 ? v : 0.0);
     }
+  }
+  if (!SPLIT) {
+    if (in) a.out[f] = own;
+    return;
   }
   __syncthreads();
   const int64_t w0 = (int64_t)blockIdx.x * per * kRecWords;
