@@ -62,8 +62,10 @@ struct BinArgs {
                                 // pj0[t] * P) split by the exclusive prefix of hist; [t][nb]
                                 // ends the step's records
   uint32_t* cursor;             // [T][nb] next free slot, from offs, one per kCurStride words
-  uint2* rec_vn;                // [P*Tp] the sample's voxel, and the same point's voxel at the
-                                // next point step (-1 at the last or outside the grid); or null
+  char* pairs;                  // a uint2 per sample, every pair_bytes: its voxel, and the same
+  uint32_t pair_bytes;          // point's voxel at the next point step (-1 at the last or outside
+                                // the grid), side by side; or, where memory is short, the records'
+                                // own pairs, which the reduce then writes once more as they are
   uint32_t* rec;                // [P*Tp][rec_words(A)] attribute values and the same voxel pair
   unsigned* err;                // bounded waits that gave up
   uint32_t* ovf;                // items (t * nb + bucket) left to the wide reduce
@@ -348,6 +350,10 @@ __device__ __forceinline__ void reduce_issue(const BinArgs& b, uint32_t a0, uint
   bulk_g2s(s_st, b.rec + (size_t)a0 * RW, 4u * n * RW, bar);
 }
 
+__device__ __forceinline__ uint2* pair_at(const BinArgs& b, uint32_t r) {
+  return reinterpret_cast<uint2*>(b.pairs + (size_t)r * b.pair_bytes);
+}
+
 // record range [r0, r1) of the item (field step t, bucket): the slots of its point steps
 __device__ __forceinline__ void item_range(const BinArgs& b, int t, int bucket, uint32_t& r0,
                                            uint32_t& r1) {
@@ -485,14 +491,16 @@ __global__ void __launch_bounds__(kBinNT, A <= 4 ? 3 : 2) k_bin_reduce(const __g
     }
     int v[PER], place[PER];
     float x[PER][A1];  // quantised attributes
+    char* pair = reinterpret_cast<char*>(pair_at(b, r0 + threadIdx.x));
+    const uint32_t pair_step = kBinNT * b.pair_bytes;
 #pragma unroll
-    for (int i = 0; i < PER; ++i) {
+    for (int i = 0; i < PER; ++i, pair += pair_step) {
       const int q = (int)threadIdx.x + kBinNT * i;
       v[i] = -1;
       place[i] = 0;
       if (q < n) {
         const uint2 vn = staged_record<A>(s_area, q, x[i]);
-        if (b.rec_vn) __stcs(b.rec_vn + r0 + q, vn);
+        __stcs(reinterpret_cast<uint2*>(pair), vn);
         v[i] = (int)(vn.x & (uint32_t)(R - 1));
         const int sh = (v[i] & 1) << 4;
         place[i] = (int)((atomicAdd(s_cnt + (v[i] >> 1), 1u << sh) >> sh) & 0xFFFFu);
@@ -648,7 +656,7 @@ __global__ void __launch_bounds__(kBinNT, 1) k_bin_reduce_wide(const __grid_cons
     for (int q = threadIdx.x; q < m; q += kBinNT) {
       float vv[A > 0 ? A : 1];
       const uint2 vn = staged_record<A>(s_st, q, vv);
-      if (b.rec_vn) __stcs(b.rec_vn + a0 + q, vn);
+      __stcs(pair_at(b, a0 + q), vn);
       const uint32_t v = vn.x & (uint32_t)(R - 1);  // voxel within the bucket
       atomicAdd(s_cnt + v, 1u);
 #pragma unroll
@@ -884,8 +892,9 @@ int bin_run(msf_ctx* ctx, unsigned flags) {
   b.hist = S.hist.as<uint32_t>();
   b.offs = S.offs.as<uint32_t>();
   b.cursor = S.cursor.as<uint32_t>();
-  b.rec_vn = S.rec_vn.as<uint2>();
   b.rec = S.rec.as<uint32_t>();
+  b.pairs = S.rec_vn.p ? S.rec_vn.as<char>() : S.rec.as<char>() + sizeof(uint32_t) * rec_pair(d.A);
+  b.pair_bytes = (uint32_t)(S.rec_vn.p ? sizeof(uint2) : sizeof(uint32_t) * RW);
   b.wait_cycles = ctx->wait_cycles;
   b.pf_ahead = ctx->sm_count * (d.A <= 4 ? 3 : 2);  // resident reduce blocks
   BinWords* dw = reinterpret_cast<BinWords*>(S.hist.as<char>() + hist_bytes);
