@@ -50,8 +50,8 @@ TRAFFIC = {
     # ncu DRAM bytes (read + write) of one launch, from a single-kernel capture of the unchanged
     # kernel (profiles/); combustion: the 4-timestep capture (--timesteps 4) scaled by 6 to the
     # 24-step launch (a launch's records and voxels grow in proportion to its field steps)
-    (3, "k_bin_reduce"): (1_074_027_000 + 1_551_283_000) * 6,
-    (3, "k_feat_points"): (679_826_000 + 8_584_000) * 6,
+    (3, "k_bin_reduce"): (1_074_023_000 + 1_551_635_000) * 6,
+    (3, "k_feat_points"): (683_966_000 + 11_454_000) * 6,
 }
 
 
