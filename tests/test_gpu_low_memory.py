@@ -10,14 +10,21 @@ pytestmark = pytest.mark.gpu
 MB = 1 << 20
 
 
-def _fill(leave):
-    """Allocations that leave about `leave` bytes of the device free (20 MB is the allocator's step)."""
-    torch.cuda.empty_cache()
+@pytest.fixture
+def fill():
+    """fill(leave): allocations that leave about `leave` bytes of the device free (20 MB is the
+    allocator's step); fill(None) frees them, as the end of the test does."""
     held = []
-    for size in (16 << 30, 1 << 30, 100 * MB, 20 * MB):
-        while torch.cuda.mem_get_info()[0] > leave + size + 8 * MB:
-            held.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
-    return held
+
+    def f(leave):
+        held.clear()
+        torch.cuda.empty_cache()
+        for size in (16 << 30, 1 << 30, 100 * MB, 20 * MB) if leave is not None else ():
+            while torch.cuda.mem_get_info()[0] > leave + size + 8 * MB:
+                held.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+
+    yield f
+    f(None)
 
 
 def _data(A, P=2 << 20, T=8, n=64):
@@ -43,7 +50,7 @@ def _same(a, b, A):
 
 
 @pytest.mark.parametrize("A", [1, 4, 8])
-def test_pairs_left_out_or_given_back(gpu, A):
+def test_pairs_left_out_or_given_back(gpu, fill, A):
     field, pos, attr = _data(A)
     T, n = field.shape[0], field.shape[1]
     args = (0, T, [(0, 0, 0, 1.2, 0.0)], 7)
@@ -65,10 +72,10 @@ def test_pairs_left_out_or_given_back(gpu, A):
         want = _answers(first, args, labels, gpu)
         # given back: a batch's scratch (about 110 MB) takes the pairs' place (134 MB)
         torch.cuda.synchronize()
-        held = _fill(32 * MB)
+        fill(32 * MB)
         assert torch.cuda.mem_get_info()[0] < 64 * MB
         first.segment_batch(queries, out)
-        del held
+        fill(None)
         for x, y in zip(out, want_batch):
             assert torch.equal(x.cpu(), y)
         _same(_answers(first, args, labels, gpu), want, A)
@@ -78,14 +85,13 @@ def test_pairs_left_out_or_given_back(gpu, A):
     NR = pos.shape[0] * pos.shape[2]
     rec = 16 if A <= 2 else 32 if A <= 6 else 48
     need = NR * (12 + 4 * A + 4 + rec) + field.numel() * (8 + 4 * A) + 64 * MB
-    held = _fill(need + NR * 8 // 2)
+    fill(need + NR * 8 // 2)
     ctx = gpu.Context(0)
     try:
         ctx.load(field, pos, attr)
         ctx.bin()
         _same(_answers(ctx, args, labels, gpu), want, A)
-        del held
-        torch.cuda.empty_cache()
+        fill(None)
         ctx.bin()                         # with room again
         _same(_answers(ctx, args, labels, gpu), want, A)
     finally:
