@@ -404,7 +404,7 @@ __device__ __forceinline__ uint2 staged_record(const uint32_t* s_st, int q,
 // where there are no records (storing NaN everywhere and the means over it, one 4-byte store per
 // non-empty voxel and attribute, issued twice the stores; sorting the records by voxel first and
 // quantising in the divergent parts made it 16,000 instructions a bucket). 8M records x 24 steps,
-// 256^3 voxels, A = 4: 4.17 ms before, 3.47 ms now. A bucket with more records than the staging
+// 256^3 voxels, A = 4: 4.17 ms before, 3.50 ms now. A bucket with more records than the staging
 // area holds is listed for k_bin_reduce_wide and left to it.
 __host__ __device__ constexpr int red_stage(int A) { return A <= 6 ? 2048 : 1536; }
 

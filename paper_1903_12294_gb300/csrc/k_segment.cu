@@ -1550,7 +1550,7 @@ __global__ void __launch_bounds__(1024) k_feat_ranks(const __grid_constant__ Seg
 // with more than kVoxHash / 2 of them groups by component instead (its features are small).
 // Members are a few per cent of a selective query's voxels and lie in rows of one or two, so
 // walking rows with a lane per voxel left most lanes idle and reduced every row's groups apart
-// (256^3 x 24, three predicates, 584K features: 3.52 ms before, 1.21 ms now; small calls, where
+// (256^3 x 24, three predicates, 584K features: 3.52 ms before, 1.15 ms now; small calls, where
 // a block's 32 rows per warp were one long chain, 45 us before, 16 us now).
 constexpr int kCompThread = 8, kCompWarp = 512, kVoxHash = 2048;
 

@@ -460,10 +460,10 @@ __device__ __forceinline__ long long quantise(float v, int k) {
 //
 // Accumulators are SoA arrays of K copies x F features (index copy * F + feature); a block adds
 // into copy blockIdx.x % K, so that the atomics of a large feature spread over K addresses;
-// k_records sums the copies. Sums of field values and squares are formed per warp group in
-// double-float (fp32 pairs with exact TwoSum/TwoProd steps) and committed as two fp64 atomics;
-// the part's fp64 pipe is narrow, so fp64 arithmetic on the SM is left to sums that one lane
-// keeps for many samples (the caches of the point samples' squares).
+// k_records sums the copies. Sums of a warp's groups (a row's voxels read from a label buffer, point
+// samples) are formed in double-float (fp32 pairs with exact TwoSum/TwoProd steps) and committed as
+// two fp64 atomics; the part's fp64 pipe is narrow, so fp64 arithmetic on the SM is left to sums that
+// one lane keeps (a feature's voxels in a tile, the squares of a warp's own feature).
 // ---------------------------------------------------------------------------------------------
 struct FeatAcc {
   unsigned long long* n_vox;
